@@ -246,7 +246,8 @@ namespace {
 
 struct Ws {
     double2 *V, *HV, *X, *HX, *R, *Dl, *Tmp;  // [.. rows][ld]
-    double2 *Hs, *G, *A, *Z, *Cs, *Part;      // small
+    double2 *Hs, *G, *A, *Z, *Cs;      // small
+    GemmWork part;                           // scratch of the FP64 products
     double2 *Cp, *CT, *PT, *QT;               // previous Ritz coefficients [nvecx+1][nb]; transposed blocks
     double2 *Y, *HY;                          // [nb][ld]: previous-direction rows kept at a restart
     double *eval, *eps, *rn2, *tk, *hdiag, *vpart;
@@ -302,7 +303,7 @@ struct DavidsonRun {
         return zgemm_cn_bf16x3(M, N, npw, A, ld, B, ld, C, ldc, sub, sub_bytes, tc_err, s);
     }
     qm_status cn64(int M, int N, const double2* A, const double2* B, double2* C, int ldc) {
-        return (ds ? zgemm_cn_ds : zgemm_cn)(M, N, npw, A, ld, B, ld, C, ldc, w.Part, zgemm_cn_splits(M, N, npw), s);
+        return (ds ? zgemm_cn_ds : zgemm_cn)(M, N, npw, A, ld, B, ld, C, ldc, w.part, s);
     }
     qm_status tn_tc(int M, int K, const double2* A, int lda, const double2* B, double2* C, bool acc,
                     double alpha = 1.0) {
@@ -310,7 +311,7 @@ struct DavidsonRun {
     }
     qm_status tn64(int M, int K, const double2* A, int lda, const double2* B, double2* C, bool acc,
                    double alpha = 1.0) {
-        return (ds ? zgemm_tn_ds : zgemm_tn)(M, npw, K, A, lda, nullptr, B, ld, C, ld, acc, s, alpha);
+        return (ds ? zgemm_tn_ds : zgemm_tn)(M, npw, K, A, lda, nullptr, B, ld, C, ld, acc, w.part, s, alpha);
     }
     // products whose precision follows the phase: H_sub columns and the Ritz vectors
     qm_status gemm_cn(int M, int N, const double2* A, const double2* B, double2* C, int ldc) {
@@ -347,15 +348,15 @@ struct DavidsonRun {
         if ((st = cuda_check(cudaGetLastError(), "k_cols_to_rows launch"))) return st;
         auto cgs = [&](double2* Pr, int n) -> qm_status {
             qm_status s2;
-            if ((s2 = zgemm_cn(nb, n, m, w.CT, nsq, Pr, nsq, w.A, n, w.Part, zgemm_cn_splits(nb, n, m), s)) ||
-                (s2 = zgemm_tn(n, m, nb, w.A, n, nullptr, w.CT, nsq, Pr, nsq, true, s, -1.0)))
+            if ((s2 = zgemm_cn(nb, n, m, w.CT, nsq, Pr, nsq, w.A, n, w.part, s)) ||
+                (s2 = zgemm_tn(n, m, nb, w.A, n, nullptr, w.CT, nsq, Pr, nsq, true, w.part, s, -1.0)))
                 return s2;
             return QM_OK;
         };
         auto cholqr_c = [&](double2* src, int n, double2* dst, double drop, int* k) -> qm_status {
             qm_status s2;
             int kk = 0;
-            if ((s2 = zgemm_cn(n, n, m, src, nsq, src, nsq, w.G, n, w.Part, zgemm_cn_splits(n, n, m), s)) ||
+            if ((s2 = zgemm_cn(n, n, m, src, nsq, src, nsq, w.G, n, w.part, s)) ||
                 (s2 = chol_transform(w.G, n, n, drop, w.sel, w.rank, w.info, w.A, w.Z, 0, s)) ||
                 (s2 = cuda_check(cudaMemcpyAsync(&kk, w.info, sizeof(int), cudaMemcpyDeviceToHost, s), "D2H kept")) ||
                 (s2 = cuda_check(cudaStreamSynchronize(s), "stream sync")))
@@ -363,7 +364,7 @@ struct DavidsonRun {
             *k = kk;
             if (kk == 0) return QM_OK;
             if ((s2 = chol_transform_rows(w.G, n, n, w.sel, w.rank, kk, w.A, w.Z, s))) return s2;
-            return zgemm_tn(kk, m, n, w.Z, kk, nullptr, src, nsq, dst, nsq, false, s);
+            return zgemm_tn(kk, m, n, w.Z, kk, nullptr, src, nsq, dst, nsq, false, w.part, s);
         };
         int k1 = 0, k2 = 0;
         if ((st = cgs(w.PT, nu)) || (st = cgs(w.PT, nu))) return st;
@@ -532,7 +533,8 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
     const size_t sqb = (size_t)nsq * nb * sizeof(double2);
     const size_t oCp = take(thick ? sqb : 0), oCT = take(thick ? sqb : 0), oPT = take(thick ? sqb : 0),
                  oQT = take(thick ? sqb : 0), oY = take(thick ? big * nb : 0), oHY = take(thick ? big * nb : 0);
-    const size_t oPart = take(gemm_cn_partial_bytes(false));
+    const size_t part_bytes = std::max(gemm_cn_partial_bytes(false), std::max(zgemm_cn_bytes(nvx, nvx, npw), zgemm_tn_bytes(nvx, npw, nvx)));
+    const size_t oPart = take(part_bytes);
     const size_t oEval = take(sizeof(double) * nsq), oEps = take(sizeof(double) * nsq),
                  oRn = take(sizeof(double) * nsq), oTk = take(sizeof(double) * nsq),
                  oSel = take(sizeof(int) * nsq), oRank = take(sizeof(int) * nsq), oInfo = take(sizeof(int) * 4),
@@ -570,7 +572,7 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
     w.A = (double2*)(base + oA);
     w.Z = (double2*)(base + oZ);
     w.Cs = (double2*)(base + oCs);
-    w.Part = (double2*)(base + oPart);
+    w.part = GemmWork{base + oPart, part_bytes};
     if (thick) {
         w.Cp = (double2*)(base + oCp);
         w.CT = (double2*)(base + oCT);

@@ -24,7 +24,7 @@ constexpr size_t kStickBudget = 48ull << 20;
 constexpr size_t kStickBudgetOverlap = 1ull << 30;
 
 struct HpsiLayout {
-    size_t vt_off, p_off, part_off, t_off, nl_off, err_off, total, t_bytes;
+    size_t vt_off, p_off, part_off, part_bytes, t_off, nl_off, err_off, total, t_bytes;
     int splits;
 };
 
@@ -42,7 +42,10 @@ static HpsiLayout hpsi_layout(qm_gspace g, int ik, int nb, int nproj, bool fp32,
     L.p_off = off;
     off = align_up(off + (size_t)nproj * nb * cs, 256);
     L.part_off = off;
-    off = align_up(off + (L.splits > 1 ? std::min((size_t)L.splits * nproj * nb * cs, gemm_cn_partial_bytes(fp32)) : 0), 256);
+    // scratch of the two FP64 projector products
+    L.part_bytes = fp32 || nproj == 0 ? 0 : std::max(std::max(zgemm_cn_bytes(nproj, nb, npw), zgemm_tn_bytes(nb, npw, nproj)),
+                                                     std::min((size_t)L.splits * nproj * nb * cs, gemm_cn_partial_bytes(false)));
+    off = align_up(off + L.part_bytes, 256);
     L.t_off = off;
     const size_t per_band = stick_buffer_bytes_per_band(g, ik, fp32);
     // the precision form keeps every band's stick buffer (K1 and K2 of all bands overlap the
@@ -110,7 +113,7 @@ qm_status qm::hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi,
     char* ws = (char*)g->ws.ptr;
     void* vt = ws + L.vt_off;
     void* P = ws + L.p_off;
-    void* part = ws + L.part_off;
+    const GemmWork gw{ws + L.part_off, L.part_bytes};
     void* T = ws + L.t_off;
 
     if (fp32 && nproj > 0) {
@@ -131,8 +134,7 @@ qm_status qm::hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi,
     if ((st = launch_vt_prepare(g, vloc_r, vt, fp32, s))) return st;
     if (nproj > 0 && !fp32) {
         st = (ds_nonlocal ? zgemm_cn_ds : zgemm_cn)(nproj, nb, npw, (const double2*)beta, ld_beta,
-                                                    (const double2*)psi, ld_psi, (double2*)P, nb, (double2*)part,
-                                                    L.splits, s);
+                                                    (const double2*)psi, ld_psi, (double2*)P, nb, gw, s);
         if (st) return st;
     }
     if ((st = launch_local_kinetic(g, ik, nb, psi, ld_psi, vt, out, ld_out, T, L.t_bytes, fp32, s, nullptr, false,
@@ -140,7 +142,7 @@ qm_status qm::hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi,
         return st;
     if (nproj > 0 && !fp32) {
         st = (ds_nonlocal ? zgemm_tn_ds : zgemm_tn)(nb, npw, nproj, (const double2*)P, nb, D, (const double2*)beta,
-                                                    ld_beta, (double2*)out, ld_out, true, s, 1.0);
+                                                    ld_beta, (double2*)out, ld_out, true, gw, s, 1.0);
         if (st) return st;
     }
     return QM_OK;

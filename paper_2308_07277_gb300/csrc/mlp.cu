@@ -818,20 +818,21 @@ extern "C" qm_status qm_mlp_pairs(qm_gspace g, int ik, int n, const void* psi, i
     qm_status st = ensure_device(g);
     if (st) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    const int splits = zgemm_cn_splits(nu, n, npw);
+    GemmWork gw;
+    gw.bytes = std::max(zgemm_cn_bytes(nu, n, npw), zgemm_tn_bytes(n, npw, nu));
     DevBuf S(s), part(s), P(s), ok(s);
-    if ((st = S.get(sizeof(double2) * (size_t)nu * n)) || (st = part.get(sizeof(double2) * (size_t)splits * nu * n)) ||
+    if ((st = S.get(sizeof(double2) * (size_t)nu * n)) || (gw.bytes && (st = part.get(gw.bytes))) ||
         (st = P.get(sizeof(double2) * (size_t)n * npw)) || (st = ok.get(sizeof(int) * (size_t)n)))
         return st;
-    if ((st = zgemm_cn(nu, n, npw, (const double2*)U, ld_u, (const double2*)psi, ld_psi, (double2*)S.p, n,
-                       (double2*)part.p, splits, s)))
+    gw.ptr = part.p;
+    if ((st = zgemm_cn(nu, n, npw, (const double2*)U, ld_u, (const double2*)psi, ld_psi, (double2*)S.p, n, gw, s)))
         return st;
     {
         ProfScope pf(PF_MLP, s);
         k_mlp_cluster<<<(n + 127) / 128, 128, 0, s>>>(lam, nu, n, cluster_tol, (double2*)S.p, n, (int*)ok.p);
     }
     if ((st = zgemm_tn(n, npw, nu, (const double2*)S.p, n, nullptr, (const double2*)U, ld_u, (double2*)P.p, npw, false,
-                       s)))
+                       gw, s)))
         return st;
     {
         ProfScope pf(PF_MLP, s);

@@ -203,22 +203,31 @@ qm_status launch_local_kinetic_tab(const DevTables& t, int nb, const void* psi, 
                                    cudaStream_t s);
 
 // ---- complex GEMMs (zgemm.cu) ----
+// Device scratch of the FP64 products: zgemm_cn_bytes / zgemm_tn_bytes of the product (or of one at
+// least as large in every dimension) serve it best; with less (none: ptr NULL) it runs with fewer
+// splits.
+struct GemmWork {
+    void* ptr = nullptr;
+    size_t bytes = 0;
+};
+size_t zgemm_cn_bytes(int M, int N, int K);
+size_t zgemm_tn_bytes(int M, int N, int K);
 // C[m][n] = sum_k conj(A[m][k]) * B[n][k]   (A: M rows, B: N rows, k contiguous);
-// split over K into `splits` partial sums reduced in a fixed order (deterministic).
+// split over K into partial sums reduced in a fixed order (deterministic).
 qm_status zgemm_cn(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb,
-                   double2* C, int ldc, double2* partial, int splits, cudaStream_t s);
+                   double2* C, int ldc, const GemmWork& w, cudaStream_t s);
 // C[m][n] (+)= alpha * sum_k A[k][m] * d[k] * B[k][n]   (d may be NULL -> 1)
 qm_status zgemm_tn(int M, int N, int K, const double2* A, int lda, const double* d,
-                   const double2* B, int ldb, double2* C, int ldc, bool accumulate,
+                   const double2* B, int ldb, double2* C, int ldc, bool accumulate, const GemmWork& w,
                    cudaStream_t s, double alpha = 1.0);
 int zgemm_cn_splits(int M, int N, int K);
 // the same two products in double-FP32 arithmetic (FP64 in and out, products and sums on the
 // FP32 pipe with error-free transformations, ~2^-46 relative accuracy): the precision form's
 // FP64 phase
 qm_status zgemm_cn_ds(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb,
-                      double2* C, int ldc, double2* partial, int splits, cudaStream_t s);
+                      double2* C, int ldc, const GemmWork& w, cudaStream_t s);
 qm_status zgemm_tn_ds(int M, int N, int K, const double2* A, int lda, const double* d,
-                      const double2* B, int ldb, double2* C, int ldc, bool accumulate,
+                      const double2* B, int ldb, double2* C, int ldc, bool accumulate, const GemmWork& w,
                       cudaStream_t s, double alpha = 1.0);
 // ---- tensor-core nonlocal step of the precision form (nonlocal_tc.cu) ----
 constexpr int kMaxUmmaSplits = 64;

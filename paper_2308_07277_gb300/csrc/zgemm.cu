@@ -10,7 +10,7 @@
 //
 // 16 x 16 threads per CTA, each owning a TM x TN block of outputs (tile 16TM x 16TN); the
 // per-call tile is chosen so that the M and N edges waste as little as possible (160
-// bands -> TM = 5, 256 projectors -> TM = 4).  With FP32 arithmetic the products of one K tile
+// bands -> TM = 5, 256 projectors -> TM = 4); FP64 has its own kernels below.  With FP32 arithmetic the products of one K tile
 // (16 terms) are summed in FP32 and the tile sums in FP64, so the rounding error does not grow
 // with K (inner products over 10^4 - 10^5 plane waves keep ~1e-7 relative accuracy).
 #include <algorithm>
@@ -341,6 +341,156 @@ k_gemm_tn(int M, int N, int K, const C* __restrict__ A, int lda, const double* _
     }
 }
 
+// ---------------------------------------------------------------- FP64
+// FP64 multiply-adds issue at two lanes per clock per SM here (a warp instruction takes 16
+// cycles), so an FP64 product is bound by that pipe whatever the operands cost: one output per
+// thread with both factors read from shared memory for every term (two 128-bit loads beside four
+// multiply-adds) keeps the pipe full, and what counts is that no lane works on padding and that
+// every SM gets a share.  Tiles are therefore small (8 x 8 with four K groups for cn, 8 x 32 for
+// tn) and cn is split over K until the CTAs fill the SMs.  The register-tiled 80 x 80 ... 32 x 32
+// tiles these replace padded 8 bands to 32 and ran a small product on one SM: 900 us for a 32 x 8
+// product of 1060 terms, 85 % of the self-consistency of an 8-atom cell.  Measured: that run's first
+// two steps 1249 -> 164 ms, H psi of the two-atom cell (8 x 8 x 411) 518 -> 65 us, and at large
+// sizes 1.22 instead of 1.01 TFLOP/s (480 x 157 x 18232, 10.9 -> 9.0 ms).
+constexpr int kCnTile = 8, kCnK = 32, kCnGroups = 4;
+__global__ void __launch_bounds__(NTH)
+k_zcn(int M, int N, int K, const double2* __restrict__ A, int lda, const double2* __restrict__ B, int ldb,
+      double2* __restrict__ out, int ldo, int kchunk) {
+    __shared__ double2 As[kCnK][kCnTile + 1], Bs[kCnK][kCnTile + 1];
+    const int tid = threadIdx.x, tx = tid & 7, ty = (tid >> 3) & 7, kg = tid >> 6;
+    const int m0 = blockIdx.y * kCnTile, n0 = blockIdx.x * kCnTile;
+    const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
+    const int lrow = tid / kCnK, lk = tid % kCnK;  // this thread's element of a tile (one row per warp)
+    double2 acc = make_double2(0.0, 0.0);
+    const bool va = m0 + lrow < M, vb = n0 + lrow < N;
+    const double2* pa = A + (size_t)(va ? m0 + lrow : 0) * lda + lk;
+    const double2* pb = B + (size_t)(vb ? n0 + lrow : 0) * ldb + lk;
+    double2 ra = make_double2(0.0, 0.0), rb = ra;
+    if (kb + lk < ke) {
+        if (va) ra = pa[kb];
+        if (vb) rb = pb[kb];
+    }
+    for (int k0 = kb; k0 < ke; k0 += kCnK) {
+        As[lk][lrow] = ra;
+        Bs[lk][lrow] = rb;
+        __syncthreads();
+        ra = rb = make_double2(0.0, 0.0);
+        if (k0 + kCnK + lk < ke) {  // the next tile's loads are in flight during this tile's products
+            if (va) ra = pa[k0 + kCnK];
+            if (vb) rb = pb[k0 + kCnK];
+        }
+#pragma unroll
+        for (int q = 0; q < kCnK / kCnGroups; ++q) {
+            const double2 a = As[kg + kCnGroups * q][ty], b = Bs[kg + kCnGroups * q][tx];
+            acc.x = fma(a.x, b.x, fma(a.y, b.y, acc.x));
+            acc.y = fma(a.x, b.y, fma(-a.y, b.x, acc.y));
+        }
+        __syncthreads();
+    }
+    double2* red = &As[0][0];  // 3 x 64 partial sums of the K groups, added in group order
+    if (kg) red[(kg - 1) * 64 + ty * 8 + tx] = acc;
+    __syncthreads();
+    if (kg == 0 && m0 + ty < M && n0 + tx < N) {
+        for (int g = 0; g < kCnGroups - 1; ++g) {
+            const double2 v = red[g * 64 + ty * 8 + tx];
+            acc.x += v.x;
+            acc.y += v.y;
+        }
+        out[((size_t)blockIdx.z * M + m0 + ty) * ldo + n0 + tx] = acc;
+    }
+}
+
+constexpr int kTnM = 8, kTnN = 32, kTnK = 16;
+__global__ void __launch_bounds__(NTH)
+k_ztn(int M, int N, int K, const double2* __restrict__ A, int lda, const double* __restrict__ d, double alpha,
+      const double2* __restrict__ B, int ldb, double2* __restrict__ C, int ldc, int accumulate) {
+    __shared__ double2 As[kTnK][kTnM], Bs[kTnK][kTnN];
+    const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+    const int n0 = blockIdx.x * kTnN, m0 = blockIdx.y * kTnM;
+    double2 acc = make_double2(0.0, 0.0);
+    for (int k0 = 0; k0 < K; k0 += kTnK) {
+        if (tid < kTnK * kTnM) {
+            const int kk = tid / kTnM, m = m0 + tid % kTnM, k = k0 + kk;
+            double2 v = make_double2(0.0, 0.0);
+            if (k < K && m < M) {
+                v = A[(size_t)k * lda + m];
+                const double sc = d ? alpha * d[k] : alpha;
+                v.x *= sc;
+                v.y *= sc;
+            }
+            As[kk][tid % kTnM] = v;
+        }
+#pragma unroll
+        for (int q = 0; q < kTnK * kTnN / NTH; ++q) {
+            const int kk = ty + q * (NTH / kTnN), k = k0 + kk, n = n0 + tx;
+            Bs[kk][tx] = (k < K && n < N) ? B[(size_t)k * ldb + n] : make_double2(0.0, 0.0);
+        }
+        __syncthreads();
+        const int kn = min(kTnK, K - k0);
+        for (int kk = 0; kk < kn; ++kk) {
+            const double2 a = As[kk][ty], b = Bs[kk][tx];
+            acc.x = fma(a.x, b.x, fma(-a.y, b.y, acc.x));
+            acc.y = fma(a.x, b.y, fma(a.y, b.x, acc.y));
+        }
+        __syncthreads();
+    }
+    const int m = m0 + ty, n = n0 + tx;
+    if (m < M && n < N) {
+        double2* p = C + (size_t)m * ldc + n;
+        if (accumulate) {
+            const double2 o = *p;
+            acc.x += o.x;
+            acc.y += o.y;
+        }
+        *p = acc;
+    }
+}
+
+// Splits of cn over K: the count that minimises (waves of one CTA per SM) x (cycles per CTA) plus
+// the reduction of the partial sums, 128 pipe cycles per term of an 8 x 8 tile; the fixed costs
+// (1500 cycles of start and loads, 4000 of the second launch) are estimates of launch latency.
+int zcn_splits(int M, int N, int K, long cap) {
+    const long tiles = (long)((M + kCnTile - 1) / kCnTile) * ((N + kCnTile - 1) / kCnTile), sms = device_sms();
+    const int smax = (int)std::max<long>(1, std::min<long>({(long)((K + kCnK - 1) / kCnK), cap, 64L}));
+    int best = 1;
+    long cost = -1;
+    for (int s = 1; s <= smax; ++s) {
+        const long kc = ((K + s - 1) / s + kCnK - 1) / kCnK * kCnK;
+        const long c = (tiles * s + sms - 1) / sms * (kc * 128 + 1500) + (s > 1 ? 4000 + 40L * s : 0);
+        if (cost < 0 || c < cost) {
+            cost = c;
+            best = s;
+        }
+    }
+    return best;
+}
+
+qm_status zcn_launch(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb, double2* C, int ldc,
+                     double2* partial, size_t partial_bytes, cudaStream_t s) {
+    const long cap = partial ? (long)(partial_bytes / sizeof(double2)) / ((long)M * N) : 1;
+    int splits = zcn_splits(M, N, K, std::max<long>(1, cap));
+    int kchunk = std::max(kCnK, ((K + splits - 1) / splits + kCnK - 1) / kCnK * kCnK);
+    splits = std::max(1, (K + kchunk - 1) / kchunk);
+    const dim3 grid((N + kCnTile - 1) / kCnTile, (M + kCnTile - 1) / kCnTile, splits);
+    {
+        ProfScope pf(PF_GEMM_CN, s);
+        k_zcn<<<grid, NTH, 0, s>>>(M, N, K, A, lda, B, ldb, splits > 1 ? partial : C, splits > 1 ? N : ldc, kchunk);
+    }
+    if (splits > 1) {
+        ProfScope pf(PF_REDUCE, s);
+        k_reduce_splits<double2><<<grid_stride_blocks((size_t)M * N, 64, 16), 64, 0, s>>>(M, N, partial, splits, C, ldc);
+    }
+    return cuda_check(cudaGetLastError(), "gemm_cn launch");
+}
+
+qm_status ztn_launch(int M, int N, int K, const double2* A, int lda, const double* d, double alpha, const double2* B,
+                     int ldb, double2* C, int ldc, bool accumulate, cudaStream_t s) {
+    ProfScope pf(PF_GEMM_TN, s);
+    const dim3 grid((N + kTnN - 1) / kTnN, (M + kTnM - 1) / kTnM);
+    k_ztn<<<grid, NTH, 0, s>>>(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate ? 1 : 0);
+    return cuda_check(cudaGetLastError(), "gemm_tn launch");
+}
+
 // thread-tile size for one dimension: the T in {5, 4, 2} (BM = 16 T) that pads n least
 int pick_t(int n) {
     int best = 4;
@@ -469,28 +619,41 @@ size_t gemm_cn_partial_bytes(bool fp32) {
 int zgemm_cn_splits(int M, int N, int K) {
     (void)M;
     (void)N;
-    return std::max(1, std::min(kMaxSlots, K / 128));
+    return std::max(1, std::min(64, (K + kCnK - 1) / kCnK));
 }
 
-qm_status zgemm_cn(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb, double2* C,
-                   int ldc, double2* partial, int splits, cudaStream_t s) {
-    return gemm_cn_impl<double2, double2>(M, N, K, A, lda, B, ldb, C, ldc, partial, splits, s);
+size_t zgemm_cn_bytes(int M, int N, int K) {
+    if (M <= 0 || N <= 0) return 0;
+    const int splits = zcn_splits(M, N, K, 64);
+    return splits > 1 ? (size_t)splits * M * N * sizeof(double2) : 0;
+}
+size_t zgemm_tn_bytes(int, int, int) { return 0; }
+
+qm_status zgemm_cn(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb, double2* C, int ldc,
+                   const GemmWork& w, cudaStream_t s) {
+    if (M <= 0 || N <= 0) return QM_OK;
+    return zcn_launch(M, N, K, A, lda, B, ldb, C, ldc, (double2*)w.ptr, w.bytes, s);
+}
+qm_status zgemm_tn(int M, int N, int K, const double2* A, int lda, const double* d, const double2* B, int ldb,
+                   double2* C, int ldc, bool accumulate, const GemmWork& w, cudaStream_t s, double alpha) {
+    if (M <= 0 || N <= 0) return QM_OK;
+    (void)w;
+    return ztn_launch(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate, s);
 }
 qm_status zgemm_cn_ds(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb, double2* C,
-                      int ldc, double2* partial, int splits, cudaStream_t s) {
-    return gemm_cn_impl<double2, ds2>(M, N, K, A, lda, B, ldb, C, ldc, partial, splits, s);
+                      int ldc, const GemmWork& w, cudaStream_t s) {
+    const size_t one = std::max<size_t>(1, (size_t)M * N * sizeof(double2));
+    return gemm_cn_impl<double2, ds2>(M, N, K, A, lda, B, ldb, C, ldc, (double2*)w.ptr,
+                                      (int)std::min<size_t>(64, w.bytes / one), s);
 }
 qm_status zgemm_tn_ds(int M, int N, int K, const double2* A, int lda, const double* d, const double2* B, int ldb,
-                      double2* C, int ldc, bool accumulate, cudaStream_t s, double alpha) {
+                      double2* C, int ldc, bool accumulate, const GemmWork& w, cudaStream_t s, double alpha) {
+    (void)w;
     return gemm_tn_impl<double2, ds2>(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate, s);
 }
 qm_status cgemm_cn(int M, int N, int K, const float2* A, int lda, const float2* B, int ldb, float2* C, int ldc,
                    float2* partial, int splits, cudaStream_t s) {
     return gemm_cn_impl<float2, float2>(M, N, K, A, lda, B, ldb, C, ldc, partial, splits, s);
-}
-qm_status zgemm_tn(int M, int N, int K, const double2* A, int lda, const double* d, const double2* B, int ldb,
-                   double2* C, int ldc, bool accumulate, cudaStream_t s, double alpha) {
-    return gemm_tn_impl<double2, double2>(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate, s);
 }
 qm_status cgemm_tn(int M, int N, int K, const float2* A, int lda, const double* d, const float2* B, int ldb,
                    float2* C, int ldc, bool accumulate, cudaStream_t s, double alpha) {
@@ -534,16 +697,16 @@ extern "C" qm_status qm_zgemm(int op, int arith, int M, int N, int K, const void
         if (!st && e) st = fail(QM_ERR_TIMEOUT, "qm_zgemm: a bounded tensor-core wait expired");
         return st;
     }
-    if (op == 1)
-        return (arith ? zgemm_tn_ds : zgemm_tn)(M, N, K, a, lda, nullptr, b, ldb, c, ldc, false, s, 1.0);
-    void* part = nullptr;
-    const int splits = zgemm_cn_splits(M, N, K);
-    const size_t bytes = std::min((size_t)splits * M * N * sizeof(double2), gemm_cn_partial_bytes(false));
-    if (cudaMallocAsync(&part, bytes, s) != cudaSuccess) {
+    const size_t part = std::min((size_t)zgemm_cn_splits(M, N, K) * M * N * sizeof(double2), gemm_cn_partial_bytes(false));
+    const size_t bytes = op == 0 ? (arith ? part : zgemm_cn_bytes(M, N, K)) : 0;
+    GemmWork w;
+    w.bytes = bytes;
+    if (bytes && cudaMallocAsync(&w.ptr, bytes, s) != cudaSuccess) {
         cudaGetLastError();
-        return fail(QM_ERR_OOM, "qm_zgemm: split-K partial sums");
+        return fail(QM_ERR_OOM, "qm_zgemm: workspace");
     }
-    qm_status st = (arith ? zgemm_cn_ds : zgemm_cn)(M, N, K, a, lda, b, ldb, c, ldc, (double2*)part, splits, s);
-    cudaFreeAsync(part, s);
+    qm_status st = op == 0 ? (arith ? zgemm_cn_ds : zgemm_cn)(M, N, K, a, lda, b, ldb, c, ldc, w, s)
+                           : (arith ? zgemm_tn_ds : zgemm_tn)(M, N, K, a, lda, nullptr, b, ldb, c, ldc, false, w, s, 1.0);
+    if (w.ptr) cudaFreeAsync(w.ptr, s);
     return st;
 }
