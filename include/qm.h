@@ -51,7 +51,7 @@ typedef enum {
 } qm_status;
 
 typedef enum {
-    QM_FP64 = 0,   /* everything in FP64 */
+    QM_FP64 = 0,   /* everything to FP64 accuracy (large complex products: see qm_zgemm, arith 0) */
     QM_MIXED = 1   /* FP32 FFT path and V multiply; nonlocal projection and application as
                       3-term BF16 split products on the tensor cores, FP32 accumulation */
 } qm_precision;
@@ -168,7 +168,7 @@ qm_status qm_hpsi_gamma(qm_gspace g, int ik, int nb,
 /*
  * qm_hpsi_check - synchronise `stream` and read (and clear) the handle's sticky error word:
  * QM_ERR_TIMEOUT if a bounded device-side wait of a tensor-core kernel launched by an earlier
- * qm_hpsi(QM_MIXED) or qm_precond_apply call on this handle expired since the last check (the
+ * qm_hpsi or qm_precond_apply call on this handle expired since the last check (the
  * outputs of such a call are undefined), else QM_OK.  qm_davidson checks it itself.
  */
 qm_status qm_hpsi_check(qm_gspace g, void* stream);
@@ -385,13 +385,10 @@ typedef struct {
                             of the unconverged bands (GD+k: Stathopoulos & Saad, ETNA 7, 163 (1998)),
                             as many as fit beside the next corrections; 1 = plain restart from the
                             Ritz vectors only */
-    int fp64_exact;      /* QM_MIXED, FP64 phase: 0 (default) = its plane-wave-length products (H_sub
-                            columns, Ritz vectors, orthogonalisation passes, and the nonlocal
-                            GEMMs of its H psi) in double-FP32 arithmetic: FP64 operands split into
-                            two FP32 halves, products and sums by error-free transformations on the
-                            FP32 pipe, partial sums in FP64 (about 2^-46 relative accuracy, 47-bit
-                            rather than 53-bit); 1 = those products in FP64 arithmetic.  QM_FP64
-                            is FP64 arithmetic throughout, whatever this field says */
+    int fp64_exact;      /* 0 or 1; both run the FP64 phase of QM_MIXED on the products of QM_FP64 (FP64
+                            multiply-adds, or exact digit products on the tensor cores where those are
+                            faster, see qm_zgemm), whose error is never above FP64 arithmetic's.  (The
+                            field chose a 47-bit arithmetic before those products existed.) */
 } qm_davidson_opts;
 
 /* Counters of one qm_davidson call (the paper's "H-psi calls" are band_applies / nb). */
@@ -538,14 +535,16 @@ qm_status qm_eigh_lowest(int m, int nev, const void* A, int lda, double* evals, 
  * own so that their arithmetic can be checked:
  *   op 0 (cn): C[m][n] = sum_k conj(A[m][k]) B[n][k]     A: M x K, B: N x K (k contiguous)
  *   op 1 (tn): C[m][n] = sum_k A[k][m] B[k][n]           A: K x M, B: K x N (m, n contiguous)
- *  arith   0 = FP64 arithmetic; 1 = double-FP32 (the precision form's FP64 phase, see
- *          qm_davidson_opts.fp64_exact): operands split into two FP32 halves, error-free
- *          products and sums on the FP32 pipe, per-tile sums in FP64; 2 = 3-term BF16 split
- *          products on the tensor cores accumulated in FP32 (the precision form's FP32 phase;
- *          FP32-level accuracy; synchronises the stream).
+ *  arith   0 = FP64: multiply-adds for small products; larger ones as exact sums of 8-bit digit
+ *          products on the tensor cores, every operand element rounded at 2^-56 of the largest
+ *          component of its row (of A or B along k) and the sum rounded once, which measures
+ *          closer to the exact value than FP64 multiply-adds (rows with non-finite values, or with
+ *          nothing above 2^-960, run in multiply-adds); 1 = the same (a 47-bit arithmetic before);
+ *          2 = 3-term BF16 split products on the tensor cores accumulated in FP32 (the precision
+ *          form's FP32 phase; FP32-level accuracy; synchronises the stream).
  *  A, B, C device, complex double, row-major with the leading dimensions given; C is written.
- *  stream  cudaStream_t.  Split-K partial sums and tensor-core workspaces are allocated with
- *          cudaMallocAsync on the stream.
+ *  stream  cudaStream_t.  Partial sums, digit planes (at most about 600 MB) and tensor-core
+ *          workspaces are allocated with cudaMallocAsync on the stream.
  * M, N, K >= 1.  Errors: QM_ERR_ARG, QM_ERR_CUDA, QM_ERR_OOM, QM_ERR_TIMEOUT (arith 2).
  */
 qm_status qm_zgemm(int op, int arith, int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C,

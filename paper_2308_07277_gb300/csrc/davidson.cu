@@ -287,10 +287,9 @@ struct DavidsonRun {
     size_t sub_bytes = 0;
     int* tc_err = nullptr;       // device error word of the tensor-core waits
 
-    bool ds = false;             // precision form: the FP64 phase's long products in double-FP32
     qm_status hpsi(const double2* in, double2* out, int n) {
         applies += n;
-        if (!mixed) return hpsi_run(g, ik, n, in, ld, vloc, nproj, beta, ldb, nullptr, D, out, ld, QM_FP64, s, ds);
+        if (!mixed) return hpsi_run(g, ik, n, in, ld, vloc, nproj, beta, ldb, nullptr, D, out, ld, QM_FP64, s);
         applies_mixed += n;
         qm_status st = convert_rows(in, ld, psi32, ld, n, npw, s);
         if (st) return st;
@@ -303,7 +302,7 @@ struct DavidsonRun {
         return zgemm_cn_bf16x3(M, N, npw, A, ld, B, ld, C, ldc, sub, sub_bytes, tc_err, s);
     }
     qm_status cn64(int M, int N, const double2* A, const double2* B, double2* C, int ldc) {
-        return (ds ? zgemm_cn_ds : zgemm_cn)(M, N, npw, A, ld, B, ld, C, ldc, w.part, s);
+        return zgemm_cn(M, N, npw, A, ld, B, ld, C, ldc, w.part, s);
     }
     qm_status tn_tc(int M, int K, const double2* A, int lda, const double2* B, double2* C, bool acc,
                     double alpha = 1.0) {
@@ -311,7 +310,7 @@ struct DavidsonRun {
     }
     qm_status tn64(int M, int K, const double2* A, int lda, const double2* B, double2* C, bool acc,
                    double alpha = 1.0) {
-        return (ds ? zgemm_tn_ds : zgemm_tn)(M, npw, K, A, lda, nullptr, B, ld, C, ld, acc, w.part, s, alpha);
+        return zgemm_tn(M, npw, K, A, lda, nullptr, B, ld, C, ld, acc, w.part, s, alpha);
     }
     // products whose precision follows the phase: H_sub columns and the Ritz vectors
     qm_status gemm_cn(int M, int N, const double2* A, const double2* B, double2* C, int ldc) {
@@ -562,7 +561,6 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
         }
         run.mixed = true;
         run.tc = true;
-        run.ds = o.fp64_exact == 0;
         run.ortho64 = o.mixed_ortho == 1;
         run.sub = base + oSub;
         run.sub_bytes = sub_bytes;
@@ -572,7 +570,7 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
     w.A = (double2*)(base + oA);
     w.Z = (double2*)(base + oZ);
     w.Cs = (double2*)(base + oCs);
-    w.part = GemmWork{base + oPart, part_bytes};
+    w.part = GemmWork{base + oPart, part_bytes, (int*)(base + oInfo) + 3};
     if (thick) {
         w.Cp = (double2*)(base + oCp);
         w.CT = (double2*)(base + oCT);
@@ -592,7 +590,7 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
     w.hdiag = (double*)(base + oHd);
     w.vpart = (double*)(base + oVp);
     run.tc_err = w.info + 3;
-    if (use_mixed && (st = cuda_check(cudaMemsetAsync(run.tc_err, 0, sizeof(int), s), "reset error word"))) return st;
+    if ((st = cuda_check(cudaMemsetAsync(run.tc_err, 0, sizeof(int), s), "reset error word"))) return st;
     const double* kin = g->k[ik].kin;
 
     // initial block: psi -> rows of Tmp (dense ld), orthonormalised into V
@@ -831,7 +829,7 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
             return st;
         if (e) return fail(QM_ERR_TIMEOUT, "qm_davidson: a bounded tensor-core wait of the learned preconditioner expired");
     }
-    if (use_mixed) {
+    {
         int e = 0;
         if ((st = cuda_check(cudaMemcpy(&e, run.tc_err, sizeof(int), cudaMemcpyDeviceToHost), "D2H error word")))
             return st;

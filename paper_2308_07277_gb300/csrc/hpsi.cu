@@ -3,9 +3,9 @@
 //
 // Launch sequence on the caller's stream (no host synchronisation):
 //   1. k_vt            V(r)/N_r laid out in the FFT path's permuted plane order
-//   2. gemm_cn         P[p][b] = <beta_p|psi_b>             (nonlocal projection, FP64)
+//   2. zgemm_cn        P[p][b] = <beta_p|psi_b>             (nonlocal projection, FP64)
 //   3. K1, K2, K3      out = 1/2|k+G|^2 psi + (V psi)(G)    (per chunk of bands)
-//   4. gemm_tn         out += sum_p beta_p D_p P[p][b]      (nonlocal apply, FP64)
+//   4. zgemm_tn        out += sum_p beta_p D_p P[p][b]      (nonlocal apply, FP64)
 // QM_MIXED: the nonlocal part runs as BF16x3 split tcgen05 products (umma.cu) on the handle's
 // second stream, concurrently with k_vt, K1 and K2 of every band: it writes
 // out = sum_p beta_p D_p P[p][b], and K3 (which waits for it) adds the local and kinetic
@@ -25,7 +25,6 @@ constexpr size_t kStickBudgetOverlap = 1ull << 30;
 
 struct HpsiLayout {
     size_t vt_off, p_off, part_off, part_bytes, t_off, nl_off, err_off, total, t_bytes;
-    int splits;
 };
 
 static HpsiLayout hpsi_layout(qm_gspace g, int ik, int nb, int nproj, bool fp32, bool own_beta, bool gamma) {
@@ -34,7 +33,6 @@ static HpsiLayout hpsi_layout(qm_gspace g, int ik, int nb, int nproj, bool fp32,
     const size_t rs = fp32 ? sizeof(float) : sizeof(double);
     const size_t nr = (size_t)g->n[0] * g->n[1] * g->n[2];
     const int npw = g->k[ik].npw;
-    L.splits = nproj > 0 ? zgemm_cn_splits(nproj, nb, npw) : 1;
     size_t off = kWsHeader;  // the header holds the handle's sticky error word
     L.err_off = 0;
     L.vt_off = off;
@@ -43,8 +41,7 @@ static HpsiLayout hpsi_layout(qm_gspace g, int ik, int nb, int nproj, bool fp32,
     off = align_up(off + (size_t)nproj * nb * cs, 256);
     L.part_off = off;
     // scratch of the two FP64 projector products
-    L.part_bytes = fp32 || nproj == 0 ? 0 : std::max(std::max(zgemm_cn_bytes(nproj, nb, npw), zgemm_tn_bytes(nb, npw, nproj)),
-                                                     std::min((size_t)L.splits * nproj * nb * cs, gemm_cn_partial_bytes(false)));
+    L.part_bytes = fp32 || nproj == 0 ? 0 : std::max(zgemm_cn_bytes(nproj, nb, npw), zgemm_tn_bytes(nb, npw, nproj));
     off = align_up(off + L.part_bytes, 256);
     L.t_off = off;
     const size_t per_band = stick_buffer_bytes_per_band(g, ik, fp32);
@@ -76,7 +73,7 @@ extern "C" qm_status qm_hpsi(qm_gspace g, int ik, int nb, const void* psi, int l
 
 qm_status qm::hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi, const double* vloc_r, int nproj,
                        const void* beta, int ld_beta, const void* beta_prepared, const double* D, void* out,
-                       int ld_out, qm_precision prec, cudaStream_t s, bool ds_nonlocal, bool gamma) {
+                       int ld_out, qm_precision prec, cudaStream_t s, bool gamma) {
     if (!g) return fail(QM_ERR_ARG, "qm_hpsi: NULL gspace");
     if (ik < 0 || ik >= g->nk) return fail(QM_ERR_ARG, "qm_hpsi: ik out of range");
     if (nb < 0 || nproj < 0) return fail(QM_ERR_ARG, "qm_hpsi: negative nb or nproj");
@@ -113,7 +110,7 @@ qm_status qm::hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi,
     char* ws = (char*)g->ws.ptr;
     void* vt = ws + L.vt_off;
     void* P = ws + L.p_off;
-    const GemmWork gw{ws + L.part_off, L.part_bytes};
+    const GemmWork gw{ws + L.part_off, L.part_bytes, (int*)(ws + L.err_off)};
     void* T = ws + L.t_off;
 
     if (fp32 && nproj > 0) {
@@ -133,16 +130,15 @@ qm_status qm::hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi,
     }
     if ((st = launch_vt_prepare(g, vloc_r, vt, fp32, s))) return st;
     if (nproj > 0 && !fp32) {
-        st = (ds_nonlocal ? zgemm_cn_ds : zgemm_cn)(nproj, nb, npw, (const double2*)beta, ld_beta,
-                                                    (const double2*)psi, ld_psi, (double2*)P, nb, gw, s);
+        st = zgemm_cn(nproj, nb, npw, (const double2*)beta, ld_beta, (const double2*)psi, ld_psi, (double2*)P, nb, gw, s);
         if (st) return st;
     }
     if ((st = launch_local_kinetic(g, ik, nb, psi, ld_psi, vt, out, ld_out, T, L.t_bytes, fp32, s, nullptr, false,
                                    gamma)))
         return st;
     if (nproj > 0 && !fp32) {
-        st = (ds_nonlocal ? zgemm_tn_ds : zgemm_tn)(nb, npw, nproj, (const double2*)P, nb, D, (const double2*)beta,
-                                                    ld_beta, (double2*)out, ld_out, true, gw, s, 1.0);
+        st = zgemm_tn(nb, npw, nproj, (const double2*)P, nb, D, (const double2*)beta, ld_beta, (double2*)out, ld_out,
+                      true, gw, s);
         if (st) return st;
     }
     return QM_OK;
@@ -153,7 +149,7 @@ extern "C" qm_status qm_hpsi_gamma(qm_gspace g, int ik, int nb, const void* psi,
                                    qm_precision prec, void* stream) {
     clear_error();
     return hpsi_run(g, ik, nb, psi, ld_psi, vloc_r, nproj, beta, ld_beta, nullptr, D, out, ld_out, prec,
-                    (cudaStream_t)stream, false, true);
+                    (cudaStream_t)stream, true);
 }
 
 extern "C" qm_status qm_hpsi_prepare(qm_gspace g, int ik, int nproj, const void* beta, int ld_beta, void* stream) {

@@ -214,7 +214,7 @@ extern "C" qm_status qm_hpsi_noalloc(qm_gspace g, int ik, int nb, const void* ps
                           (float2*)part, splits, s);
         else
             st = zgemm_cn(nproj, nb, npw, (const double2*)beta, ld_beta, (const double2*)psi, ld_psi, (double2*)P,
-                          nb, GemmWork{part, splits > 1 ? (size_t)splits * pbytes_split : 0}, s);
+                          nb, GemmWork{part, splits > 1 ? (size_t)splits * pbytes_split : 0, nullptr, false}, s);
         if (st) return st;
     }
     if ((st = launch_local_kinetic_tab(t, nb, psi, ld_psi, vt, out, ld_out, T, t_bytes, fp32, s))) return st;
@@ -224,7 +224,7 @@ extern "C" qm_status qm_hpsi_noalloc(qm_gspace g, int ik, int nb, const void* ps
                           ld_out, true, s);
         else
             st = zgemm_tn(nb, npw, nproj, (const double2*)P, nb, D, (const double2*)beta, ld_beta, (double2*)out,
-                          ld_out, true, GemmWork{}, s);
+                          ld_out, true, GemmWork{nullptr, 0, nullptr, false}, s);
         if (st) return st;
     }
     return cuda_check(cudaGetLastError(), "qm_hpsi_noalloc launches");

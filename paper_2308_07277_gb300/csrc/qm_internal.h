@@ -205,10 +205,20 @@ qm_status launch_local_kinetic_tab(const DevTables& t, int nb, const void* psi, 
 // ---- complex GEMMs (zgemm.cu) ----
 // Device scratch of the FP64 products: zgemm_cn_bytes / zgemm_tn_bytes of the product (or of one at
 // least as large in every dimension) serve it best; with less (none: ptr NULL) it runs with fewer
-// splits.
+// splits and without the digit products.  digits = false: FP64 multiply-adds at every size.
+// err (may be NULL): device word set when a bounded wait of the digit products expired.
 struct GemmWork {
     void* ptr = nullptr;
     size_t bytes = 0;
+    int* err = nullptr;
+    bool digits = true;
+};
+// Rows of a product that the digit products leave to the FP64 kernels: *any != 0 if there are some,
+// output (m, n) is one if em[m] or en[n] equals `flag`.  any = NULL: every output.
+struct GemmFlags {
+    const int* any = nullptr;
+    const int *em = nullptr, *en = nullptr;
+    int flag = 0;
 };
 size_t zgemm_cn_bytes(int M, int N, int K);
 size_t zgemm_tn_bytes(int M, int N, int K);
@@ -221,14 +231,14 @@ qm_status zgemm_tn(int M, int N, int K, const double2* A, int lda, const double*
                    const double2* B, int ldb, double2* C, int ldc, bool accumulate, const GemmWork& w,
                    cudaStream_t s, double alpha = 1.0);
 int zgemm_cn_splits(int M, int N, int K);
-// the same two products in double-FP32 arithmetic (FP64 in and out, products and sums on the
-// FP32 pipe with error-free transformations, ~2^-46 relative accuracy): the precision form's
-// FP64 phase
-qm_status zgemm_cn_ds(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb,
-                      double2* C, int ldc, const GemmWork& w, cudaStream_t s);
-qm_status zgemm_tn_ds(int M, int N, int K, const double2* A, int lda, const double* d,
-                      const double2* B, int ldb, double2* C, int ldc, bool accumulate, const GemmWork& w,
-                      cudaStream_t s, double alpha = 1.0);
+// the same products on the tensor cores by digit splitting (zdigits.cu); *done = false: not served
+// (small, or too little scratch), nothing launched.  *flags: what is left to the FP64 kernels
+qm_status zdigits_cn(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb, double2* C, int ldc,
+                     const GemmWork& w, cudaStream_t s, GemmFlags* flags, bool* done);
+qm_status zdigits_tn(int M, int N, int K, const double2* A, int lda, const double* d, double alpha, const double2* B,
+                     int ldb, double2* C, int ldc, bool accumulate, const GemmWork& w, cudaStream_t s, GemmFlags* flags,
+                     bool* done);
+size_t zdigits_bytes(bool cn, int M, int N, int K);
 // ---- tensor-core nonlocal step of the precision form (nonlocal_tc.cu) ----
 constexpr int kMaxUmmaSplits = 64;
 // out[b][g] (+)= sum_p beta[p][g] D_p <beta_p|psi_b> (FP32 complex in/out) as BF16x3 split
@@ -246,12 +256,11 @@ size_t nonlocal_tc_beta_bytes(int nproj, int nb, int npw);
 qm_status nonlocal_tc_prepare(int nproj, int nb, int npw, const float2* beta, int ld_beta, void* beta_work,
                               cudaStream_t s);
 // qm_hpsi with the precision form's projectors optionally pre-split (beta_prepared, see
-// nonlocal_tc); qm_hpsi itself passes NULL.  ds_nonlocal (QM_FP64 only): the nonlocal GEMMs in
-// double-FP32 arithmetic (zgemm_cn_ds / zgemm_tn_ds), for the precision form's FP64 phase.
+// nonlocal_tc); qm_hpsi itself passes NULL.
 // gamma: the Gamma-point real-wavefunction FFT path (qm_hpsi_gamma; two bands per transform).
 qm_status hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi, const double* vloc_r, int nproj,
                    const void* beta, int ld_beta, const void* beta_prepared, const double* D, void* out, int ld_out,
-                   qm_precision prec, cudaStream_t s, bool ds_nonlocal = false, bool gamma = false);
+                   qm_precision prec, cudaStream_t s, bool gamma = false);
 // Subspace products of the Davidson FP32 phase on the tensor cores: FP64 storage rounded to
 // FP32 on load, BF16x3 split products accumulated in FP32 per K split, splits summed in FP64.
 //   cn: C[i][j] = sum_k conj(A[i][k]) B[j][k]                (as zgemm_cn)
