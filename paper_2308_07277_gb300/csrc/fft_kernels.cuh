@@ -221,6 +221,13 @@ struct CPlan {
 constexpr CPlan make_cplan(int n, int ord = 0) {
     int rs[kMaxStages] = {}, nr = 0, m = n;
     while (m % 8 == 0) { rs[nr++] = 8; m /= 8; }
+    bool tail = false;  // a 3 or 5 is left besides the 9s: the 9s go first (90 = 9 x 10, 54 = 9 x 6, 108 = 9 x 12 in two groups)
+    {
+        int t = m;
+        while (t % 9 == 0) t /= 9;
+        tail = t % 3 == 0 || t % 5 == 0;
+    }
+    while (tail && m % 9 == 0) { rs[nr++] = 9; m /= 9; }
     if (m % 4 == 0) { rs[nr++] = 4; m /= 4; }
     if (m % 2 == 0) { rs[nr++] = 2; m /= 2; }
     while (m % 9 == 0) { rs[nr++] = 9; m /= 9; }

@@ -14,8 +14,12 @@ extern template qm_status local_kinetic_tab_impl<float>(const DevTables&, int, c
                                                         int, void*, size_t, cudaStream_t);
 
 // ---------------------------------------------------------------- host launchers
-size_t stick_buffer_bytes_per_band(qm_gspace g, int ik, bool fp32) {
-    return (size_t)g->n[0] * g->k[ik].nstick_pad * (fp32 ? sizeof(float2) : sizeof(double2));
+size_t stick_buffer_bytes(qm_gspace g, int ik, bool fp32, int ntr, size_t budget) {
+    const bool pair = fp32 && pair_path(g, ntr);
+    const size_t unit = pair ? pair_unit_bytes(g, ik)
+                             : (size_t)g->n[0] * g->k[ik].nstick_pad * (fp32 ? sizeof(float2) : sizeof(double2));
+    const size_t units = pair ? ((size_t)ntr + 1) / 2 : (size_t)ntr;
+    return std::max<size_t>(1, std::min(units, budget / unit)) * unit;
 }
 
 qm_status launch_vt_prepare(qm_gspace g, const double* vloc, void* vt, bool fp32, cudaStream_t s) {
@@ -33,6 +37,10 @@ qm_status launch_vt_prepare(qm_gspace g, const double* vloc, void* vt, bool fp32
 qm_status launch_local_kinetic(qm_gspace g, int ik, int nb, const void* psi, int ld_psi, const void* vt,
                                void* out, int ld_out, void* tbuf, size_t tbuf_bytes, bool fp32, cudaStream_t s,
                                cudaEvent_t wait_k3, bool accumulate, bool gamma) {
+    // pairs of transforms where the grid allows (fft_pair.cuh); single ones on the other grids and
+    // where the buffer holds no pair
+    if (fp32 && pair_path(g, gamma ? (nb + 1) / 2 : nb) && tbuf_bytes >= pair_unit_bytes(g, ik))
+        return local_kinetic_pair(g, ik, nb, psi, ld_psi, vt, out, ld_out, tbuf, tbuf_bytes, s, wait_k3, accumulate, gamma);
     if (fp32)
         return local_kinetic_impl<float>(g, ik, nb, psi, ld_psi, vt, out, ld_out, tbuf, tbuf_bytes, s, wait_k3,
                                          accumulate, gamma);

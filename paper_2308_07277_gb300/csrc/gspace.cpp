@@ -138,6 +138,11 @@ void fft_plan(int n, int order, AxisPlan& p, std::vector<int>& rev) {
     // radices reversed (must match the compile-time plans of the FFT kernels, make_cplan)
     std::vector<int> rs;
     while (m % 8 == 0) { rs.push_back(8); m /= 8; }
+    // (the 9s before the 4 and the 2 where a 3 or a 5 follows, as make_cplan in fft_kernels.cuh)
+    int t9 = m;
+    while (t9 % 9 == 0) t9 /= 9;
+    const bool tail = t9 % 3 == 0 || t9 % 5 == 0;
+    while (tail && m % 9 == 0) { rs.push_back(9); m /= 9; }
     if (m % 4 == 0) { rs.push_back(4); m /= 4; }
     if (m % 2 == 0) { rs.push_back(2); m /= 2; }
     while (m % 9 == 0) { rs.push_back(9); m /= 9; }
@@ -205,7 +210,9 @@ qm_status ensure_device(qm_gspace g) {
             (st = upload((void**)&kt.rows, kt.h_rows.data(), sizeof(int) * kt.h_rows.size())) ||
             (st = upload((void**)&kt.g_code, kt.h_code.data(), sizeof(int2) * kt.h_code.size())) ||
             (st = upload((void**)&kt.kin, kt.h_kin.data(), sizeof(double) * kt.h_kin.size())) ||
-            (st = upload((void**)&kt.kin_f, kinf.data(), sizeof(float) * kinf.size())))
+            (st = upload((void**)&kt.kin_f, kinf.data(), sizeof(float) * kinf.size())) ||
+            (st = upload((void**)&kt.ymap, kt.h_ymap.data(), sizeof(int) * kt.h_ymap.size())) ||
+            (st = upload((void**)&kt.runs, kt.h_runs.data(), sizeof(int4) * kt.h_runs.size())))
             return st;
         if (kt.gamma && (st = upload((void**)&kt.gtile, kt.h_gtile.data(), sizeof(int2) * kt.h_gtile.size())))
             return st;
@@ -427,6 +434,24 @@ extern "C" qm_status qm_gspace_create(const double lattice[9], int nk, const dou
                 kt.h_gtile = std::move(tiles);
             }
         }
+        // active rows as [0, lo) and [hi, N3): the sphere's rows are a run of m_3 around the rows' fold
+        kt.lo = 0;
+        kt.hi = N3;
+        for (int i3 : rows) {
+            if (2 * i3 < N3) kt.lo = std::max(kt.lo, i3 + 1);
+            else kt.hi = std::min(kt.hi, i3);
+        }
+        kt.h_ymap.assign((size_t)(kt.lo + N3 - kt.hi) * N2, -1);
+        kt.h_runs.assign(kt.nstick + 1, make_int4(kt.npw, 0, 0, 0));
+        for (int s2 = 0; s2 < kt.nstick; ++s2) {
+            const int64_t key = pws[g0[s2]].idx / N1;
+            const int i2 = (int)(key % N2), i3 = (int)(key / N2);
+            kt.h_ymap[(size_t)(i3 < kt.lo ? i3 : kt.lo + i3 - kt.hi) * N2 + i2] = s2;
+            // the plane waves of a stick are a run of m_1, i.e. at most two runs of i1
+            int c = g0[s2] + 1;
+            while (c < g0[s2 + 1] && code[c].y == code[c - 1].y + 1) ++c;
+            kt.h_runs[s2] = make_int4(g0[s2], code[g0[s2]].y, c - g0[s2], c < g0[s2 + 1] ? code[c].y : 0);
+        }
         kt.h_g0 = std::move(g0);
         kt.h_plane = std::move(plane);
         kt.h_rows = std::move(rows);
@@ -501,6 +526,8 @@ extern "C" void qm_gspace_destroy(qm_gspace g) {
             cudaFree(kt.kin);
             cudaFree(kt.kin_f);
             cudaFree(kt.gtile);
+            cudaFree(kt.ymap);
+            cudaFree(kt.runs);
         }
         for (int d = 0; d < 3 && !g->shared_tables; ++d) {
             cudaFree(g->tw64[d]);

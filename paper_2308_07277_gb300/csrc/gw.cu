@@ -46,6 +46,8 @@ extern "C" qm_status qm_gw_mel(qm_gspace g, int ik_left, int ik_right, int nl, c
     if ((st = ensure_device(g)) || (st = ensure_device(geps))) return st;
     if (g->device != geps->device) return fail(QM_ERR_ARG, "qm_gw_mel: the handles live on different devices");
     cudaStream_t s = (cudaStream_t)stream;
+    if (prec == QM_MIXED && pair_path(g))
+        return gw_mel_pair(g, ik_left, ik_right, nl, psi_l, ld_l, nr, psi_r, ld_r, geps, iq, M, ld_m, s);
     if (prec == QM_MIXED)
         return gw_mel_impl<float>(g, ik_left, ik_right, nl, psi_l, ld_l, nr, psi_r, ld_r, geps, iq, M, ld_m, s);
     return gw_mel_impl<double>(g, ik_left, ik_right, nl, psi_l, ld_l, nr, psi_r, ld_r, geps, iq, M, ld_m, s);

@@ -44,14 +44,12 @@ static HpsiLayout hpsi_layout(qm_gspace g, int ik, int nb, int nproj, bool fp32,
     L.part_bytes = fp32 || nproj == 0 ? 0 : std::max(zgemm_cn_bytes(nproj, nb, npw), zgemm_tn_bytes(nb, npw, nproj));
     off = align_up(off + L.part_bytes, 256);
     L.t_off = off;
-    const size_t per_band = stick_buffer_bytes_per_band(g, ik, fp32);
     // the precision form keeps every band's stick buffer (K1 and K2 of all bands overlap the
     // nonlocal part; K3 runs once it is done; without projectors the larger launches are faster
     // too), the FP64 form chunks the bands to stay in L2
     const size_t budget = fp32 ? kStickBudgetOverlap : kStickBudget;
     const size_t ntr = gamma ? (size_t)(nb + 1) / 2 : (size_t)nb;  // transforms (band pairs at Gamma)
-    const size_t nbc = std::max<size_t>(1, std::min<size_t>(ntr, budget / per_band));
-    L.t_bytes = nbc * per_band;
+    L.t_bytes = stick_buffer_bytes(g, ik, fp32, (int)ntr, budget);
     off = align_up(off + L.t_bytes, 256);
     L.nl_off = off;  // tensor-core split operands (precision form)
     off = align_up(off + (fp32 && nproj > 0 ? nonlocal_tc_bytes(nproj, nb, npw, own_beta) : 0), 256);

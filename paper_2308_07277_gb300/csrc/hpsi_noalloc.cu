@@ -131,7 +131,7 @@ extern "C" qm_status qm_hpsi_noalloc(qm_gspace g, int ik, int nb, const void* ps
     const size_t room = (size_t)QM_HPSI_NOALLOC_SCRATCH_BYTES - c.off;
     // stick buffer: up to the L2-sized chunk of qm_hpsi, leaving room for the partial sums
     const size_t pbytes_split = (size_t)nproj * nb * cs;
-    size_t t_bytes = std::min(room, std::max(per_band, std::min<size_t>(48ull << 20, (size_t)nb * per_band)));
+    size_t t_bytes = std::min(room, std::max(per_band, std::min<size_t>(48ull << 20, (size_t)(nb + nb % 2) * per_band)));
     t_bytes = t_bytes / per_band * per_band;
     const size_t o_t = c.take(t_bytes);
     int splits = 1;
@@ -217,7 +217,12 @@ extern "C" qm_status qm_hpsi_noalloc(qm_gspace g, int ik, int nb, const void* ps
                           nb, GemmWork{part, splits > 1 ? (size_t)splits * pbytes_split : 0, nullptr, false}, s);
         if (st) return st;
     }
-    if ((st = launch_local_kinetic_tab(t, nb, psi, ld_psi, vt, out, ld_out, T, t_bytes, fp32, s))) return st;
+    // the paired FP32 path reads the handle's own tables, so it serves the calls that have them in place
+    if (fp32 && in_place && pair_path(g, nb) && t_bytes >= pair_unit_bytes(g, ik))
+        st = local_kinetic_pair(g, ik, nb, psi, ld_psi, vt, out, ld_out, T, t_bytes, s, nullptr, false, false);
+    else
+        st = launch_local_kinetic_tab(t, nb, psi, ld_psi, vt, out, ld_out, T, t_bytes, fp32, s);
+    if (st) return st;
     if (nproj > 0) {
         if (fp32)
             st = cgemm_tn(nb, npw, nproj, (const float2*)P, nb, D, (const float2*)beta, ld_beta, (float2*)out,

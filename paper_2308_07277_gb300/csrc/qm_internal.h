@@ -36,6 +36,11 @@ struct KTables {
     int* rows = nullptr;         // [nrow]    active i3 values
     int2* g_code = nullptr;      // [npw]     {stick id, i1}
     double* kin = nullptr;       // [npw]     |k+G|^2 / 2
+    // the paired FP32 path (fft_pair.cuh): active rows are within [0, lo) and [hi, N3);
+    int lo = 0, hi = 0;
+    int* ymap = nullptr;         // [(lo + N3 - hi) * N2]  stick at (row, i2), -1: none
+    int4* runs = nullptr;        // [nstick+1]  first plane wave; first i1 and length of the run of lower i1;
+                                 //             first i1 of the run of higher i1
     float* kin_f = nullptr;      // [npw]     same, FP32
     // Gamma point only (k = 0): tiles of the x-forward pass of the real-wavefunction form, each
     // of kGammaTile slots {stick id (-1: empty), slot of the stick holding -G}; a stick and its
@@ -46,7 +51,8 @@ struct KTables {
     // host copies (the device tables are uploaded from these on first use)
     std::vector<int32_t> h_idx, h_miller;
     std::vector<double> h_kpg, h_kin;
-    std::vector<int> h_g0, h_plane, h_rows;
+    std::vector<int> h_g0, h_plane, h_rows, h_ymap;
+    std::vector<int4> h_runs;
     std::vector<int2> h_code, h_gtile;
 };
 
@@ -180,7 +186,17 @@ qm_status launch_local_kinetic(qm_gspace g, int ik, int nb, const void* psi, int
                                const void* vt, void* out, int ld_out, void* tbuf,
                                size_t tbuf_bytes, bool fp32, cudaStream_t s,
                                cudaEvent_t wait_k3 = nullptr, bool accumulate = false, bool gamma = false);
-size_t stick_buffer_bytes_per_band(qm_gspace g, int ik, bool fp32);
+// stick buffer for ntr transforms within `budget` bytes (at least one launch's least), and that least
+size_t stick_buffer_bytes(qm_gspace g, int ik, bool fp32, int ntr, size_t budget);
+// ---- FP32 path on two transforms at once (fft_pair.cu) ----
+// whether it serves the grid (every length in its list, two planes at once in shared memory) and, given
+// the number of transforms (0: any), whether that many fill the GPU in pairs
+bool pair_path(qm_gspace g, int ntr = 0);
+size_t pair_unit_bytes(qm_gspace g, int ik);  // stick buffer of one pair of transforms
+qm_status local_kinetic_pair(qm_gspace g, int ik, int nb, const void* psi, int ld_psi, const void* vt, void* out, int ld_out,
+                             void* tbuf, size_t tbuf_bytes, cudaStream_t s, cudaEvent_t wait_k3, bool accumulate, bool gamma);
+qm_status gw_mel_pair(qm_gspace g, int ikl, int ikr, int nl, const void* psi_l, int ld_l, int nr, const void* psi_r, int ld_r,
+                      qm_gspace ge, int iq, void* M, int ld_m, cudaStream_t s);
 
 // The FFT path's tables of one k-point given by explicit device pointers (twiddles and kin
 // in the precision of the call).
