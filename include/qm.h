@@ -52,8 +52,9 @@ typedef enum {
 
 typedef enum {
     QM_FP64 = 0,   /* everything to FP64 accuracy (large complex products: see qm_zgemm, arith 0) */
-    QM_MIXED = 1   /* FP32 FFT path and V multiply; nonlocal projection and application as
-                      3-term BF16 split products on the tensor cores, FP32 accumulation */
+    QM_MIXED = 1   /* FP32 FFT path and V multiply; nonlocal projection and application as split
+                      products of FP16 pairs (row-scaled, 23 bits) on the tensor cores, FP32
+                      accumulation; FP32 products on the CUDA cores for small ones */
 } qm_precision;
 
 /*
@@ -176,7 +177,7 @@ qm_status qm_hpsi_check(qm_gspace g, void* stream);
 /*
  * qm_hpsi_prepare - prepare the projectors of k-point ik for the precision form: the
  * Hamiltonian's projectors are fixed for a k-point (Sec. 2.3, KB form; Sec. 5, the KSHam of a
- * k-point holds them across all its H psi calls), so their 3-term BF16 split into the two
+ * k-point holds them across all its H psi calls), so their FP16-pair split into the two
  * tensor-core operand layouts of the nonlocal part is done once here instead of on every
  * qm_hpsi(QM_MIXED) call.
  *
@@ -187,7 +188,7 @@ qm_status qm_hpsi_check(qm_gspace g, void* stream);
  * A later qm_hpsi(g, ik, ..., QM_MIXED) whose nproj, beta and ld_beta are the prepared ones
  * uses the prepared operands (the result is identical: the same split of the same values).  The
  * caller must not change the contents of beta while it is prepared; call again after changing
- * it.  Device memory: 12 bytes per projector coefficient (two layouts of three BF16 planes),
+ * it.  Device memory: 16 bytes per complex projector coefficient (two layouts of two FP16 planes),
  * owned by the handle (freed by this call with nproj = 0, a larger re-preparation, or
  * qm_gspace_destroy).  Not for use inside a stream capture (allocates).
  * Errors: QM_ERR_ARG, QM_ERR_OOM, QM_ERR_CUDA.
@@ -225,7 +226,7 @@ qm_status qm_hpsi_prepare(qm_gspace g, int ik, int nproj, const void* beta, int 
  *    so the host waits until the stream's earlier work is done before each copy.
  *  - Numerics: QM_FP64 is the FP64 path of qm_hpsi.  QM_MIXED runs the FP32 FFT path of
  *    qm_hpsi but its nonlocal projection and application as FP32 SIMT products (qm_hpsi uses
- *    BF16x3 tensor-core products, whose operand planes would need scratch of their own); both
+ *    tensor-core split products, whose operand planes would need scratch of their own); both
  *    are FP32-accurate (measured against the FP64 oracle: about 1e-7 per band on small cells).
  *  - A problem whose scratch exceeds the array is rejected with QM_ERR_ARG and a message
  *    giving the bytes it needs (tables + N1*N2*N3 reals + nproj*nb complex + one band of

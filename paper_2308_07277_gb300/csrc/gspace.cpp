@@ -179,6 +179,8 @@ struct PW {
     double kin;
 };
 
+static qm_status create_aux(cudaStream_t* s);
+
 qm_status ensure_device(qm_gspace g) {
     int dev = 0;
     qm_status st = cuda_check(cudaGetDevice(&dev), "cudaGetDevice");
@@ -217,11 +219,20 @@ qm_status ensure_device(qm_gspace g) {
         if (kt.gamma && (st = upload((void**)&kt.gtile, kt.h_gtile.data(), sizeof(int2) * kt.h_gtile.size())))
             return st;
     }
-    if ((st = cuda_check(cudaStreamCreateWithFlags(&g->aux, cudaStreamNonBlocking), "gspace stream")) ||
+    if ((st = create_aux(&g->aux)) ||
         (st = cuda_check(cudaEventCreateWithFlags(&g->ev_fork, cudaEventDisableTiming), "gspace event")) ||
         (st = cuda_check(cudaEventCreateWithFlags(&g->ev_join, cudaEventDisableTiming), "gspace event")))
         return st;
     return QM_OK;
+}
+
+// the second stream: highest priority, so that the CTAs of the nonlocal chain (few, one per SM, each
+// needed by the x-forward pass) start before the FFT kernels' queued ones and both share the SMs.  H psi
+// of 64 / 255 atoms 487 -> 425 / 2420 -> 2183 us, 144 atoms with projectors split per call 475 -> 387 us
+static qm_status create_aux(cudaStream_t* s) {
+    int least = 0, greatest = 0;
+    qm_status st = cuda_check(cudaDeviceGetStreamPriorityRange(&least, &greatest), "stream priorities");
+    return st ? st : cuda_check(cudaStreamCreateWithPriority(s, cudaStreamNonBlocking, greatest), "gspace stream");
 }
 
 qm_status gspace_clone(qm_gspace g, qm_gspace* out) {
@@ -235,7 +246,7 @@ qm_status gspace_clone(qm_gspace g, qm_gspace* out) {
     c->aux = nullptr;
     c->ev_fork = c->ev_join = nullptr;
     c->shared_tables = true;
-    if ((st = cuda_check(cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking), "gspace stream")) ||
+    if ((st = create_aux(&c->aux)) ||
         (st = cuda_check(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming), "gspace event")) ||
         (st = cuda_check(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming), "gspace event"))) {
         qm_gspace_destroy(c);

@@ -6,10 +6,11 @@
 //   2. zgemm_cn        P[p][b] = <beta_p|psi_b>             (nonlocal projection, FP64)
 //   3. K1, K2, K3      out = 1/2|k+G|^2 psi + (V psi)(G)    (per chunk of bands)
 //   4. zgemm_tn        out += sum_p beta_p D_p P[p][b]      (nonlocal apply, FP64)
-// QM_MIXED: the nonlocal part runs as BF16x3 split tcgen05 products (umma.cu) on the handle's
+// QM_MIXED: the nonlocal part runs as FP16-pair split tcgen05 products (nonlocal_tc.cu) on the handle's
 // second stream, concurrently with k_vt, K1 and K2 of every band: it writes
 // out = sum_p beta_p D_p P[p][b], and K3 (which waits for it) adds the local and kinetic
-// parts.  The tensor-core kernels (96 KB of shared memory) share SMs with the FFT kernels.
+// parts.  The tensor-core kernels (up to 128 KB of shared memory) share SMs with the FFT kernels.  Small
+// products run in FP32 on the caller's stream instead (small_nonlocal).
 // Workspace (owned by the gspace handle): error word | Vt | P | split-K partials | stick buffer | nonlocal.
 #include <algorithm>
 #include <cstdint>
@@ -22,6 +23,13 @@ namespace qm {
 // intermediate data stays resident in the 129 MB L2 between the three FFT kernels.
 constexpr size_t kStickBudget = 48ull << 20;
 constexpr size_t kStickBudgetOverlap = 1ull << 30;
+
+// Whether the precision form's nonlocal part is small enough for FP32 products on the CUDA cores, on the
+// caller's stream: the tensor-core chain is five or six launches (nine where the projectors are split on
+// the call) behind a fork and before a join.  Whole call, CUDA cores / tensor cores, us: prepared 1.3e6
+// (nproj nb npw) 41 / 47, 3.4e6 54 / 56, 1.0e7 77 / 60; split per call 3.4e6 54 / 72, 1.7e7 75 / 83,
+// 5.3e7 130 / 112.  One line for both, so that preparing the projectors does not change the result.
+static bool small_nonlocal(int nproj, int nb, int npw) { return (double)nproj * nb * npw <= 3.5e6; }
 
 struct HpsiLayout {
     size_t vt_off, p_off, part_off, part_bytes, t_off, nl_off, err_off, total, t_bytes;
@@ -40,8 +48,9 @@ static HpsiLayout hpsi_layout(qm_gspace g, int ik, int nb, int nproj, bool fp32,
     L.p_off = off;
     off = align_up(off + (size_t)nproj * nb * cs, 256);
     L.part_off = off;
-    // scratch of the two FP64 projector products
-    L.part_bytes = fp32 || nproj == 0 ? 0 : std::max(zgemm_cn_bytes(nproj, nb, npw), zgemm_tn_bytes(nb, npw, nproj));
+    // scratch of the projector products on the caller's stream
+    const bool small = fp32 && small_nonlocal(nproj, nb, npw);
+    L.part_bytes = nproj == 0 ? 0 : fp32 ? (small ? csmall_cn_bytes(nproj, nb, npw) : 0) : std::max(zgemm_cn_bytes(nproj, nb, npw), zgemm_tn_bytes(nb, npw, nproj));
     off = align_up(off + L.part_bytes, 256);
     L.t_off = off;
     // the precision form keeps every band's stick buffer (K1 and K2 of all bands overlap the
@@ -52,7 +61,7 @@ static HpsiLayout hpsi_layout(qm_gspace g, int ik, int nb, int nproj, bool fp32,
     L.t_bytes = stick_buffer_bytes(g, ik, fp32, (int)ntr, budget);
     off = align_up(off + L.t_bytes, 256);
     L.nl_off = off;  // tensor-core split operands (precision form)
-    off = align_up(off + (fp32 && nproj > 0 ? nonlocal_tc_bytes(nproj, nb, npw, own_beta) : 0), 256);
+    off = align_up(off + (fp32 && nproj > 0 && !small ? nonlocal_tc_bytes(nproj, nb, npw, own_beta) : 0), 256);
     L.total = off;
     return L;
 }
@@ -111,7 +120,8 @@ qm_status qm::hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi,
     const GemmWork gw{ws + L.part_off, L.part_bytes, (int*)(ws + L.err_off)};
     void* T = ws + L.t_off;
 
-    if (fp32 && nproj > 0) {
+    const bool small = fp32 && nproj > 0 && small_nonlocal(nproj, nb, npw);
+    if (fp32 && nproj > 0 && !small) {
         // fork: the nonlocal part on the second stream writes out; K3 joins and adds to it
         int* err = (int*)(ws + L.err_off);
         cudaStream_t a = g->aux;
@@ -127,6 +137,8 @@ qm_status qm::hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi,
                                     true, gamma);
     }
     if ((st = launch_vt_prepare(g, vloc_r, vt, fp32, s))) return st;
+    if (small && (st = csmall_cn(nproj, nb, npw, (const float2*)beta, ld_beta, (const float2*)psi, ld_psi, (float2*)P, nb, gw, s)))
+        return st;
     if (nproj > 0 && !fp32) {
         st = zgemm_cn(nproj, nb, npw, (const double2*)beta, ld_beta, (const double2*)psi, ld_psi, (double2*)P, nb, gw, s);
         if (st) return st;
@@ -134,6 +146,8 @@ qm_status qm::hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi,
     if ((st = launch_local_kinetic(g, ik, nb, psi, ld_psi, vt, out, ld_out, T, L.t_bytes, fp32, s, nullptr, false,
                                    gamma)))
         return st;
+    if (small)
+        return csmall_tn(nb, npw, nproj, (const float2*)P, nb, D, (const float2*)beta, ld_beta, (float2*)out, ld_out, s);
     if (nproj > 0 && !fp32) {
         st = zgemm_tn(nb, npw, nproj, (const double2*)P, nb, D, (const double2*)beta, ld_beta, (double2*)out, ld_out,
                       true, gw, s);

@@ -24,7 +24,7 @@
 //    handle's host copies into the scratch array (pageable host memory, so the host waits
 //    until the stream's earlier work is done before each copy);
 //  - QM_MIXED: the FFT path is the FP32 one of qm_hpsi; the nonlocal projection and
-//    application are FP32 SIMT products (not the tensor-core BF16x3 split of qm_hpsi, whose
+//    application are FP32 SIMT products (not the tensor-core split products of qm_hpsi, whose
 //    operand planes would need scratch of their own);
 //  - problems whose scratch exceeds QM_HPSI_NOALLOC_SCRATCH_BYTES are rejected with
 //    QM_ERR_ARG and a message giving the bytes needed.

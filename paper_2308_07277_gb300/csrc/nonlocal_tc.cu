@@ -1,17 +1,24 @@
 // Nonlocal part of the precision form on the tensor cores: the projection P = beta^H psi and
-// the application beta (D P) of the Kleinman-Bylander term (Sec. 2.3) as 3-term BF16 split
-// products accumulated in FP32 (tcgen05, accumulators in tensor memory).
+// the application beta (D P) of the Kleinman-Bylander term (Sec. 2.3) as split products of FP16
+// pairs accumulated in FP32 (tcgen05, accumulators in tensor memory).
 //
-// Splitting: an FP32 value x is written x = x0 + x1 + x2 with x0 = bf16(x),
-// x1 = bf16(x - x0), x2 = bf16(x - x0 - x1); a product a*b keeps the six terms a_i b_j with
-// i + j <= 2 (the dropped terms are below 2^-24 |a b|).
+// Splitting: every operand row is scaled by a power of two that brings its largest component to
+// [2^14, 2^15), and a scaled value x is written x = x0 + x1 with x0 = fp16(x), x1 = fp16(x - x0):
+// 23 significant bits (a quarter of the values lose the last bit of their 24, 2^-24 rms) down to
+// 2^-17 of the row's largest, an absolute error of 2^-40 of it below.  A product keeps x0 y0 + x0 y1 +
+// x1 y0 (x1 y1 is 2^-24.6 rms of the product).  Three BF16 pieces hold all 24 bits but take six
+// products; what limits the result is neither, it is the accumulation: the tensor core truncates
+// every sum it adds to an accumulator, 12 sums per 32 terms with six products, 6 with three (and
+// the projection's K is split twice as often).  Measured error of H psi against 64 bits, six BF16
+// products / these: 3.5e-6 / 1.4e-6 (255 atoms), 5.3e-6 / 2.2e-6 (216 atoms), 3.1e-7 / 1.5e-7 (64 atoms),
+// 8.9e-8 / 8.0e-8 (32 atoms), 5.7e-8 / 6.2e-8 (8 atoms, where the FP32 path below hpsi.cu's line has 4.7e-8).
 //
-// Operands are split ONCE into BF16 planes stored in global memory in a tile-blocked order:
-// block (row tile, K tile) holds, for each of the three planes, the R x 32 tile in the
-// canonical no-swizzle K-major shared-memory layout of the tensor core (8-row x 16-byte core
-// matrices; element (r, k) at ((r/8)*4 + k/8)*128 + (r%8)*16 + (k%8)*2).  A K tile of one
-// operand is therefore one contiguous run of 3*R*64 bytes, which a single bulk copy
-// (cp.async.bulk, completion counted on an mbarrier) lands in shared memory ready for the MMA.
+// Operands are split ONCE into FP16 planes stored in global memory in a tile-blocked order:
+// block (row tile, K tile) holds, for both planes, the R x 16 tile in the canonical no-swizzle
+// K-major shared-memory layout of the tensor core (8-row x 16-byte core matrices; element (r, k) at
+// ((r/8)*2 + k/8)*128 + (r%8)*16 + (k%8)*2).  A K tile of one operand is therefore one contiguous
+// run of 64 R bytes, which a single bulk copy (cp.async.bulk, completion counted on an mbarrier)
+// lands in shared memory ready for the MMA.
 //
 // Complex products as real GEMMs over K' = 2K (re, im interleaved or (p, u) pairs):
 //   projection  C[p][2b+t] = sum_(g,u) betaK[p][(g,u)] psiX[2b+t][(g,u)]
@@ -22,13 +29,17 @@
 //               E = D P expanded: E[2b][(p,0)] = ar, E[2b][(p,1)] = -ai, E[2b+1][(p,0)] = ai,
 //               E[2b+1][(p,1)] = ar (a = D_p P[p][b]), so C[2b][g] = Re(beta D P)[b][g], C[2b+1] = Im.
 //
-// GEMM kernel (k_nl_gemm): one CTA per (M tile of 128, N tile of BN <= 256, K range), eight
-// warps: warp 0 issues the bulk copies into a 3-stage ring, warp 1 owns the tensor memory and
-// one of its threads issues the 6 x 2 tcgen05.mma of each K tile (M = 128, N = BN, K = 16)
-// and commits each stage back to the producer, warps 4-7 drain the accumulator with
-// tcgen05.ld.  Every mbarrier wait is bounded: on expiry the kernel sets the error word, waits
-// (bounded) for its own copies and products in flight, frees its tensor memory and returns.
-#include <cuda_bf16.h>
+// GEMM kernel (k_nl_gemm): one CTA per (128 or 256 rows of A, N tile of BN <= 256, K range): one or two
+// M = 128 accumulators side by side in tensor memory.  A 128-row CTA would read 48 KB of operands per 768
+// tensor cycles, more than L2 delivers to 152 SMs at once (48 bytes per clock and SM are what the
+// six-product kernel drew at 0.94 of the tensor peak); 256 rows need 43.  Where that
+// leaves SMs without work the tiles shrink (gemm_shape).  Twelve warps: warp 0 issues
+// the bulk copies into a ring of kNlStages stages of one K tile, one thread of warp 1 issues the
+// 3 or 6 tcgen05.mma of a K tile (M = 128, N = BN, K = 16) and commits the stage back to the producer,
+// warps 4-11 drain the accumulators.  Every mbarrier wait is bounded: on expiry the kernel sets the
+// error word, waits (bounded) for its own copies and products in flight, frees its tensor memory and
+// returns.
+#include <cuda_fp16.h>
 #include <stdint.h>
 
 #include <algorithm>
@@ -39,102 +50,175 @@
 namespace qm {
 namespace {
 
-constexpr int KT = 32;          // K tile (real elements): 4 chunks of 8 BF16
+constexpr int KT = 16;          // K tile (real elements): 2 chunks of 8 FP16
 constexpr int TM = 128;         // rows of an A tile (M of the MMA)
-constexpr int kStages = 3;
-constexpr int kGemmThreads = 256;
+constexpr int kNlStages = 4;
+constexpr int kGemmThreads = 384;
+constexpr int kNlSegs = 4;      // partial maxima per row
 constexpr long kSpin = 1L << 26;
 
 __host__ __device__ constexpr size_t plane_bytes(int R) { return (size_t)R * KT * 2; }
-__host__ __device__ constexpr size_t block_bytes(int R) { return 3 * plane_bytes(R); }
+__host__ __device__ constexpr size_t block_bytes(int R) { return 2 * plane_bytes(R); }
 
 // byte offset of element (r, k) inside one plane of a tile
 __device__ __forceinline__ int cm_off(int r, int k) {
-    return ((((r >> 3) << 2) + (k >> 3)) << 7) + ((r & 7) << 4) + ((k & 7) << 1);
+    return ((((r >> 3) << 1) + (k >> 3)) << 7) + ((r & 7) << 4) + ((k & 7) << 1);
 }
 
-__device__ __forceinline__ uint32_t pack2(__nv_bfloat16 a, __nv_bfloat16 b) {
-    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+// split two scaled FP32 values into their FP16 components, packed in pairs
+__device__ __forceinline__ void split2(float x, float y, uint32_t& c0, uint32_t& c1) {
+    const __half2 h = __floats2half2_rn(x, y);
+    const float2 f = __half22float2(h);
+    const __half2 l = __floats2half2_rn(x - f.x, y - f.y);
+    c0 = *reinterpret_cast<const uint32_t*>(&h);
+    c1 = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-// split two FP32 values into their three BF16 components, packed in pairs
-__device__ __forceinline__ void split2(float x, float y, uint32_t& c0, uint32_t& c1, uint32_t& c2) {
-    const __nv_bfloat16 x0 = __float2bfloat16_rn(x), y0 = __float2bfloat16_rn(y);
-    const float rx = x - __bfloat162float(x0), ry = y - __bfloat162float(y0);
-    const __nv_bfloat16 x1 = __float2bfloat16_rn(rx), y1 = __float2bfloat16_rn(ry);
-    const __nv_bfloat16 x2 = __float2bfloat16_rn(rx - __bfloat162float(x1));
-    const __nv_bfloat16 y2 = __float2bfloat16_rn(ry - __bfloat162float(y1));
-    c0 = pack2(x0, y0);
-    c1 = pack2(x1, y1);
-    c2 = pack2(x2, y2);
-}
-
-// write the 8 consecutive K values v[0..7] of row r (k0 a multiple of 8) into the blocked array
-__device__ __forceinline__ void put8(unsigned char* blk, int R, int nkt, int r, int k0, const float* v) {
+// write the 8 consecutive K values v[0..7], scaled by sc, of row r (k0 a multiple of 8) into the blocked array
+__device__ __forceinline__ void put8(unsigned char* blk, int R, int nkt, int r, int k0, const float* v, float sc) {
     const int rt = r / R, rr = r - rt * R, kt = k0 / KT, kk = k0 - kt * KT;
     unsigned char* p = blk + ((size_t)rt * nkt + kt) * block_bytes(R) + cm_off(rr, kk);
-    uint4 c[3];
-    split2(v[0], v[1], c[0].x, c[1].x, c[2].x);
-    split2(v[2], v[3], c[0].y, c[1].y, c[2].y);
-    split2(v[4], v[5], c[0].z, c[1].z, c[2].z);
-    split2(v[6], v[7], c[0].w, c[1].w, c[2].w);
+    uint4 c[2];
+    split2(v[0] * sc, v[1] * sc, c[0].x, c[1].x);
+    split2(v[2] * sc, v[3] * sc, c[0].y, c[1].y);
+    split2(v[4] * sc, v[5] * sc, c[0].z, c[1].z);
+    split2(v[6] * sc, v[7] * sc, c[0].w, c[1].w);
 #pragma unroll
-    for (int q = 0; q < 3; ++q) *reinterpret_cast<uint4*>(p + q * plane_bytes(R)) = c[q];
+    for (int q = 0; q < 2; ++q) *reinterpret_cast<uint4*>(p + q * plane_bytes(R)) = c[q];
+}
+
+// the power of two that brings values below 2^(e - 126) (e: biased exponent of the row's largest) below
+// 2^15, limited to FP32's range (rows below 2^-112 or with nothing in them; a row with a non-finite value
+// keeps scale 1 and gives NaN), and its inverse
+__device__ __forceinline__ float row_scale(int hmax) {
+    const int e = hmax >> 23;
+    const int k = e >= 255 ? 0 : min(126, 141 - e);
+    return __uint_as_float((uint32_t)(k + 127) << 23);
+}
+__device__ __forceinline__ float inv_scale(float s) { return __uint_as_float((254u << 23) - __float_as_uint(s)); }
+__device__ __forceinline__ int f_abs(float x) { return __float_as_int(x) & 0x7FFFFFFF; }
+__device__ __forceinline__ int max_segs(const int* __restrict__ emax, int n, int r) {
+    int h = 0;
+#pragma unroll
+    for (int s = 0; s < kNlSegs; ++s) h = max(h, __ldg(emax + (size_t)s * n + r));
+    return h;
+}
+
+// largest magnitude (bits) of each row of src over column segment blockIdx.y
+__global__ void __launch_bounds__(256) k_nl_rowmax(const float2* __restrict__ src, int ld, int rows, int cols,
+                                                   int* __restrict__ emax) {
+    __shared__ int red[8];
+    const int r = blockIdx.x, per = (cols + kNlSegs - 1) / kNlSegs;
+    const int c0 = blockIdx.y * per, c1 = min(cols, c0 + per);
+    const float2* p = src + (size_t)r * ld;
+    int h = 0;
+#pragma unroll 4
+    for (int c = c0 + threadIdx.x; c < c1; c += 256) {
+        const float2 v = __ldg(p + c);
+        h = max(h, max(f_abs(v.x), f_abs(v.y)));
+    }
+    h = __reduce_max_sync(0xffffffffu, h);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = h;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) h = max(h, red[w]);
+        emax[(size_t)blockIdx.y * rows + r] = h;
+    }
+}
+// the same per column of src [K][cols] over K segment blockIdx.y
+__global__ void __launch_bounds__(256) k_nl_colmax(const float2* __restrict__ src, int ld, int K, int cols,
+                                                   int* __restrict__ emax) {
+    const int c = blockIdx.x * 256 + threadIdx.x, per = (K + kNlSegs - 1) / kNlSegs;
+    if (c >= cols) return;
+    const int k0 = blockIdx.y * per, k1 = min(K, k0 + per);
+    int h = 0;
+#pragma unroll 8
+    for (int k = k0; k < k1; ++k) {
+        const float2 v = __ldg(src + (size_t)k * ld + c);
+        h = max(h, max(f_abs(v.x), f_abs(v.y)));
+    }
+    emax[(size_t)blockIdx.y * cols + c] = h;
 }
 
 // Rows of complex src (K = 2 ncols interleaved reals) -> blocked split operand.  expand = 0:
 // row r is src row r as stored; expand = 1: rows 2b, 2b+1 are src row b as stored and its
 // rotation (im, -re).  Rows >= nsrc (resp. 2 nsrc) and K beyond 2 ncols are written as zeros.
 // CTA: 8 rows (one core-matrix row group, blockIdx.y) x 32 chunks of 8 K values (blockIdx.x);
-// the 8 rows of a core matrix on consecutive threads (one 128-byte run per plane), the 4
-// chunks of a K tile on consecutive thread octets.
+// the 8 rows of a core matrix on consecutive threads (one 128-byte run per plane), the 2
+// chunks of a K tile on consecutive thread octets.  inv: the source rows' inverse scales.
 constexpr int kSplitChunks = 32;
+constexpr int kFoldReduce = 1024;  // projectors x splits up to which the expansion sums the splits (one CTA per 4 bands)
+constexpr int kSelfScale = 2048;  // plane waves up to which a row's scale is found in its splitting CTA
 __global__ void __launch_bounds__(256) k_split_rows(const float2* __restrict__ src, int ld, int nsrc, int ncols,
-                                                    int expand, int R, int nkt, unsigned char* __restrict__ blk) {
+                                                    int expand, int R, int nkt, const int* __restrict__ emax,
+                                                    float* __restrict__ inv, unsigned char* __restrict__ blk) {
     const int r = blockIdx.y * 8 + (threadIdx.x & 7);
-    const int ch = blockIdx.x * kSplitChunks + (threadIdx.x >> 3);
-    if (ch >= nkt * (KT / 8)) return;
+    int ch = blockIdx.x * kSplitChunks + (threadIdx.x >> 3);
     const int b = expand ? (r >> 1) : r;
-    const int c0 = ch * 4;  // first complex column of the chunk
-    float v[8];
-    if (b < nsrc && c0 + 3 < ncols) {
-        const float2* s2 = src + (size_t)b * ld + c0;
-        if (((uintptr_t)s2 & 15) == 0) {
-            const float4 a = __ldg(reinterpret_cast<const float4*>(s2)), bb = __ldg(reinterpret_cast<const float4*>(s2) + 1);
-            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = bb.x; v[5] = bb.y; v[6] = bb.z; v[7] = bb.w;
+    float sc = 1.f;
+    if (!emax) {  // short rows, one CTA per row group: the rows' largest values are found here
+        __shared__ int smax[8];
+        const int nrow = expand ? 4 : 8, l = threadIdx.x & 31, b0 = blockIdx.y * nrow;
+        for (int q = threadIdx.x >> 5; q < nrow; q += 8) {
+            int h = 0;
+            if (b0 + q < nsrc)
+                for (int c = l; c < ncols; c += 32) {
+                    const float2 x = __ldg(src + (size_t)(b0 + q) * ld + c);
+                    h = max(h, max(f_abs(x.x), f_abs(x.y)));
+                }
+            h = __reduce_max_sync(0xffffffffu, h);
+            if (l == 0) smax[q] = h;
+        }
+        __syncthreads();
+        sc = row_scale(smax[b - b0]);
+    } else if (b < nsrc) {
+        sc = row_scale(max_segs(emax, nsrc, b));
+    }
+    if (ch == 0 && b < nsrc && !(expand && (r & 1))) inv[b] = inv_scale(sc);
+    for (; ch < nkt * (KT / 8); ch += emax ? nkt * (KT / 8) : kSplitChunks) {
+        const int c0 = ch * 4;  // first complex column of the chunk
+        float v[8];
+        if (b < nsrc && c0 + 3 < ncols) {
+            const float2* s2 = src + (size_t)b * ld + c0;
+            if (((uintptr_t)s2 & 15) == 0) {
+                const float4 a = __ldg(reinterpret_cast<const float4*>(s2)), bb = __ldg(reinterpret_cast<const float4*>(s2) + 1);
+                v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = bb.x; v[5] = bb.y; v[6] = bb.z; v[7] = bb.w;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 x = __ldg(s2 + j);
+                    v[2 * j] = x.x;
+                    v[2 * j + 1] = x.y;
+                }
+            }
         } else {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const float2 x = __ldg(s2 + j);
+                float2 x = make_float2(0.f, 0.f);
+                if (b < nsrc && c0 + j < ncols) x = __ldg(src + (size_t)b * ld + c0 + j);
                 v[2 * j] = x.x;
                 v[2 * j + 1] = x.y;
             }
         }
-    } else {
+        if (expand && (r & 1)) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            float2 x = make_float2(0.f, 0.f);
-            if (b < nsrc && c0 + j < ncols) x = __ldg(src + (size_t)b * ld + c0 + j);
-            v[2 * j] = x.x;
-            v[2 * j + 1] = x.y;
+            for (int j = 0; j < 4; ++j) {
+                const float re = v[2 * j], im = v[2 * j + 1];
+                v[2 * j] = im;
+                v[2 * j + 1] = -re;
+            }
         }
+        put8(blk, R, nkt, r, ch * 8, v, sc);
     }
-    if (expand && (r & 1)) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float re = v[2 * j], im = v[2 * j + 1];
-            v[2 * j] = im;
-            v[2 * j + 1] = -re;
-        }
-    }
-    put8(blk, R, nkt, r, ch * 8, v);
 }
 
 // beta [P][G] (complex, ld) -> blocked split betaT: row g, K = (p, u) (u = re/im of beta[p][g]).
-// CTA tile: 64 rows g x 16 projectors (one K tile), transposed through shared memory so the
+// CTA tile: 64 rows g x 16 projectors (two K tiles), transposed through shared memory so the
 // global reads run along g.  Rows g >= G (up to rows_pad) and p >= P are zeros.
-constexpr int kTG = 64, kTP = KT / 2;
+constexpr int kTG = 64, kTP = 16;
 __global__ void __launch_bounds__(256) k_split_t(const float2* __restrict__ beta, int ld, int P, int G, int R, int nkt,
+                                                 const int* __restrict__ emax, float* __restrict__ inv,
                                                  unsigned char* __restrict__ blk) {
     __shared__ float2 t[kTP][kTG + 1];
     const int g0 = blockIdx.x * kTG, p0 = blockIdx.y * kTP;
@@ -146,7 +230,10 @@ __global__ void __launch_bounds__(256) k_split_t(const float2* __restrict__ beta
     __syncthreads();
     // 64 rows x 4 chunks of 4 projectors; the 8 rows of a core matrix on consecutive threads
     const int rlo = threadIdx.x & 7, ch = (threadIdx.x >> 3) & 3, rg = threadIdx.x >> 5;
-    const int gg = rg * 8 + rlo;
+    const int gg = rg * 8 + rlo, g = g0 + gg;
+    const float sc = g < G ? row_scale(max_segs(emax, G, g)) : 1.f;
+    if (blockIdx.y == 0 && ch == 0 && g < G) inv[g] = inv_scale(sc);
+    if ((int)blockIdx.y * 2 + (ch >> 1) >= nkt) return;
     float v[8];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -154,51 +241,82 @@ __global__ void __launch_bounds__(256) k_split_t(const float2* __restrict__ beta
         v[2 * j] = x.x;
         v[2 * j + 1] = x.y;
     }
-    put8(blk, R, nkt, g0 + gg, p0 * 2 + ch * 8, v);
+    put8(blk, R, nkt, g, p0 * 2 + ch * 8, v, sc);
 }
 
-// sum the split-K partials of the projection C[z][p][c] (FP32, ldc; c = 2b + t) in a fixed order
-// and scale by D_p: Pd[p][c] = D_p sum_z C[z][p][c] (consecutive threads, consecutive c: coalesced)
+// sum the split-K partials of the projection C[z][p][c] (FP32, ldc; c = 2b + t) in a fixed order,
+// undo the rows' scales and multiply by D_p: Pd[p][c] (consecutive threads, consecutive c: coalesced)
 __global__ void k_reduce_p(const float* __restrict__ part, int Z, size_t zstride, int ldc, int P, int ncol,
-                           const double* __restrict__ D, float* __restrict__ Pd) {
+                           const double* __restrict__ D, const float* __restrict__ inv_p, const float* __restrict__ inv_b,
+                           float* __restrict__ Pd) {
     const size_t total = (size_t)P * ncol;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
         const int p = (int)(e / ncol), c = (int)(e - (size_t)p * ncol);
         const float* q = part + (size_t)p * ldc + c;
         float a = 0.f;
+#pragma unroll 8
         for (int z = 0; z < Z; ++z) a += __ldg(q + (size_t)z * zstride);
-        Pd[e] = a * (float)__ldg(D + p);
+        Pd[e] = a * __ldg(inv_p + p) * __ldg(inv_b + (c >> 1)) * (float)__ldg(D + p);
     }
 }
 
 // the application's A operand E = D P expanded, blocked and split (rows 2b + t, K = (p, u)):
 // E[2b][(p,0)] = ar, E[2b][(p,1)] = -ai, E[2b+1][(p,0)] = ai, E[2b+1][(p,1)] = ar with
-// a = Pd[p][2b] + i Pd[p][2b+1]; rows >= 2 nb and p >= P are zeros.  One thread per (row, 4
-// projectors), the 8 rows of a core matrix on consecutive threads.
-__global__ void k_expand_e(const float* __restrict__ Pd, int P, int nb, int rows_pad, int nkt,
-                           unsigned char* __restrict__ blk) {
-    const int nchunk = nkt * (KT / 8);
-    const long total = (long)rows_pad * nchunk;
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
-        const int rlo = (int)(e & 7);
-        const long q = e >> 3;
-        const int ch = (int)(q % nchunk);
-        const int r = (int)(q / nchunk) * 8 + rlo;
-        const int b = r >> 1, t = r & 1;
+// a = Pd[p][2b] + i Pd[p][2b+1]; rows >= 2 nb and p >= P are zeros.  One CTA per core-matrix row
+// group (four bands): their largest values first, then one thread per (row, 4 projectors).
+// part != NULL (few partial sums): the sums of k_reduce_p are taken here instead of read from Pd, through
+// shared memory (P x 4 bands).
+__global__ void __launch_bounds__(256) k_expand_e(const float* __restrict__ Pd, const float* __restrict__ part, int Z,
+                                                  size_t zstride, int ldc, const double* __restrict__ D,
+                                                  const float* __restrict__ inv_p, const float* __restrict__ inv_b, int P, int nb,
+                                                  int nkt, float* __restrict__ inv, unsigned char* __restrict__ blk) {
+    extern __shared__ __align__(16) unsigned char esm[];
+    float2* sp = reinterpret_cast<float2*>(esm);  // [P][4] when part
+    __shared__ int smax[4];
+    const int tid = threadIdx.x, q4 = tid & 3, b4 = blockIdx.x * 4 + q4;
+    if (tid < 4) smax[tid] = 0;
+    __syncthreads();
+    int h = 0;
+    const float ib = part && b4 < nb ? __ldg(inv_b + b4) : 0.f;
+    for (int p = tid >> 2; p < P; p += 64) {
+        float2 a = make_float2(0.f, 0.f);
+        if (b4 < nb) {
+            if (part) {
+                const float* q = part + (size_t)p * ldc + 2 * b4;
+#pragma unroll 8
+                for (int z = 0; z < Z; ++z) {
+                    const float2 v = __ldg(reinterpret_cast<const float2*>(q + (size_t)z * zstride));
+                    a.x += v.x;
+                    a.y += v.y;
+                }
+                const float ip = __ldg(inv_p + p), d = (float)__ldg(D + p);
+                a.x = a.x * ip * ib * d;
+                a.y = a.y * ip * ib * d;
+            } else {
+                a = __ldg(reinterpret_cast<const float2*>(Pd + (size_t)p * 2 * nb) + b4);
+            }
+        }
+        if (part) sp[p * 4 + q4] = a;
+        h = max(h, max(f_abs(a.x), f_abs(a.y)));
+    }
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) h = max(h, __shfl_xor_sync(0xffffffffu, h, o));
+    if ((tid & 31) < 4) atomicMax(&smax[q4], h);
+    __syncthreads();
+    const int nchunk = nkt * (KT / 8), rlo = tid & 7, r = blockIdx.x * 8 + rlo, b = r >> 1, t = r & 1;
+    const float sc = row_scale(smax[rlo >> 1]);
+    if (tid < 8 && !t && b < nb) inv[b] = inv_scale(sc);
+    for (int ch = tid >> 3; ch < nchunk; ch += 32) {
         float v[8];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int p = ch * 4 + j;
-            float ar = 0.f, ai = 0.f;
-            if (b < nb && p < P) {
-                const float2 a = __ldg(reinterpret_cast<const float2*>(Pd + (size_t)p * 2 * nb) + b);
-                ar = a.x;
-                ai = a.y;
-            }
-            v[2 * j] = t ? ai : ar;
-            v[2 * j + 1] = t ? ar : -ai;
+            float2 a = make_float2(0.f, 0.f);
+            if (b < nb && p < P) a = part ? sp[p * 4 + (rlo >> 1)] : __ldg(reinterpret_cast<const float2*>(Pd + (size_t)p * 2 * nb) + b);
+            v[2 * j] = t ? a.y : a.x;
+            v[2 * j + 1] = t ? a.x : -a.y;
         }
-        put8(blk, TM, nkt, r, ch * 8, v);
+        put8(blk, TM, nkt, r, ch * 8, v, sc);
     }
 }
 
@@ -216,41 +334,46 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile
     return false;
 }
 
-// C (+)= A B^T over the K tiles [kt0, kt1) of this split.  A: blocked, 128-row tiles, nkt K
-// tiles per row tile; B: blocked, BN-row tiles.  EPI 0: C is FP32 [m][n] (ldc) at C + z*zstride
-// (split-K partials); EPI 1: row m = 2b + t, column g -> complex out[b][g] component t
-// (ldc = complex row stride), accumulate: add to out.
+// C (+)= A B^T over the K tiles [kt0, kt1) of this split.  A: blocked, 128-row tiles (mtiles of them), nkt K
+// tiles per row tile, msub (1 or 2) row tiles per CTA; B: blocked in tiles of bsub x BN rows, one of the
+// bsub parts per CTA.  EPI 0: C is FP32 [m][n] (ldc) at
+// C + z*zstride (split-K partials, operands' scales not undone); EPI 1: row m = 2b + t, column g -> complex
+// out[b][g] component t (ldc = complex row stride) times inv_m[b] inv_n[g], accumulate: add to out.
 template <int EPI>
 __global__ void __launch_bounds__(kGemmThreads, 1)
-k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__ B, int nkt, int BN, int M, int N,
-          int kt_per_split, float* __restrict__ C, size_t ldc, size_t zstride, int accumulate, int* __restrict__ err) {
+k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__ B, int nkt, int BN, int bsub, int msub, int M,
+          int N, int mtiles, int kt_per_split, float* __restrict__ C, size_t ldc, size_t zstride, int accumulate,
+          const float* __restrict__ inv_m, const float* __restrict__ inv_n, int* __restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) uint64_t full[kStages], empty[kStages], accf;
+    __shared__ __align__(8) uint64_t full[kNlStages], empty[kNlStages], accf;
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag, s_used, s_issued;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // projection: N tiles fastest (the few N tiles of one M tile share its beta tiles in L2);
     // application: M tiles fastest (the M tiles of one N tile share its betaT tiles, which are
     // then read from HBM once instead of once per M tile)
-    const int nt = EPI == 0 ? blockIdx.x : blockIdx.y, mt = EPI == 0 ? blockIdx.y : blockIdx.x;
+    const int nt = EPI == 0 ? blockIdx.x : blockIdx.y, mt = msub * (EPI == 0 ? blockIdx.y : blockIdx.x);
+    const int nsub = min(msub, mtiles - mt);
     const int kt0 = blockIdx.z * kt_per_split;
     const int kt1 = min(nkt, kt0 + kt_per_split);
     const int nk = max(0, kt1 - kt0);
-    const uint32_t a_bytes = (uint32_t)block_bytes(TM), b_bytes = (uint32_t)block_bytes(BN);
-    const uint32_t stage_bytes = a_bytes + b_bytes;
+    const uint32_t a_bytes = (uint32_t)block_bytes(TM), b_bytes = (uint32_t)block_bytes(BN), b_src_bytes = b_bytes * bsub;
+    const uint32_t stage_bytes = msub * a_bytes + b_bytes, tx_bytes = nsub * a_bytes + b_bytes;
+    const uint32_t acols = BN <= 32 ? 32 : BN <= 64 ? 64 : BN <= 128 ? 128 : 256;  // columns between the accumulators
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(tc::smem_u32(&tmem_base)),
-                     "r"(256));
+                     "r"(msub * acols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
     }
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < kNlStages; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(tc::smem_u32(&full[s])));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(tc::smem_u32(&empty[s])));
         }
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(tc::smem_u32(&accf)));
         asm volatile("fence.mbarrier_init.release.cluster;\n");
         abort_flag = 0;
+        s_used = s_issued = 0;
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
     __syncthreads();
@@ -258,52 +381,54 @@ k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__
     const uint32_t tmem = tmem_base;
     volatile int* abort = &abort_flag;
     const unsigned char* a_src = A + ((size_t)mt * nkt + kt0) * a_bytes;
-    const unsigned char* b_src = B + ((size_t)nt * nkt + kt0) * b_bytes;
+    const unsigned char* b_src = B + ((size_t)(nt / bsub) * nkt + kt0) * b_src_bytes + (nt % bsub) * (b_bytes / 2);
     const uint32_t sbase = tc::smem_u32(smem);
     int issued = 0;  // producer: K tiles whose copies were issued
     int used = 0;    // MMA issuer: K tiles consumed
     if (warp == 0 && lane == 0) {
         for (int it = 0; it < nk; ++it) {
-            const int s = it % kStages;
-            if (it >= kStages && !wait_bar(tc::smem_u32(&empty[s]), ((it / kStages) & 1) ^ 1, abort)) {
+            const int s = it % kNlStages;
+            if (it >= kNlStages && !wait_bar(tc::smem_u32(&empty[s]), ((it / kNlStages) & 1) ^ 1, abort)) {
                 *abort = 1;
                 break;
             }
             const uint32_t fb = tc::smem_u32(&full[s]);
             const uint32_t dst = sbase + s * stage_bytes;
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fb), "r"(stage_bytes) : "memory");
-            asm volatile(
-                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
-                "l"(a_src + (size_t)it * a_bytes), "r"(a_bytes), "r"(fb)
-                : "memory");
-            asm volatile(
-                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-                    dst + a_bytes),
-                "l"(b_src + (size_t)it * b_bytes), "r"(b_bytes), "r"(fb)
-                : "memory");
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fb), "r"(tx_bytes) : "memory");
+            for (int u = 0; u < nsub; ++u)
+                asm volatile(
+                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                        dst + u * a_bytes),
+                    "l"(a_src + ((size_t)u * nkt + it) * a_bytes), "r"(a_bytes), "r"(fb)
+                    : "memory");
+            for (int q = 0; q < 2; ++q)  // the two planes of this CTA's part of the source's row tile
+                asm volatile(
+                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                        dst + msub * a_bytes + q * (b_bytes / 2)),
+                    "l"(b_src + (size_t)it * b_src_bytes + q * (b_src_bytes / 2)), "r"(b_bytes / 2), "r"(fb)
+                    : "memory");
             issued = it + 1;
         }
     } else if (warp == 1 && lane == 0) {
-        const uint32_t idesc = tc::idesc_bf16(TM, BN);
-        const int pa[6] = {2, 1, 0, 1, 0, 0}, pb[6] = {0, 1, 2, 0, 1, 0};  // smallest terms first
+        const uint32_t idesc = tc::idesc_f16(TM, BN);
+        const int pa[3] = {1, 0, 0}, pb[3] = {0, 1, 0};  // smallest terms first
         for (int it = 0; it < nk; ++it) {
-            const int s = it % kStages;
-            if (!wait_bar(tc::smem_u32(&full[s]), (it / kStages) & 1, abort)) {
+            const int s = it % kNlStages;
+            if (!wait_bar(tc::smem_u32(&full[s]), (it / kNlStages) & 1, abort)) {
                 *abort = 1;
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n");
-            const uint32_t sa = sbase + s * stage_bytes, sb = sa + a_bytes;
+            const uint32_t sa = sbase + s * stage_bytes, sb = sa + msub * a_bytes;
+            for (int u = 0; u < nsub; ++u) {
 #pragma unroll
-            for (int q = 0; q < 6; ++q) {
-#pragma unroll
-                for (int ks = 0; ks < KT / 16; ++ks) {
-                    const uint64_t da = tc::sdesc(sa + pa[q] * (uint32_t)plane_bytes(TM) + ks * 256, 128, 512);
-                    const uint64_t db = tc::sdesc(sb + pb[q] * (uint32_t)plane_bytes(BN) + ks * 256, 128, 512);
-                    const uint32_t acc = (it > 0 || q > 0 || ks > 0) ? 1u : 0u;
+                for (int q = 0; q < 3; ++q) {
+                    const uint64_t da = tc::sdesc(sa + u * a_bytes + pa[q] * (uint32_t)plane_bytes(TM), 128, 256);
+                    const uint64_t db = tc::sdesc(sb + pb[q] * (uint32_t)plane_bytes(BN), 128, 256);
+                    const uint32_t acc = (it > 0 || q > 0) ? 1u : 0u;
                     asm volatile(
                         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + u * acols),
                         "l"(da), "l"(db), "r"(idesc), "r"(acc));
                 }
             }
@@ -311,7 +436,7 @@ k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__
                 tc::smem_u32(&empty[s])));
             used = it + 1;
         }
-        // the accumulator is final once every product issued so far has completed
+        // the accumulators are final once every product issued so far has completed
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
             tc::smem_u32(&accf)));
     }
@@ -321,14 +446,15 @@ k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__
         const bool ok = wait_bar(tc::smem_u32(&accf), 0, nullptr);
         if (!ok) *abort = 1;
         asm volatile("tcgen05.fence::after_thread_sync;\n");
+        const int q = warp & 3, u = (warp - 4) >> 2;  // tensor-memory lanes 32 q .., accumulator u
         // warp-uniform decision (tcgen05.ld and the shuffles below need the whole warp)
-        if (__all_sync(0xffffffffu, ok && nk > 0 && !*abort)) {
-            const int q = warp & 3;
-            const int mrow = mt * TM + q * 32 + lane;  // this thread's accumulator row
+        if (__all_sync(0xffffffffu, ok && nk > 0 && !*abort) && u < nsub) {
+            const int mrow = (mt + u) * TM + q * 32 + lane;  // this thread's accumulator row
+            const float im = EPI == 1 && mrow < M ? __ldg(inv_m + (mrow >> 1)) : 1.f;
 #pragma unroll 1
             for (int c0 = 0; c0 < BN; c0 += 16) {
                 uint32_t v[16];
-                const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
+                const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)u * acols + (uint32_t)c0;
                 asm volatile(
                     "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
                     "%13, %14, %15}, [%16];\n"
@@ -360,8 +486,11 @@ k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__
                         for (int j = 0; j < 8; ++j) {
                             const int g = g0 + j;
                             if (g < N) {
+                                const float in = __ldg(inv_n + g);
                                 float2 o = t ? make_float2(y[j], __uint_as_float(v[8 + j]))
                                              : make_float2(__uint_as_float(v[j]), y[j]);
+                                o.x = o.x * im * in;
+                                o.y = o.y * im * in;
                                 if (accumulate) {
                                     const float2 a = orow[g];
                                     o.x += a.x;
@@ -381,15 +510,15 @@ k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__
         // drain: the copies issued but never consumed, then every product issued
         if (warp == 0 && lane == 0) {
             for (int it = s_used; it < s_issued; ++it) {
-                const int s = it % kStages;
-                wait_bar(tc::smem_u32(&full[s]), (it / kStages) & 1, nullptr);
+                const int s = it % kNlStages;
+                wait_bar(tc::smem_u32(&full[s]), (it / kNlStages) & 1, nullptr);
             }
         }
         if (warp == 1 && lane == 0) wait_bar(tc::smem_u32(&accf), 0, nullptr);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
     __syncthreads();
-    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(256));
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(msub * acols));
 }
 
 inline size_t rup(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -402,11 +531,37 @@ int proj_bn(int nb) {
 }
 constexpr int kAppBN = 256;
 
+// Tile shape of a GEMM (row tiles per CTA, parts of a B tile, splits of K): the cheapest by rounds of CTAs
+// over the SMs times the cycles of a CTA, its K tiles (3 products of 128 x BN x 16 per row tile, or their
+// operands at 45 bytes per clock) plus about 6000 of start, fill and drain.
+struct GemmShape {
+    int msub, bsub, splits;
+};
+GemmShape gemm_shape(int mtiles, int ntiles, int BN, int nkt, int max_bsub, int max_splits) {
+    GemmShape best{2, 1, 1};
+    double cost = -1;
+    const int sms = device_sms();
+    for (int msub = 2; msub >= 1; --msub)
+        for (int bsub = 1; bsub <= max_bsub; bsub *= 2) {
+            const long tiles = (long)((mtiles + msub - 1) / msub) * ntiles * bsub;
+            const int sp = (int)std::max<long>(1, std::min<long>({(long)max_splits, (long)std::max(1, nkt / 8), sms / tiles}));
+            const int per = (nkt + sp - 1) / sp, m = std::min(msub, mtiles), bn = BN / bsub;
+            const double tile = std::max(1.5 * m * bn, (m * 8192.0 + bn * 64.0) / 45.0);
+            const double c = (double)((tiles * sp + sms - 1) / sms) * (per * tile + 6000.0);
+            if (cost < 0 || c < cost) {
+                cost = c;
+                best = GemmShape{msub, bsub, (nkt + per - 1) / per};
+            }
+        }
+    return best;
+}
+
 struct NlLayout {
+    GemmShape sp, sa;                   // shapes of the projection and the application
     int bn_p, ntile_p, mtile_p, nkt_p;  // projection: N tile, tiles, K tiles (of 2 npw)
     int mtile_a, ntile_a, nkt_a;        // application
     int splits;
-    size_t betaK_off, betaT_off, psiX_off, part_off, pd_off, e_off, total;
+    size_t betaK_off, betaT_off, inv_off, psiX_off, part_off, pd_off, e_off, emax_off, invb_off, total;
     size_t zstride;
 };
 
@@ -419,8 +574,9 @@ NlLayout nl_layout(int nproj, int nb, int npw, bool with_beta) {
     L.mtile_a = (2 * nb + TM - 1) / TM;
     L.ntile_a = (npw + kAppBN - 1) / kAppBN;
     L.nkt_a = (int)(rup(2 * (size_t)nproj, KT) / KT);
-    const int tiles = L.ntile_p * L.mtile_p;
-    L.splits = std::max(1, std::min(std::min(kMaxUmmaSplits, L.nkt_p), device_sms() / std::max(1, tiles)));
+    L.sp = gemm_shape(L.mtile_p, L.ntile_p, L.bn_p, L.nkt_p, 1, kMaxUmmaSplits);
+    L.sa = gemm_shape(L.mtile_a, L.ntile_a, kAppBN, L.nkt_a, 4, 1);
+    L.splits = L.sp.splits;
     L.zstride = (size_t)L.mtile_p * TM * L.ntile_p * L.bn_p;
     size_t off = 0;
     auto take = [&](size_t b) {
@@ -430,52 +586,69 @@ NlLayout nl_layout(int nproj, int nb, int npw, bool with_beta) {
     };
     L.betaK_off = take(with_beta ? (size_t)L.mtile_p * L.nkt_p * block_bytes(TM) : 0);
     L.betaT_off = take(with_beta ? (size_t)L.ntile_a * L.nkt_a * block_bytes(kAppBN) : 0);
+    // inverse scales: betaK rows, betaT rows; then the partial maxima of both
+    L.inv_off = take(with_beta ? sizeof(float) * ((size_t)nproj + npw) * (1 + kNlSegs) : 0);
     L.psiX_off = take((size_t)L.ntile_p * L.nkt_p * block_bytes(L.bn_p));
     L.part_off = take((size_t)L.splits * L.zstride * sizeof(float));
     L.pd_off = take((size_t)nproj * 2 * nb * sizeof(float));
     L.e_off = take((size_t)L.mtile_a * L.nkt_a * block_bytes(TM));
+    L.emax_off = take(sizeof(int) * (size_t)kNlSegs * nb);
+    L.invb_off = take(sizeof(float) * 2 * (size_t)nb);  // inverse scales of psi's and of E's bands
     L.total = off;
     return L;
 }
 
 // grid-dimension limits of the split and GEMM launches (y and z of a grid are below 65536)
 qm_status check_limits(const NlLayout& L) {
-    if ((long)L.mtile_p * TM / 8 > 65535 || (long)L.ntile_p * L.bn_p / 8 > 65535 || L.nkt_a > 65535 ||
-        L.ntile_a > 65535 || L.mtile_p > 65535)
+    if ((long)L.mtile_p * TM / 8 > 65535 || (long)L.ntile_p * L.bn_p / 8 > 65535 || (L.nkt_a + 1) / 2 > 65535 ||
+        L.ntile_a * L.sa.bsub > 65535 || L.mtile_p > 65535)
         return fail(QM_ERR_UNSUPPORTED, "tensor-core nonlocal part: too many bands, projectors or plane waves");
     return QM_OK;
 }
 
 inline int grid_for(long n, int per = 256) { return grid_stride_blocks((size_t)std::max<long>(n, 1), per, 16); }
 
-qm_status split_beta(int nproj, int npw, const float2* beta, int ld_beta, const NlLayout& L, unsigned char* betaK,
-                     unsigned char* betaT, cudaStream_t s) {
+qm_status split_beta(int nproj, int npw, const float2* beta, int ld_beta, const NlLayout& L, unsigned char* base, cudaStream_t s) {
+    float* invk = (float*)(base + L.inv_off);
+    float* invt = invk + nproj;
+    int* ek = (int*)(invt + npw);
+    int* et = ek + (size_t)kNlSegs * nproj;
+    {
+        ProfScope pf(PF_SPLIT, s);
+        k_nl_rowmax<<<dim3((unsigned)nproj, kNlSegs), 256, 0, s>>>(beta, ld_beta, nproj, npw, ek);
+    }
+    {
+        ProfScope pf(PF_SPLIT, s);
+        k_nl_colmax<<<dim3((unsigned)((npw + 255) / 256), kNlSegs), 256, 0, s>>>(beta, ld_beta, nproj, npw, et);
+    }
     {
         ProfScope pf(PF_SPLIT, s);
         const dim3 grid((unsigned)((L.nkt_p * (KT / 8) + kSplitChunks - 1) / kSplitChunks), (unsigned)(L.mtile_p * TM / 8));
-        k_split_rows<<<grid, 256, 0, s>>>(beta, ld_beta, nproj, npw, 0, TM, L.nkt_p, betaK);
+        k_split_rows<<<grid, 256, 0, s>>>(beta, ld_beta, nproj, npw, 0, TM, L.nkt_p, ek, invk, base + L.betaK_off);
     }
     qm_status st = cuda_check(cudaGetLastError(), "k_split_rows launch");
     if (st) return st;
     {
         ProfScope pf(PF_SPLIT, s);
-        dim3 grid((unsigned)(L.ntile_a * kAppBN / kTG), (unsigned)L.nkt_a);
-        k_split_t<<<grid, 256, 0, s>>>(beta, ld_beta, nproj, npw, kAppBN, L.nkt_a, betaT);
+        dim3 grid((unsigned)(L.ntile_a * kAppBN / kTG), (unsigned)((L.nkt_a + 1) / 2));
+        k_split_t<<<grid, 256, 0, s>>>(beta, ld_beta, nproj, npw, kAppBN, L.nkt_a, et, invt, base + L.betaT_off);
     }
     return cuda_check(cudaGetLastError(), "k_split_t launch");
 }
 
 template <int EPI>
-qm_status gemm_launch(const unsigned char* A, const unsigned char* B, int nkt, int BN, int M, int N, int mt, int ntl,
-                      int splits, float* C, size_t ldc, size_t zstride, bool accumulate, int* err, cudaStream_t s) {
-    const int per = (nkt + splits - 1) / splits;
-    splits = (nkt + per - 1) / per;
-    const size_t smem = (size_t)kStages * (block_bytes(TM) + block_bytes(BN));
+qm_status gemm_launch(const unsigned char* A, const unsigned char* B, int nkt, int BN, const GemmShape& sh, int M, int N, int mt,
+                      int ntl, float* C, size_t ldc, size_t zstride, bool accumulate, const float* inv_m, const float* inv_n,
+                      int* err, cudaStream_t s) {
+    const int per = (nkt + sh.splits - 1) / sh.splits, bn = BN / sh.bsub;
+    const size_t smem = (size_t)kNlStages * (sh.msub * block_bytes(TM) + block_bytes(bn));
     qm_status st = allow_dynamic_smem((const void*)k_nl_gemm<EPI>, smem, "tensor-core nonlocal GEMM shared memory");
     if (st) return st;
     ProfScope pf(PF_UMMA, s);
-    const dim3 grid = EPI == 0 ? dim3(ntl, mt, splits) : dim3(mt, ntl, splits);
-    k_nl_gemm<EPI><<<grid, kGemmThreads, smem, s>>>(A, B, nkt, BN, M, N, per, C, ldc, zstride, accumulate ? 1 : 0, err);
+    const int mg = (mt + sh.msub - 1) / sh.msub, ng = ntl * sh.bsub;
+    const dim3 grid = EPI == 0 ? dim3(ng, mg, sh.splits) : dim3(mg, ng, sh.splits);
+    k_nl_gemm<EPI><<<grid, kGemmThreads, smem, s>>>(A, B, nkt, bn, sh.bsub, sh.msub, M, N, mt, per, C, ldc, zstride,
+                                                  accumulate ? 1 : 0, inv_m, inv_n, err);
     return cuda_check(cudaGetLastError(), "k_nl_gemm launch");
 }
 
@@ -487,7 +660,7 @@ size_t nonlocal_tc_bytes(int nproj, int nb, int npw, bool with_beta) {
 
 size_t nonlocal_tc_beta_bytes(int nproj, int nb, int npw) {
     const NlLayout L = nl_layout(nproj, nb, npw, true);
-    return L.psiX_off;  // betaK and betaT come first
+    return L.psiX_off;  // betaK, betaT and their scales come first
 }
 
 qm_status nonlocal_tc_prepare(int nproj, int nb, int npw, const float2* beta, int ld_beta, void* beta_work,
@@ -496,7 +669,7 @@ qm_status nonlocal_tc_prepare(int nproj, int nb, int npw, const float2* beta, in
     const NlLayout L = nl_layout(nproj, nb, npw, true);
     if (qm_status st0 = check_limits(L)) return st0;
     unsigned char* w = (unsigned char*)beta_work;
-    return split_beta(nproj, npw, beta, ld_beta, L, w + L.betaK_off, w + L.betaT_off, s);
+    return split_beta(nproj, npw, beta, ld_beta, L, w, s);
 }
 
 qm_status nonlocal_tc(int nproj, int nb, int npw, const float2* beta, int ld_beta, const void* beta_prepared,
@@ -507,51 +680,61 @@ qm_status nonlocal_tc(int nproj, int nb, int npw, const float2* beta, int ld_bet
     const NlLayout L = nl_layout(nproj, nb, npw, own_beta);
     if (qm_status st0 = check_limits(L)) return st0;
     unsigned char* w = (unsigned char*)work;
-    const unsigned char* betaK;
-    const unsigned char* betaT;
     qm_status st;
+    const unsigned char* bw = w;  // the split projectors: in the workspace or prepared
+    NlLayout Lb = L;
     if (own_beta) {
-        if ((st = split_beta(nproj, npw, beta, ld_beta, L, w + L.betaK_off, w + L.betaT_off, s))) return st;
-        betaK = w + L.betaK_off;
-        betaT = w + L.betaT_off;
+        if ((st = split_beta(nproj, npw, beta, ld_beta, L, w, s))) return st;
     } else {
-        const NlLayout Lb = nl_layout(nproj, nb, npw, true);
-        betaK = (const unsigned char*)beta_prepared + Lb.betaK_off;
-        betaT = (const unsigned char*)beta_prepared + Lb.betaT_off;
+        Lb = nl_layout(nproj, nb, npw, true);
+        bw = (const unsigned char*)beta_prepared;
     }
+    const unsigned char *betaK = bw + Lb.betaK_off, *betaT = bw + Lb.betaT_off;
+    const float *invk = (const float*)(bw + Lb.inv_off), *invt = invk + nproj;
     unsigned char* psiX = w + L.psiX_off;
     float* part = (float*)(w + L.part_off);
     unsigned char* E = w + L.e_off;
+    int* emax = (int*)(w + L.emax_off);
+    float *invb = (float*)(w + L.invb_off), *inve = invb + nb;
+    // short rows find their scale in the splitting kernel (one launch less, one CTA per four bands)
+    const bool self = npw <= kSelfScale;
+    if (!self) {
+        ProfScope pf(PF_SPLIT, s);
+        k_nl_rowmax<<<dim3((unsigned)nb, kNlSegs), 256, 0, s>>>(psi, ld_psi, nb, npw, emax);
+    }
     {
         ProfScope pf(PF_SPLIT, s);
-        const dim3 grid((unsigned)((L.nkt_p * (KT / 8) + kSplitChunks - 1) / kSplitChunks), (unsigned)(L.ntile_p * L.bn_p / 8));
-        k_split_rows<<<grid, 256, 0, s>>>(psi, ld_psi, nb, npw, 1, L.bn_p, L.nkt_p, psiX);
+        const dim3 grid(self ? 1u : (unsigned)((L.nkt_p * (KT / 8) + kSplitChunks - 1) / kSplitChunks),
+                        (unsigned)(L.ntile_p * L.bn_p / 8));
+        k_split_rows<<<grid, 256, 0, s>>>(psi, ld_psi, nb, npw, 1, L.bn_p, L.nkt_p, self ? nullptr : emax, invb, psiX);
     }
     if ((st = cuda_check(cudaGetLastError(), "k_split_rows launch"))) return st;
     // projection C[p][2b + t] = <beta_p | psi_b>, split over K
     const size_t ldc_p = (size_t)L.ntile_p * L.bn_p;
-    if ((st = gemm_launch<0>(betaK, psiX, L.nkt_p, L.bn_p, nproj, 2 * nb, L.mtile_p, L.ntile_p, L.splits, part, ldc_p,
-                             L.zstride, false, err, s)))
+    if ((st = gemm_launch<0>(betaK, psiX, L.nkt_p, L.bn_p, L.sp, nproj, 2 * nb, L.mtile_p, L.ntile_p, part, ldc_p, L.zstride,
+                             false, nullptr, nullptr, err, s)))
         return st;
     const int Z = [&] {
         const int per = (L.nkt_p + L.splits - 1) / L.splits;
         return (L.nkt_p + per - 1) / per;
     }();
     float* Pd = (float*)(w + L.pd_off);
-    {
+    // few projectors: the split-K sums are taken in the expansion (one launch less)
+    const bool fold = (long)nproj * Z <= kFoldReduce;
+    if (!fold) {
         ProfScope pf(PF_SPLIT, s);
-        k_reduce_p<<<grid_for((long)nproj * 2 * nb), 256, 0, s>>>(part, Z, L.zstride, (int)ldc_p, nproj, 2 * nb, D, Pd);
+        k_reduce_p<<<grid_for((long)nproj * 2 * nb), 256, 0, s>>>(part, Z, L.zstride, (int)ldc_p, nproj, 2 * nb, D, invk, invb, Pd);
     }
     if ((st = cuda_check(cudaGetLastError(), "k_reduce_p launch"))) return st;
     {
         ProfScope pf(PF_SPLIT, s);
-        const long n = (long)L.mtile_a * TM * L.nkt_a * (KT / 8);
-        k_expand_e<<<grid_for(n), 256, 0, s>>>(Pd, nproj, nb, L.mtile_a * TM, L.nkt_a, E);
+        k_expand_e<<<(unsigned)(L.mtile_a * TM / 8), 256, fold ? (size_t)nproj * 4 * sizeof(float2) : 0, s>>>(
+            Pd, fold ? part : nullptr, Z, L.zstride, (int)ldc_p, D, invk, invb, nproj, nb, L.nkt_a, inve, E);
     }
     if ((st = cuda_check(cudaGetLastError(), "k_expand_e launch"))) return st;
     // application out[b][g] (+)= sum_p beta[p][g] D_p P[p][b]
-    return gemm_launch<1>(E, betaT, L.nkt_a, kAppBN, 2 * nb, npw, L.mtile_a, L.ntile_a, 1, (float*)out, (size_t)ld_out,
-                          0, accumulate, err, s);
+    return gemm_launch<1>(E, betaT, L.nkt_a, kAppBN, L.sa, 2 * nb, npw, L.mtile_a, L.ntile_a, (float*)out, (size_t)ld_out, 0, accumulate,
+                          inve, invt, err, s);
 }
 
 }  // namespace qm

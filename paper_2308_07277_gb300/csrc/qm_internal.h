@@ -257,9 +257,9 @@ qm_status zdigits_tn(int M, int N, int K, const double2* A, int lda, const doubl
 size_t zdigits_bytes(bool cn, int M, int N, int K);
 // ---- tensor-core nonlocal step of the precision form (nonlocal_tc.cu) ----
 constexpr int kMaxUmmaSplits = 64;
-// out[b][g] (+)= sum_p beta[p][g] D_p <beta_p|psi_b> (FP32 complex in/out) as BF16x3 split
+// out[b][g] (+)= sum_p beta[p][g] D_p <beta_p|psi_b> (FP32 complex in/out) as FP16-pair split
 // tcgen05 products; err: device int set on a timed-out wait.
-// The same product with operands pre-split into tile-blocked BF16 planes in global memory and
+// The same product with operands pre-split into tile-blocked FP16 planes in global memory and
 // streamed by bulk copies through a warp-specialised tcgen05 pipeline (nonlocal_tc.cu).
 // beta_prepared: NULL (beta is split on every call, in `work`) or the output of
 // nonlocal_tc_prepare (nonlocal_tc_beta_bytes bytes; depends on nproj and npw only).
@@ -318,6 +318,12 @@ qm_status chol_transform(double2* S, int lds, int nd, double drop_rel, int* keep
 qm_status chol_transform_rows(const double2* L, int lds, int nd, const int* keep, const int* rank, int kept,
                               double2* X, double2* W, cudaStream_t s);
 
+// FP32: small products (C (+)= with tn), and register-tiled ones (qm_hpsi_noalloc)
+size_t csmall_cn_bytes(int M, int N, int K);
+qm_status csmall_cn(int M, int N, int K, const float2* A, int lda, const float2* B, int ldb, float2* C, int ldc,
+                    const GemmWork& w, cudaStream_t s);
+qm_status csmall_tn(int M, int N, int K, const float2* A, int lda, const double* d, const float2* B, int ldb, float2* C,
+                    int ldc, cudaStream_t s);
 qm_status cgemm_cn(int M, int N, int K, const float2* A, int lda, const float2* B, int ldb,
                    float2* C, int ldc, float2* partial, int splits, cudaStream_t s);
 qm_status cgemm_tn(int M, int N, int K, const float2* A, int lda, const double* d,

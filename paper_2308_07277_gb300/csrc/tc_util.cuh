@@ -24,6 +24,9 @@ constexpr uint32_t idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// the same with A = B = FP16
+constexpr uint32_t idesc_f16(int M, int N) { return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24); }
+
 // wait for the phase `phase` of the mbarrier to complete; false after `limit` polls
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t phase, long limit) {
     for (long i = 0; i < limit; ++i) {

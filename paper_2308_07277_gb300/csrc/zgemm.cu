@@ -208,20 +208,20 @@ k_gemm_tn(int M, int N, int K, const float2* __restrict__ A, int lda, const doub
 // two steps 1249 -> 164 ms, H psi of the two-atom cell (8 x 8 x 411) 518 -> 65 us, and at large
 // sizes 1.22 instead of 1.01 TFLOP/s (480 x 157 x 18232, 10.9 -> 9.0 ms).
 constexpr int kCnTile = 8, kCnK = 32, kCnGroups = 4;
+template <class C>
 __global__ void __launch_bounds__(NTH)
-k_zcn(int M, int N, int K, const double2* __restrict__ A, int lda, const double2* __restrict__ B, int ldb,
-      double2* __restrict__ out, int ldo, int kchunk, const GemmFlags f) {
+k_cn(int M, int N, int K, const C* __restrict__ A, int lda, const C* __restrict__ B, int ldb, C* __restrict__ out, int ldo, int kchunk, const GemmFlags f) {
     if (f.any && !*f.any) return;
-    __shared__ double2 As[kCnK][kCnTile + 1], Bs[kCnK][kCnTile + 1];
+    __shared__ C As[kCnK][kCnTile + 1], Bs[kCnK][kCnTile + 1];
     const int tid = threadIdx.x, tx = tid & 7, ty = (tid >> 3) & 7, kg = tid >> 6;
     const int m0 = blockIdx.y * kCnTile, n0 = blockIdx.x * kCnTile;
     const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
     const int lrow = tid / kCnK, lk = tid % kCnK;  // this thread's element of a tile (one row per warp)
-    double2 acc = make_double2(0.0, 0.0);
+    C acc = czero<C>();
     const bool va = m0 + lrow < M, vb = n0 + lrow < N;
-    const double2* pa = A + (size_t)(va ? m0 + lrow : 0) * lda + lk;
-    const double2* pb = B + (size_t)(vb ? n0 + lrow : 0) * ldb + lk;
-    double2 ra = make_double2(0.0, 0.0), rb = ra;
+    const C* pa = A + (size_t)(va ? m0 + lrow : 0) * lda + lk;
+    const C* pb = B + (size_t)(vb ? n0 + lrow : 0) * ldb + lk;
+    C ra = czero<C>(), rb = ra;
     if (kb + lk < ke) {
         if (va) ra = pa[kb];
         if (vb) rb = pb[kb];
@@ -230,25 +230,25 @@ k_zcn(int M, int N, int K, const double2* __restrict__ A, int lda, const double2
         As[lk][lrow] = ra;
         Bs[lk][lrow] = rb;
         __syncthreads();
-        ra = rb = make_double2(0.0, 0.0);
+        ra = rb = czero<C>();
         if (k0 + kCnK + lk < ke) {  // the next tile's loads are in flight during this tile's products
             if (va) ra = pa[k0 + kCnK];
             if (vb) rb = pb[k0 + kCnK];
         }
 #pragma unroll
         for (int q = 0; q < kCnK / kCnGroups; ++q) {
-            const double2 a = As[kg + kCnGroups * q][ty], b = Bs[kg + kCnGroups * q][tx];
+            const C a = As[kg + kCnGroups * q][ty], b = Bs[kg + kCnGroups * q][tx];
             acc.x = fma(a.x, b.x, fma(a.y, b.y, acc.x));
             acc.y = fma(a.x, b.y, fma(-a.y, b.x, acc.y));
         }
         __syncthreads();
     }
-    double2* red = &As[0][0];  // 3 x 64 partial sums of the K groups, added in group order
+    C* red = &As[0][0];  // 3 x 64 partial sums of the K groups, added in group order
     if (kg) red[(kg - 1) * 64 + ty * 8 + tx] = acc;
     __syncthreads();
     if (kg == 0 && m0 + ty < M && n0 + tx < N && (!f.any || f.em[m0 + ty] == f.flag || f.en[n0 + tx] == f.flag)) {
         for (int g = 0; g < kCnGroups - 1; ++g) {
-            const double2 v = red[g * 64 + ty * 8 + tx];
+            const C v = red[g * 64 + ty * 8 + tx];
             acc.x += v.x;
             acc.y += v.y;
         }
@@ -257,21 +257,22 @@ k_zcn(int M, int N, int K, const double2* __restrict__ A, int lda, const double2
 }
 
 constexpr int kTnM = 8, kTnN = 32, kTnK = 16;
+template <class T>
 __global__ void __launch_bounds__(NTH)
-k_ztn(int M, int N, int K, const double2* __restrict__ A, int lda, const double* __restrict__ d, double alpha,
-      const double2* __restrict__ B, int ldb, double2* __restrict__ C, int ldc, int accumulate, const GemmFlags f) {
+k_tn(int M, int N, int K, const T* __restrict__ A, int lda, const double* __restrict__ d, double alpha,
+     const T* __restrict__ B, int ldb, T* __restrict__ C, int ldc, int accumulate, const GemmFlags f) {
     if (f.any && !*f.any) return;
-    __shared__ double2 As[kTnK][kTnM], Bs[kTnK][kTnN];
+    __shared__ T As[kTnK][kTnM], Bs[kTnK][kTnN];
     const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
     const int n0 = blockIdx.x * kTnN, m0 = blockIdx.y * kTnM;
-    double2 acc = make_double2(0.0, 0.0);
+    T acc = czero<T>();
     for (int k0 = 0; k0 < K; k0 += kTnK) {
         if (tid < kTnK * kTnM) {
             const int kk = tid / kTnM, m = m0 + tid % kTnM, k = k0 + kk;
-            double2 v = make_double2(0.0, 0.0);
+            T v = czero<T>();
             if (k < K && m < M) {
                 v = A[(size_t)k * lda + m];
-                const double sc = d ? alpha * d[k] : alpha;
+                const auto sc = (decltype(v.x))(d ? alpha * d[k] : alpha);
                 v.x *= sc;
                 v.y *= sc;
             }
@@ -280,12 +281,12 @@ k_ztn(int M, int N, int K, const double2* __restrict__ A, int lda, const double*
 #pragma unroll
         for (int q = 0; q < kTnK * kTnN / NTH; ++q) {
             const int kk = ty + q * (NTH / kTnN), k = k0 + kk, n = n0 + tx;
-            Bs[kk][tx] = (k < K && n < N) ? B[(size_t)k * ldb + n] : make_double2(0.0, 0.0);
+            Bs[kk][tx] = (k < K && n < N) ? B[(size_t)k * ldb + n] : czero<T>();
         }
         __syncthreads();
         const int kn = min(kTnK, K - k0);
         for (int kk = 0; kk < kn; ++kk) {
-            const double2 a = As[kk][ty], b = Bs[kk][tx];
+            const T a = As[kk][ty], b = Bs[kk][tx];
             acc.x = fma(a.x, b.x, fma(-a.y, b.y, acc.x));
             acc.y = fma(a.x, b.y, fma(a.y, b.x, acc.y));
         }
@@ -293,9 +294,9 @@ k_ztn(int M, int N, int K, const double2* __restrict__ A, int lda, const double*
     }
     const int m = m0 + ty, n = n0 + tx;
     if (m < M && n < N && (!f.any || f.em[m] == f.flag || f.en[n] == f.flag)) {
-        double2* p = C + (size_t)m * ldc + n;
+        T* p = C + (size_t)m * ldc + n;
         if (accumulate) {
-            const double2 o = *p;
+            const T o = *p;
             acc.x += o.x;
             acc.y += o.y;
         }
@@ -304,16 +305,16 @@ k_ztn(int M, int N, int K, const double2* __restrict__ A, int lda, const double*
 }
 
 // Splits of cn over K: the count that minimises (waves of one CTA per SM) x (cycles per CTA) plus
-// the reduction of the partial sums, 128 pipe cycles per term of an 8 x 8 tile; the fixed costs
+// the reduction of the partial sums, 128 pipe cycles per term of an 8 x 8 tile in FP64, about 12 in FP32; the fixed costs
 // (1500 cycles of start and loads, 4000 of the second launch) are estimates of launch latency.
-int zcn_splits(int M, int N, int K, long cap) {
+int zcn_splits(int M, int N, int K, long cap, int per_term = 128) {
     const long tiles = (long)((M + kCnTile - 1) / kCnTile) * ((N + kCnTile - 1) / kCnTile), sms = device_sms();
     const int smax = (int)std::max<long>(1, std::min<long>({(long)((K + kCnK - 1) / kCnK), cap, 64L}));
     int best = 1;
     long cost = -1;
     for (int s = 1; s <= smax; ++s) {
         const long kc = ((K + s - 1) / s + kCnK - 1) / kCnK * kCnK;
-        const long c = (tiles * s + sms - 1) / sms * (kc * 128 + 1500) + (s > 1 ? 4000 + 40L * s : 0);
+        const long c = (tiles * s + sms - 1) / sms * (kc * per_term + 1500) + (s > 1 ? 4000 + 40L * s : 0);
         if (cost < 0 || c < cost) {
             cost = c;
             best = s;
@@ -322,29 +323,30 @@ int zcn_splits(int M, int N, int K, long cap) {
     return best;
 }
 
-qm_status zcn_launch(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb, double2* C, int ldc,
-                     double2* partial, size_t partial_bytes, const GemmFlags& f, cudaStream_t s) {
-    const long cap = partial ? (long)(partial_bytes / sizeof(double2)) / ((long)M * N) : 1;
-    int splits = zcn_splits(M, N, K, std::max<long>(1, cap));
+template <class T>
+qm_status cn_small(int M, int N, int K, const T* A, int lda, const T* B, int ldb, T* C, int ldc, T* partial, size_t partial_bytes, const GemmFlags& f, cudaStream_t s) {
+    const long cap = partial ? (long)(partial_bytes / sizeof(T)) / ((long)M * N) : 1;
+    int splits = zcn_splits(M, N, K, std::max<long>(1, cap), sizeof(T) == 8 ? 12 : 128);
     int kchunk = std::max(kCnK, ((K + splits - 1) / splits + kCnK - 1) / kCnK * kCnK);
     splits = std::max(1, (K + kchunk - 1) / kchunk);
     const dim3 grid((N + kCnTile - 1) / kCnTile, (M + kCnTile - 1) / kCnTile, splits);
     {
         ProfScope pf(PF_GEMM_CN, s);
-        k_zcn<<<grid, NTH, 0, s>>>(M, N, K, A, lda, B, ldb, splits > 1 ? partial : C, splits > 1 ? N : ldc, kchunk, f);
+        k_cn<T><<<grid, NTH, 0, s>>>(M, N, K, A, lda, B, ldb, splits > 1 ? partial : C, splits > 1 ? N : ldc, kchunk, f);
     }
     if (splits > 1) {
         ProfScope pf(PF_REDUCE, s);
-        k_reduce_splits<double2><<<grid_stride_blocks((size_t)M * N, 64, 16), 64, 0, s>>>(M, N, partial, splits, C, ldc);
+        k_reduce_splits<T><<<grid_stride_blocks((size_t)M * N, 64, 16), 64, 0, s>>>(M, N, partial, splits, C, ldc);
     }
     return cuda_check(cudaGetLastError(), "gemm_cn launch");
 }
 
-qm_status ztn_launch(int M, int N, int K, const double2* A, int lda, const double* d, double alpha, const double2* B,
-                     int ldb, double2* C, int ldc, bool accumulate, const GemmFlags& f, cudaStream_t s) {
+template <class T>
+qm_status tn_small(int M, int N, int K, const T* A, int lda, const double* d, double alpha, const T* B, int ldb, T* C,
+                   int ldc, bool accumulate, const GemmFlags& f, cudaStream_t s) {
     ProfScope pf(PF_GEMM_TN, s);
     const dim3 grid((N + kTnN - 1) / kTnN, (M + kTnM - 1) / kTnM);
-    k_ztn<<<grid, NTH, 0, s>>>(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate ? 1 : 0, f);
+    k_tn<T><<<grid, NTH, 0, s>>>(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate ? 1 : 0, f);
     return cuda_check(cudaGetLastError(), "gemm_tn launch");
 }
 
@@ -480,8 +482,8 @@ qm_status zgemm_cn(int M, int N, int K, const double2* A, int lda, const double2
     bool done = false;
     qm_status st = w.digits ? zdigits_cn(M, N, K, A, lda, B, ldb, C, ldc, w, s, &f, &done) : QM_OK;
     if (st) return st;
-    return done ? zcn_launch(M, N, K, A, lda, B, ldb, C, ldc, nullptr, 0, f, s)
-                : zcn_launch(M, N, K, A, lda, B, ldb, C, ldc, (double2*)w.ptr, w.bytes, f, s);
+    return done ? cn_small(M, N, K, A, lda, B, ldb, C, ldc, (double2*)nullptr, 0, f, s)
+                : cn_small(M, N, K, A, lda, B, ldb, C, ldc, (double2*)w.ptr, w.bytes, f, s);
 }
 qm_status zgemm_tn(int M, int N, int K, const double2* A, int lda, const double* d, const double2* B, int ldb,
                    double2* C, int ldc, bool accumulate, const GemmWork& w, cudaStream_t s, double alpha) {
@@ -490,7 +492,21 @@ qm_status zgemm_tn(int M, int N, int K, const double2* A, int lda, const double*
     bool done = false;
     qm_status st = w.digits ? zdigits_tn(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate, w, s, &f, &done) : QM_OK;
     if (st) return st;
-    return ztn_launch(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate, f, s);
+    return tn_small(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate, f, s);
+}
+// FP32 products on the same small tiles (the precision form's nonlocal part of small cells): sums of at
+// most a few tens of terms per thread, then of the groups and splits, in FP32
+size_t csmall_cn_bytes(int M, int N, int K) {
+    const int splits = zcn_splits(M, N, K, 64, 12);
+    return splits > 1 ? (size_t)splits * M * N * sizeof(float2) : 0;
+}
+qm_status csmall_cn(int M, int N, int K, const float2* A, int lda, const float2* B, int ldb, float2* C, int ldc,
+                    const GemmWork& w, cudaStream_t s) {
+    return cn_small(M, N, K, A, lda, B, ldb, C, ldc, (float2*)w.ptr, w.bytes, GemmFlags{}, s);
+}
+qm_status csmall_tn(int M, int N, int K, const float2* A, int lda, const double* d, const float2* B, int ldb, float2* C,
+                    int ldc, cudaStream_t s) {
+    return tn_small(M, N, K, A, lda, d, 1.0, B, ldb, C, ldc, true, GemmFlags{}, s);
 }
 qm_status cgemm_cn(int M, int N, int K, const float2* A, int lda, const float2* B, int ldb, float2* C, int ldc,
                    float2* partial, int splits, cudaStream_t s) {
