@@ -52,9 +52,9 @@ namespace {
 
 constexpr int KT = 16;          // K tile (real elements): 2 chunks of 8 FP16
 constexpr int TM = 128;         // rows of an A tile (M of the MMA)
-constexpr int kNlStages = 4;
+constexpr int kNlStages = 4;    // K tiles in flight: at most 128 KB, which leaves room for an FFT CTA (77 to 87 KB) on the SM
 constexpr int kGemmThreads = 384;
-constexpr int kNlSegs = 4;      // partial maxima per row
+constexpr int kNlSegs = 8;      // partial maxima per row
 constexpr long kSpin = 1L << 26;
 
 __host__ __device__ constexpr size_t plane_bytes(int R) { return (size_t)R * KT * 2; }
@@ -245,17 +245,25 @@ __global__ void __launch_bounds__(256) k_split_t(const float2* __restrict__ beta
 }
 
 // sum the split-K partials of the projection C[z][p][c] (FP32, ldc; c = 2b + t) in a fixed order,
-// undo the rows' scales and multiply by D_p: Pd[p][c] (consecutive threads, consecutive c: coalesced)
-__global__ void k_reduce_p(const float* __restrict__ part, int Z, size_t zstride, int ldc, int P, int ncol,
-                           const double* __restrict__ D, const float* __restrict__ inv_p, const float* __restrict__ inv_b,
-                           float* __restrict__ Pd) {
-    const size_t total = (size_t)P * ncol;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-        const int p = (int)(e / ncol), c = (int)(e - (size_t)p * ncol);
+// undo the rows' scales and multiply by D_p: Pd[p][c].  CTA: 32 consecutive outputs x 8 parts of the
+// splits (one thread per output took 7 us for 64 splits of a few thousand outputs, all of it latency).
+__global__ void __launch_bounds__(256) k_reduce_p(const float* __restrict__ part, int Z, size_t zstride, int ldc, int P,
+                                                  int ncol, const double* __restrict__ D, const float* __restrict__ inv_p,
+                                                  const float* __restrict__ inv_b, float* __restrict__ Pd) {
+    __shared__ float red[8][32];
+    const size_t total = (size_t)P * ncol, e = blockIdx.x * (size_t)32 + (threadIdx.x & 31);
+    const int w = threadIdx.x >> 5, p = (int)(e / ncol), c = (int)(e - (size_t)p * ncol);
+    float a = 0.f;
+    if (e < total) {
         const float* q = part + (size_t)p * ldc + c;
-        float a = 0.f;
 #pragma unroll 8
-        for (int z = 0; z < Z; ++z) a += __ldg(q + (size_t)z * zstride);
+        for (int z = w; z < Z; z += 8) a += __ldg(q + (size_t)z * zstride);
+    }
+    red[w][threadIdx.x & 31] = a;
+    __syncthreads();
+    if (w == 0 && e < total) {
+#pragma unroll
+        for (int i = 1; i < 8; ++i) a += red[i][threadIdx.x];
         Pd[e] = a * __ldg(inv_p + p) * __ldg(inv_b + (c >> 1)) * (float)__ldg(D + p);
     }
 }
@@ -278,25 +286,28 @@ __global__ void __launch_bounds__(256) k_expand_e(const float* __restrict__ Pd, 
     __syncthreads();
     int h = 0;
     const float ib = part && b4 < nb ? __ldg(inv_b + b4) : 0.f;
-    for (int p = tid >> 2; p < P; p += 64) {
+    if (!part && b4 < nb) {
+#pragma unroll 8
+        for (int p = tid >> 2; p < P; p += 64) {
+            const float2 a = __ldg(reinterpret_cast<const float2*>(Pd + (size_t)p * 2 * nb) + b4);
+            h = max(h, max(f_abs(a.x), f_abs(a.y)));
+        }
+    }
+    for (int p = tid >> 2; part && p < P; p += 64) {
         float2 a = make_float2(0.f, 0.f);
         if (b4 < nb) {
-            if (part) {
-                const float* q = part + (size_t)p * ldc + 2 * b4;
+            const float* q = part + (size_t)p * ldc + 2 * b4;
 #pragma unroll 8
-                for (int z = 0; z < Z; ++z) {
-                    const float2 v = __ldg(reinterpret_cast<const float2*>(q + (size_t)z * zstride));
-                    a.x += v.x;
-                    a.y += v.y;
-                }
-                const float ip = __ldg(inv_p + p), d = (float)__ldg(D + p);
-                a.x = a.x * ip * ib * d;
-                a.y = a.y * ip * ib * d;
-            } else {
-                a = __ldg(reinterpret_cast<const float2*>(Pd + (size_t)p * 2 * nb) + b4);
+            for (int z = 0; z < Z; ++z) {
+                const float2 v = __ldg(reinterpret_cast<const float2*>(q + (size_t)z * zstride));
+                a.x += v.x;
+                a.y += v.y;
             }
+            const float ip = __ldg(inv_p + p), d = (float)__ldg(D + p);
+            a.x = a.x * ip * ib * d;
+            a.y = a.y * ip * ib * d;
         }
-        if (part) sp[p * 4 + q4] = a;
+        sp[p * 4 + q4] = a;
         h = max(h, max(f_abs(a.x), f_abs(a.y)));
     }
 #pragma unroll
@@ -305,8 +316,8 @@ __global__ void __launch_bounds__(256) k_expand_e(const float* __restrict__ Pd, 
     __syncthreads();
     const int nchunk = nkt * (KT / 8), rlo = tid & 7, r = blockIdx.x * 8 + rlo, b = r >> 1, t = r & 1;
     const float sc = row_scale(smax[rlo >> 1]);
-    if (tid < 8 && !t && b < nb) inv[b] = inv_scale(sc);
-    for (int ch = tid >> 3; ch < nchunk; ch += 32) {
+    if (tid < 8 && !t && b < nb && blockIdx.y == 0) inv[b] = inv_scale(sc);
+    for (int ch = blockIdx.y * 32 + (tid >> 3); ch < nchunk; ch += 32 * gridDim.y) {
         float v[8];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -532,8 +543,8 @@ int proj_bn(int nb) {
 constexpr int kAppBN = 256;
 
 // Tile shape of a GEMM (row tiles per CTA, parts of a B tile, splits of K): the cheapest by rounds of CTAs
-// over the SMs times the cycles of a CTA, its K tiles (3 products of 128 x BN x 16 per row tile, or their
-// operands at 45 bytes per clock) plus about 6000 of start, fill and drain.
+// over the SMs times the cycles of a CTA's K tiles (3 products of 128 x BN x 16 per row tile, or their
+// operands at 45 bytes per clock, at least the 400 a step takes), plus start, fill and drain.
 struct GemmShape {
     int msub, bsub, splits;
 };
@@ -547,7 +558,12 @@ GemmShape gemm_shape(int mtiles, int ntiles, int BN, int nkt, int max_bsub, int 
             const int sp = (int)std::max<long>(1, std::min<long>({(long)max_splits, (long)std::max(1, nkt / 8), sms / tiles}));
             const int per = (nkt + sp - 1) / sp, m = std::min(msub, mtiles), bn = BN / bsub;
             const double tile = std::max(1.5 * m * bn, (m * 8192.0 + bn * 64.0) / 45.0);
-            const double c = (double)((tiles * sp + sms - 1) / sms) * (per * tile + 6000.0);
+            // CTAs an SM holds, by shared memory and tensor memory; more than one share its throughput
+            const int cols = msub * (bn <= 32 ? 32 : bn <= 64 ? 64 : bn <= 128 ? 128 : 256);
+            const long occ = std::min<long>((226 << 10) / (long)(kNlStages * (msub * block_bytes(TM) + block_bytes(bn))), 512 / cols);
+            const long n = tiles * sp;
+            const double load = occ > 1 ? std::max(1.0, (double)n / sms) : (double)((n + sms - 1) / sms);
+            const double c = std::max(load * per * tile, (double)((n + sms * occ - 1) / (sms * occ)) * per * std::max(tile, 400.0)) + 6000.0;
             if (cost < 0 || c < cost) {
                 cost = c;
                 best = GemmShape{msub, bsub, (nkt + per - 1) / per};
@@ -606,8 +622,6 @@ qm_status check_limits(const NlLayout& L) {
     return QM_OK;
 }
 
-inline int grid_for(long n, int per = 256) { return grid_stride_blocks((size_t)std::max<long>(n, 1), per, 16); }
-
 qm_status split_beta(int nproj, int npw, const float2* beta, int ld_beta, const NlLayout& L, unsigned char* base, cudaStream_t s) {
     float* invk = (float*)(base + L.inv_off);
     float* invt = invk + nproj;
@@ -641,7 +655,8 @@ qm_status gemm_launch(const unsigned char* A, const unsigned char* B, int nkt, i
                       int ntl, float* C, size_t ldc, size_t zstride, bool accumulate, const float* inv_m, const float* inv_n,
                       int* err, cudaStream_t s) {
     const int per = (nkt + sh.splits - 1) / sh.splits, bn = BN / sh.bsub;
-    const size_t smem = (size_t)kNlStages * (sh.msub * block_bytes(TM) + block_bytes(bn));
+    const size_t stage = sh.msub * block_bytes(TM) + block_bytes(bn);
+    const size_t smem = kNlStages * stage;
     qm_status st = allow_dynamic_smem((const void*)k_nl_gemm<EPI>, smem, "tensor-core nonlocal GEMM shared memory");
     if (st) return st;
     ProfScope pf(PF_UMMA, s);
@@ -723,12 +738,14 @@ qm_status nonlocal_tc(int nproj, int nb, int npw, const float2* beta, int ld_bet
     const bool fold = (long)nproj * Z <= kFoldReduce;
     if (!fold) {
         ProfScope pf(PF_SPLIT, s);
-        k_reduce_p<<<grid_for((long)nproj * 2 * nb), 256, 0, s>>>(part, Z, L.zstride, (int)ldc_p, nproj, 2 * nb, D, invk, invb, Pd);
+        k_reduce_p<<<(unsigned)(((size_t)nproj * 2 * nb + 31) / 32), 256, 0, s>>>(part, Z, L.zstride, (int)ldc_p, nproj, 2 * nb, D, invk, invb, Pd);
     }
     if ((st = cuda_check(cudaGetLastError(), "k_reduce_p launch"))) return st;
     {
         ProfScope pf(PF_SPLIT, s);
-        k_expand_e<<<(unsigned)(L.mtile_a * TM / 8), 256, fold ? (size_t)nproj * 4 * sizeof(float2) : 0, s>>>(
+        // the chunks of a row group over up to eight CTAs (each finds the bands' largest values for itself)
+        const dim3 grid((unsigned)(L.mtile_a * TM / 8), fold ? 1u : (unsigned)std::min(8, (L.nkt_a + 15) / 16));
+        k_expand_e<<<grid, 256, fold ? (size_t)nproj * 4 * sizeof(float2) : 0, s>>>(
             Pd, fold ? part : nullptr, Z, L.zstride, (int)ldc_p, D, invk, invb, nproj, nb, L.nkt_a, inve, E);
     }
     if ((st = cuda_check(cudaGetLastError(), "k_expand_e launch"))) return st;
