@@ -27,7 +27,7 @@ __global__ void k_chol_orig(const double2* __restrict__ S, int lds, int nd, doub
         orig[i] = S[(size_t)i * lds + i].x;
 }
 
-// factor the nb x nb diagonal block at (k0, k0) in shared memory (nb <= kNB); 1024 threads
+// factor the nb x nb diagonal block at (k0, k0) in shared memory (nb <= kNB), a warp per row
 __global__ void __launch_bounds__(1024)
 k_chol_diag(double2* __restrict__ S, int lds, int k0, int nb, const double* __restrict__ orig, double drop_rel,
             int* __restrict__ keep) {
@@ -35,17 +35,20 @@ k_chol_diag(double2* __restrict__ S, int lds, int k0, int nb, const double* __re
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // column, row
     if (ty < nb && tx <= ty) a[ty][tx] = S[(size_t)(k0 + ty) * lds + k0 + tx];
     __syncthreads();
+    // (the pivot's root and reciprocal are taken by one warp: a warp's FP64 instruction holds
+    // its partition's pipe for 64 cycles, and a square root and a division are about 16 of them; 8 columns: 7 us, 35 us with every warp's own)
     for (int j = 0; j < nb; ++j) {
-        const double piv = a[j][j].x;
-        const bool ok = piv > drop_rel * orig[k0 + j] && piv > 0.0 && isfinite(piv);
-        __syncthreads();  // every thread has read the pivot
-        if (ty == j && tx == 0) {
-            a[j][j] = make_double2(ok ? sqrt(piv) : 0.0, 0.0);
-            keep[k0 + j] = ok ? 1 : 0;
-        }
-        if (tx == j && ty > j) {  // column j below the diagonal
-            const double il = ok ? 1.0 / sqrt(piv) : 0.0;
-            a[ty][j] = make_double2(a[ty][j].x * il, a[ty][j].y * il);
+        if (ty == j) {
+            const double piv = a[j][j].x;
+            const bool ok = piv > drop_rel * orig[k0 + j] && piv > 0.0 && isfinite(piv);
+            const double root = ok ? sqrt(piv) : 0.0, il = ok ? 1.0 / root : 0.0;
+            __syncwarp();
+            if (tx == 0) {
+                a[j][j] = make_double2(root, 0.0);
+                keep[k0 + j] = ok ? 1 : 0;
+            }
+            const int i = j + 1 + tx;  // column j below the diagonal, one row per lane
+            if (i < nb) a[i][j] = make_double2(a[i][j].x * il, a[i][j].y * il);
         }
         __syncthreads();
         if (ty > j && tx > j && tx <= ty) {  // a[i][k] -= L[i][j] conj(L[k][j])
@@ -178,6 +181,33 @@ k_trinv_rows(const double2* __restrict__ L, int lds, int nd, const int* __restri
         if (keep[k]) W[(size_t)c * ldw + rank[k]] = make_double2(x[k].x, -x[k].y);
 }
 
+// the same for nd <= 32: lane i holds x_i, L in shared memory, the reciprocals of the diagonal taken by all
+// lanes at once; column by column, so a row costs a broadcast and a multiply-add instead of a reduction
+// over lanes and a division (8 columns: 3.6 us, 12 us)
+__global__ void __launch_bounds__(32)
+k_trinv_small(const double2* __restrict__ L, int lds, int nd, const int* __restrict__ keep,
+              const int* __restrict__ rank, double2* __restrict__ W, int ldw) {
+    __shared__ double2 l[32][33];
+    const int c = blockIdx.x, i = threadIdx.x;
+    for (int r = c; r < nd; ++r)
+        if (i <= r) l[r][i] = L[(size_t)r * lds + i];
+    const bool kept = i < nd && keep[i];
+    __syncwarp();
+    const double inv = kept && i >= c ? 1.0 / l[i][i].x : 0.0;
+    double2 x = make_double2(i == c ? 1.0 : 0.0, 0.0);  // right-hand side, then solution
+    for (int j = c; j < nd; ++j) {
+        const double f = __shfl_sync(0xffffffffu, inv, j);  // 0 for a dropped j
+        const double2 xj = make_double2(__shfl_sync(0xffffffffu, x.x, j) * f, __shfl_sync(0xffffffffu, x.y, j) * f);
+        if (i == j) x = xj;
+        if (i > j && i < nd) {
+            const double2 a = l[i][j];
+            x.x = fma(-a.x, xj.x, fma(a.y, xj.y, x.x));
+            x.y = fma(-a.x, xj.y, fma(-a.y, xj.x, x.y));
+        }
+    }
+    if (kept) W[(size_t)c * ldw + rank[i]] = i < c ? make_double2(0.0, 0.0) : make_double2(x.x, -x.y);
+}
+
 __global__ void k_rank(const int* __restrict__ keep, int nd, int* __restrict__ rank, int* __restrict__ kept) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         int r = 0;
@@ -207,7 +237,7 @@ qm_status chol_transform(double2* S, int lds, int nd, double drop_rel, int* keep
         const int nb = std::min(kNB, nd - k0), below = nd - k0 - nb;
         {
             ProfScope pf(PF_CHOL, s);
-            k_chol_diag<<<1, 1024, 0, s>>>(S, lds, k0, nb, orig, drop_rel, keep);
+            k_chol_diag<<<1, 32 * nb, 0, s>>>(S, lds, k0, nb, orig, drop_rel, keep);
         }
         if (below > 0) {
             const int nt = (below + 31) / 32;
@@ -232,7 +262,8 @@ qm_status chol_transform(double2* S, int lds, int nd, double drop_rel, int* keep
 qm_status chol_transform_rows(const double2* L, int lds, int nd, const int* keep, const int* rank, int kept,
                               double2* X, double2* W, cudaStream_t s) {
     ProfScope pf(PF_CHOL, s);
-    k_trinv_rows<<<nd, 32, 0, s>>>(L, lds, nd, keep, rank, kept, X, nd, W, kept);
+    if (nd <= 32) k_trinv_small<<<nd, 32, 0, s>>>(L, lds, nd, keep, rank, W, kept);
+    else k_trinv_rows<<<nd, 32, 0, s>>>(L, lds, nd, keep, rank, kept, X, nd, W, kept);
     return cuda_check(cudaGetLastError(), "k_trinv_rows launch");
 }
 

@@ -8,6 +8,7 @@
 //                     reflector makes every subdiagonal element real).  One cooperative
 //                     launch, one grid barrier per column, rows resident in shared memory
 //                     (k_tridiag: two barriers per column, for matrices beyond that).
+//                     (k_tridiag_small: one CTA, matrices up to kTriSmall.)
 //   2. k_multisect    the j-th smallest eigenvalue of T by multisection on Sturm counts
 //                     (Sec. 8.4.1): a warp tests 32 points per round, 12 rounds.
 //   3. k_inviter      eigenvectors of T by inverse iteration (LU with partial pivoting of the
@@ -317,51 +318,204 @@ k_tridiag_rows(double2* __restrict__ A, int lda, int m, double2* __restrict__ Vh
     }
 }
 
-// number of eigenvalues of T smaller than x (Sturm sequence with a pivot guard)
-__device__ __forceinline__ int sturm_count(const double* __restrict__ d, const double* __restrict__ e2, int m,
-                                           double x, double pivmin) {
+// The reduction of a small matrix (m <= kTriSmall) in one CTA, the matrix in shared memory: a column of the
+// grid-wide reduction costs 8 us of barriers and launch-wide latency whatever its length.  The FP64 pipe
+// takes 16 cycles per warp instruction, so the work is laid out to need few of them: four threads per row in
+// the product A v (two shuffle steps instead of five), the rank-2 update on the lower triangle only, the
+// reflector's divisions once.  Warp 0 updates the next column first and builds its reflector (a root, a
+// division and two reductions in a chain) while the others update the rest.  Eight-band solves (m up to 32):
+// 115 us on average, 248 us with the grid-wide kernel.
+constexpr int kTriSmall = 64;
+__global__ void __launch_bounds__(256)
+k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restrict__ Vh, double2* __restrict__ tau,
+                double* __restrict__ d, double* __restrict__ e) {
+    extern __shared__ double2 smt[];
+    const int ld = m + 1;
+    double2 *a = smt, *vb = smt + m * ld, *w = vb + 2 * m;  // [m][ld], reflectors of two columns, product
+    __shared__ double2 s_t[2];
+    const int tid = threadIdx.x, lane = tid & 31;
+    for (int i = tid; i < m * m; i += 256) a[(i / m) * ld + i % m] = A[(size_t)(i / m) * lda + i % m];
+    // the reflector of column k (one warp)
+    auto reflector = [&](int k) {
+        const int n = m - k - 1;
+        double2* v = vb + (k & 1) * m;
+        double part = 0.0;
+        for (int i = 1 + lane; i < n; i += 32) {
+            const double2 x = a[(k + 1 + i) * ld + k];
+            part += x.x * x.x + x.y * x.y;
+        }
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+        const double2 alpha = a[(k + 1) * ld + k];
+        double2 t = make_double2(0.0, 0.0), scale = make_double2(0.0, 0.0);
+        double beta = alpha.x;
+        if (part > 0.0 || alpha.y != 0.0) {
+            beta = -copysign(sqrt(alpha.x * alpha.x + alpha.y * alpha.y + part), alpha.x);
+            const double2 den = make_double2(alpha.x - beta, alpha.y);
+            // the two reciprocals on two lanes
+            const double inv = 1.0 / (lane & 1 ? den.x * den.x + den.y * den.y : beta);
+            const double ib = __shfl_sync(0xffffffffu, inv, 0), id = __shfl_sync(0xffffffffu, inv, 1);
+            t = make_double2((beta - alpha.x) * ib, -alpha.y * ib);
+            scale = make_double2(den.x * id, -den.y * id);
+        }
+        for (int i = lane; i < n; i += 32) {
+            const double2 x = i ? cmul(a[(k + 1 + i) * ld + k], scale) : make_double2(1.0, 0.0);
+            v[i] = x;
+            Vh[(size_t)k * m + k + 1 + i] = x;
+        }
+        if (lane == 0) {
+            s_t[k & 1] = t;
+            tau[k] = t;
+            e[k] = beta;
+            d[k] = a[k * ld + k].x;
+        }
+    };
+    __syncthreads();
+    if (tid < 32) reflector(0);
+    for (int k = 0; k < m - 1; ++k) {
+        __syncthreads();
+        const int n = m - k - 1;
+        double2* a22 = a + (k + 1) * ld + k + 1;
+        const double2 t = s_t[k & 1], *v = vb + (k & 1) * m;
+        const bool any = t.x != 0.0 || t.y != 0.0;  // (uniform)
+        if (any) {
+            // w = t A22 v
+            for (int r0 = 0; r0 < n; r0 += 64) {
+                const int r = r0 + (tid >> 2);
+                double2 acc = make_double2(0.0, 0.0);
+                if (r < n)
+                    for (int j = tid & 3; j < n; j += 4) {
+                        const double2 x = a22[r * ld + j], y = v[j];
+                        acc.x = fma(x.x, y.x, fma(-x.y, y.y, acc.x));
+                        acc.y = fma(x.x, y.y, fma(x.y, y.x, acc.y));
+                    }
+#pragma unroll
+                for (int o = 1; o < 4; o <<= 1) {
+                    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+                    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+                }
+                if (r < n && (tid & 3) == 0) w[r] = cmul(t, acc);
+            }
+            __syncthreads();
+            if (tid < 32) {  // w -= t (w^H v) / 2 v
+                double2 dp = make_double2(0.0, 0.0);
+                for (int i = lane; i < n; i += 32) {
+                    const double2 c = cmulc(w[i], v[i]);
+                    dp.x += c.x;
+                    dp.y += c.y;
+                }
+                for (int o = 16; o > 0; o >>= 1) {
+                    dp.x += __shfl_xor_sync(0xffffffffu, dp.x, o);
+                    dp.y += __shfl_xor_sync(0xffffffffu, dp.y, o);
+                }
+                const double2 a2 = cmul(make_double2(-0.5 * t.x, -0.5 * t.y), dp);
+                for (int i = lane; i < n; i += 32) {
+                    const double2 c = cmul(a2, v[i]);
+                    w[i].x += c.x;
+                    w[i].y += c.y;
+                }
+            }
+            __syncthreads();
+        }
+        // A22 -= v w^H + w v^H: lower triangle, mirrored
+        auto update = [&](int i, int j) {
+            const double2 vi = v[i], wi = w[i], vj = v[j], wj = w[j];
+            double2 x = a22[i * ld + j];
+            x.x = fma(-vi.x, wj.x, fma(-vi.y, wj.y, fma(-wi.x, vj.x, fma(-wi.y, vj.y, x.x))));
+            x.y = fma(-vi.y, wj.x, fma(vi.x, wj.y, fma(-wi.y, vj.x, fma(wi.x, vj.y, x.y))));
+            if (i == j) x.y = 0.0;
+            a22[i * ld + j] = x;
+            if (j > 0 && i != j) a22[j * ld + i] = make_double2(x.x, -x.y);
+        };
+        if (tid < 32) {
+            if (any)
+                for (int i = lane; i < n; i += 32) update(i, 0);
+            __syncwarp();
+            if (k + 1 < m - 1) reflector(k + 1);
+        } else if (any) {
+            for (int q = tid - 32; q < n * (n - 1) / 2; q += 224) {  // rows and columns 1 .. n-1
+                int i = (int)((sqrtf(8.0f * (float)q + 1.0f) - 1.0f) * 0.5f);
+                while ((i + 1) * (i + 2) / 2 <= q) ++i;
+                while (i * (i + 1) / 2 > q) --i;
+                update(i + 1, q - i * (i + 1) / 2 + 1);
+            }
+        }
+    }
+    __syncthreads();
+    if (tid == 0) d[m - 1] = a[(m - 1) * ld + m - 1].x;
+}
+
+// number of eigenvalues of T smaller than x: sign changes of the leading minors' determinants by their
+// three-term recurrence p_i = (d_i - x) p_(i-1) - e_(i-1)^2 p_(i-2) (Wilkinson, The Algebraic Eigenvalue
+// Problem, Ch. 5, Sec. 37), T scaled below 2 in magnitude.  (Eight-band solves: 66 us, 150 us with quotients.)  A ratio p_i / p_(i-1) below 2^-100 is replaced
+// by -2^-100 (a shift of d_i by less than 2^-99, and a zero counts as negative), so eight rows change the
+// pair by factors between 2^-900 and 2^40 and its rescaling every eight rows keeps it in range.  The
+// quotient form has a division in the chain of every row, about 450 cycles on this GPU's FP64 pipe; a
+// multiply-add is 45, and eight unrolled rows keep the loads and differences off the chain.
+__device__ __forceinline__ int sturm_count(const double* __restrict__ d, const double* __restrict__ e2, int m, double x) {
     int c = 0;
-    double q = d[0] - x;
-    if (fabs(q) < pivmin) q = -pivmin;
-    if (q < 0.0) ++c;
-    for (int i = 1; i < m; ++i) {
-        q = (d[i] - x) - e2[i - 1] / q;
-        if (fabs(q) < pivmin) q = -pivmin;
-        if (q < 0.0) ++c;
+    double p0 = 1.0, p1 = d[0] - x;
+    if (fabs(p1) < 0x1p-100) p1 = -0x1p-100;
+    if (p1 < 0.0) ++c;
+    for (int i0 = 1; i0 < m; i0 += 8) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {  // (rows m .. of the last group are padding: d = 4, e = 0, no sign change)
+            const int i = i0 + q;
+            double p = fma(d[i] - x, p1, -e2[i - 1] * p0);
+            const int hp = __double2hiint(p), h1 = __double2hiint(p1);
+            if ((hp & 0x7FF00000) < (h1 & 0x7FF00000) - (100 << 20)) p = -0x1p-100 * p1;
+            c += (int)((unsigned)(__double2hiint(p) ^ h1) >> 31);
+            p0 = p1;
+            p1 = p;
+        }
+        // divide the pair by the power of two of the larger one
+        const int ex = max(__double2hiint(p0) & 0x7FF00000, __double2hiint(p1) & 0x7FF00000);
+        const double sc = __hiloint2double(max(0x7FE00000 - ex, 0x00100000), 0);
+        p0 *= sc;
+        p1 *= sc;
     }
     return c;
 }
 
-__global__ void k_sq(const double* __restrict__ e, double* __restrict__ e2, int n) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) e2[i] = e[i] * e[i];
-}
-
-// one warp per wanted eigenvalue j < nev
-__global__ void k_multisect(const double* __restrict__ d, const double* __restrict__ e, const double* __restrict__ e2,
-                            int m, int nev, double* __restrict__ evals) {
-    const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
+// one warp (CTA) per wanted eigenvalue j < nev; d and e^2, scaled, in shared memory (2 (m + 8) doubles)
+__global__ void __launch_bounds__(32) k_multisect(const double* __restrict__ d, const double* __restrict__ e, int m, int nev,
+                                                  double* __restrict__ evals) {
+    extern __shared__ double sms[];
+    double *sd = sms, *se = sms + m + 8;
+    const int j = blockIdx.x, lane = threadIdx.x;
     if (j >= nev) return;
-    // Gershgorin interval and pivot guard
-    double lo = 1e300, hi = -1e300, emax = 0.0;
+    // Gershgorin interval
+    double lo = 1e300, hi = -1e300;
     for (int i = lane; i < m; i += 32) {
         const double r = (i > 0 ? fabs(e[i - 1]) : 0.0) + (i < m - 1 ? fabs(e[i]) : 0.0);
         lo = fmin(lo, d[i] - r);
         hi = fmax(hi, d[i] + r);
-        if (i < m - 1) emax = fmax(emax, e2[i]);
     }
     for (int o = 16; o > 0; o >>= 1) {
         lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
         hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-        emax = fmax(emax, __shfl_xor_sync(0xffffffffu, emax, o));
     }
     const double span = fmax(hi - lo, 1e-300);
     lo -= 1e-14 * span + 1e-300;
     hi += 1e-14 * span + 1e-300;
-    const double pivmin = fmax(1e-300, 2.2250738585072014e-308 * fmax(1.0, emax));
+    // a power of two near 1 / max(|lo|, |hi|): scaled entries below 2
+    int ex = 0;
+    frexp(fmax(fabs(lo), fabs(hi)), &ex);
+    const double scale = ldexp(1.0, -ex), back = ldexp(1.0, ex);
+    for (int i = lane; i < m; i += 32) {
+        sd[i] = d[i] * scale;
+        const double t = i < m - 1 ? e[i] * scale : 0.0;
+        se[i] = t * t;
+    }
+    if (lane < 8) {
+        sd[m + lane] = 4.0;
+        se[m + lane] = 0.0;
+    }
+    lo *= scale;
+    hi *= scale;
+    __syncwarp();
     for (int round = 0; round < 14; ++round) {
         const double x = lo + (hi - lo) * (double)(lane + 1) / 33.0;
-        const int c = sturm_count(d, e2, m, x, pivmin);
+        const int c = sturm_count(sd, se, m, x);
         const unsigned above = __ballot_sync(0xffffffffu, c > j);
         double nlo = lo, nhi = hi;
         if (above) {
@@ -375,64 +529,72 @@ __global__ void k_multisect(const double* __restrict__ d, const double* __restri
         hi = nhi;
         if (hi - lo <= 4.0e-16 * fmax(fabs(lo), fabs(hi)) + 1e-300) break;
     }
-    if (lane == 0) evals[j] = 0.5 * (lo + hi);
+    if (lane == 0) evals[j] = 0.5 * (lo + hi) * back;
 }
 
-// solve (T - lam) x = b in place (b -> x), T = tridiag(e, d, e); LU with partial pivoting.
-// The row being eliminated is carried in registers (each finished row is stored once and only
-// read back by the back substitution), so the loop has no read-after-write through memory.
-// work: 3 arrays of m doubles (finished rows: pivot, first and second super-diagonal).
-__device__ void tri_solve(const double* __restrict__ d, const double* __restrict__ e, int m, double lam,
-                          double tiny, double* __restrict__ a, double* __restrict__ c, double* __restrict__ c2,
-                          double* __restrict__ b) {
-    // current row i: diag ai, super ci (and super-super c2i = 0 unless a swap put it there), rhs bi
-    double ai = d[0] - lam, ci = (m > 1) ? e[0] : 0.0, bi = b[0];
+// LU with partial pivoting of T - lam, T = tridiag(e, d, e): row i of U is (1 / r[i], c[i], c2[i]), the
+// multiplier f[i] eliminates row i + 1, sw[i] = 1 marks a swap of rows i and i + 1 before it.
+// The row being eliminated is carried in registers.  Pivots below cut are raised to tiny = eps |T|.
+__device__ __forceinline__ void tri_factor(const double* __restrict__ d, const double* __restrict__ e, int m, double lam, double tiny, double cut,
+                                           double* __restrict__ r, double* __restrict__ c, double* __restrict__ c2,
+                                           double* __restrict__ f, unsigned char* __restrict__ sw) {
+    double ai = d[0] - lam, ci = (m > 1) ? e[0] : 0.0;
     for (int i = 0; i < m - 1; ++i) {
         const double sub = e[i];
-        // next original row i+1: sub, diag, sup, rhs
-        double an = d[i + 1] - lam, cn = (i + 1 < m - 1) ? e[i + 1] : 0.0, bn = b[i + 1];
-        double c2i = 0.0;
-        if (fabs(ai) >= fabs(sub)) {
-            if (ai == 0.0) ai = tiny;
-            const double f = sub / ai;
-            an -= f * ci;
-            bn -= f * bi;
-        } else {  // swap rows i and i+1
-            const double f = ai / sub;
-            const double ai0 = ai, ci0 = ci, bi0 = bi;
-            ai = sub;
-            ci = an;
-            c2i = cn;
-            bi = bn;
-            an = ci0 - f * an;
-            cn = -f * cn;
-            bn = bi0 - f * bn;
-            (void)ai0;
+        double an = d[i + 1] - lam, cn = (i + 1 < m - 1) ? e[i + 1] : 0.0;
+        const bool keep = fabs(ai) >= fabs(sub) || fabs(sub) < cut;
+        if (keep && fabs(ai) < cut) ai = copysign(tiny, ai);
+        const double piv = keep ? ai : sub, inv = 1.0 / piv, fi = (keep ? sub : ai) * inv;
+        r[i] = inv;
+        f[i] = fi;
+        sw[i] = keep ? 0 : 1;
+        if (keep) {
+            c[i] = ci;
+            c2[i] = 0.0;
+            an -= fi * ci;
+        } else {  // rows i and i+1 swapped
+            c[i] = an;
+            c2[i] = cn;
+            an = ci - fi * an;
+            cn = -fi * cn;
         }
-        a[i] = ai;
-        c[i] = ci;
-        c2[i] = c2i;
-        b[i] = bi;
         ai = an;
         ci = cn;
-        bi = bn;
     }
-    if (ai == 0.0) ai = tiny;
-    a[m - 1] = ai;
-    double x1 = bi / ai, x2 = 0.0;  // x[i+1], x[i+2]
+    if (fabs(ai) < cut) ai = copysign(tiny, ai);
+    r[m - 1] = 1.0 / ai;
+}
+// solve with that factorisation in place (b -> x): no division in the chains
+__device__ __forceinline__ void tri_apply(int m, const double* __restrict__ r, const double* __restrict__ c,
+                                          const double* __restrict__ c2, const double* __restrict__ f,
+                                          const unsigned char* __restrict__ sw, double* __restrict__ b) {
+    double bi = b[0];
+#pragma unroll 4
+    for (int i = 0; i < m - 1; ++i) {
+        double bn = b[i + 1];
+        if (sw[i]) {
+            const double t = bi;
+            bi = bn;
+            bn = t;
+        }
+        b[i] = bi;
+        bi = fma(-f[i], bi, bn);
+    }
+    double x1 = bi * r[m - 1], x2 = 0.0;  // x[i+1], x[i+2]
     b[m - 1] = x1;
+#pragma unroll 4
     for (int i = m - 2; i >= 0; --i) {
-        const double xi = (b[i] - c[i] * x1 - c2[i] * x2) / a[i];
+        const double xi = fma(-c2[i], x2, fma(-c[i], x1, b[i])) * r[i];
         b[i] = xi;
         x2 = x1;
         x1 = xi;
     }
 }
 
-// infinity norm of T and the cluster tolerance: eigenvalues closer than ctol form a cluster whose
-// vectors are orthogonalised explicitly; outside clusters inverse iteration alone leaves a
-// non-orthogonality of about eps * |T| / gap <= 1e-11
-__device__ double tri_ctol(const double* __restrict__ d, const double* __restrict__ e, int m) {
+// infinity norm of T.  Eigenvalues closer than a part ctol of it form a cluster whose vectors are
+// orthogonalised explicitly; outside clusters inverse iteration alone leaves a non-orthogonality of about
+// eps |T| / gap: 1e-13 where the chain of dot products is short (m <= 128, ctol = 1e-3), 1e-11 (1e-5) above
+__device__ double tri_norm(const double* __restrict__ d, const double* __restrict__ e, int m) {
     double tn = 0.0;
     for (int i = threadIdx.x & 31; i < m; i += 32)
         tn = fmax(tn, fabs(d[i]) + (i > 0 ? fabs(e[i - 1]) : 0.0) + (i < m - 1 ? fabs(e[i]) : 0.0));
@@ -440,41 +602,59 @@ __device__ double tri_ctol(const double* __restrict__ d, const double* __restric
     return tn;
 }
 
-// one warp per eigenvalue j: lane 0 runs the (sequential) tridiagonal solves of three inverse
-// iterations from a deterministic start, the warp shares the O(m) vector work; the normalised
+// deterministic pseudo-random start vector (a counter hash of (j, i))
+__device__ __forceinline__ double start_entry(int j, int i) {
+    unsigned h = 2654435761u * (unsigned)(j + 1) ^ (2246822519u * (unsigned)(i + 1));
+    h ^= h >> 15;
+    h *= 2246822519u;
+    h ^= h >> 13;
+    return ((double)(h >> 8) / 16777216.0) - 0.5;
+}
+
+// one warp per eigenvalue j: lane 0 factors T - lambda_j once and runs the (sequential) solves of three
+// inverse iterations from a deterministic start, the warp shares the O(m) vector work; the normalised
 // vector is left in x_j = work + (4 j + 3) m.  Vectors of one cluster are orthogonalised
-// afterwards (k_cluster_orth), so every eigenvalue's iterations run in parallel.
+// afterwards (k_cluster_orth), so every eigenvalue's iterations run in parallel.  kSmem: the factors, T
+// and the vector live in shared memory (57 m bytes), else in work and wf.
+__host__ __device__ constexpr size_t inviter_smem(int m) { return (size_t)m * (7 * sizeof(double) + 1); }
+template <bool kSmem>
 __global__ void __launch_bounds__(32)
-k_inviter(const double* __restrict__ d, const double* __restrict__ e, int m, int nev,
-          const double* __restrict__ evals, double* __restrict__ work) {
+k_inviter(const double* __restrict__ dg, const double* __restrict__ eg, int m, int nev,
+          const double* __restrict__ evals, double* __restrict__ work, double* __restrict__ wf, unsigned char* __restrict__ wsw) {
+    extern __shared__ double smi[];
     const int j = blockIdx.x, lane = threadIdx.x;
     if (j >= nev) return;
-    const double tn = tri_ctol(d, e, m);
-    double* a = work + (size_t)j * 4 * m;
-    double* c = a + m;
-    double* c2 = c + m;
-    double* x = c2 + m;
+    const double tn = tri_norm(dg, eg, m);
+    double* xg = work + ((size_t)j * 4 + 3) * m;
+    double *r = kSmem ? smi : work + (size_t)j * 4 * m, *c = r + m, *c2 = c + m;
+    double* f = kSmem ? smi + 3 * m : wf + (size_t)j * m;
+    double* x = kSmem ? smi + 4 * m : xg;
+    const double *d = dg, *e = eg;
+    unsigned char* sw = kSmem ? (unsigned char*)(smi + 7 * m) : wsw + (size_t)j * m;
+    if (kSmem) {
+        double *sd = smi + 5 * m, *se = smi + 6 * m;
+        for (int i = lane; i < m; i += 32) {
+            sd[i] = dg[i];
+            se[i] = i < m - 1 ? eg[i] : 0.0;
+        }
+        d = sd;
+        e = se;
+    }
     const double tiny = 2.2e-16 * fmax(tn, 1e-200);
     const double lam = evals[j];
-    // deterministic pseudo-random start (a counter hash of (j, i))
-    for (int i = lane; i < m; i += 32) {
-        unsigned h = 2654435761u * (unsigned)(j + 1) ^ (2246822519u * (unsigned)(i + 1));
-        h ^= h >> 15;
-        h *= 2246822519u;
-        h ^= h >> 13;
-        x[i] = ((double)(h >> 8) / 16777216.0) - 0.5;
-    }
+    for (int i = lane; i < m; i += 32) x[i] = start_entry(j, i);
     __syncwarp();
+    if (lane == 0) tri_factor(d, e, m, lam, tiny, 0x1p-100 * fmax(tn, 1e-200), r, c, c2, f, sw);
     for (int it = 0; it < 3; ++it) {
-        if (lane == 0) tri_solve(d, e, m, lam, tiny, a, c, c2, x);
+        if (lane == 0) tri_apply(m, r, c, c2, f, sw, x);
         __syncwarp();
         double xm = 0.0;  // rescale before any sum of squares can overflow
         for (int i = lane; i < m; i += 32) xm = fmax(xm, fabs(x[i]));
         for (int o = 16; o > 0; o >>= 1) xm = fmax(xm, __shfl_xor_sync(0xffffffffu, xm, o));
-        const double r = (xm > 0.0 && xm < 1e300) ? 1.0 / xm : 1.0;
+        const double rs = (xm > 0.0 && xm < 1e300) ? 1.0 / xm : 1.0;
         double nrm = 0.0;
         for (int i = lane; i < m; i += 32) {
-            x[i] *= r;
+            x[i] *= rs;
             nrm += x[i] * x[i];
         }
         for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
@@ -482,44 +662,31 @@ k_inviter(const double* __restrict__ d, const double* __restrict__ e, int m, int
         for (int i = lane; i < m; i += 32) x[i] *= nrm;
         __syncwarp();
     }
+    if (kSmem)
+        for (int i = lane; i < m; i += 32) xg[i] = x[i];
 }
 
 // One CTA per cluster leader (eigenvalue j0 not within ctol of j0-1): the cluster's vectors
 // j0..j1-1 are orthonormalised in order by two classical Gram-Schmidt passes against the
 // earlier ones (dot products split over the warps), then written as columns of Y (imag 0).
+// A vector that loses more than nine tenths of its length (graded couplings beside equal diagonal
+// entries make the iterates of several eigenvalues agree) is started afresh, then iterated from what the
+// orthogonalisation leaves, at most 8 times, with pivots of at least eps |T| so that eigenvalues that agree
+// to rounding count alike; factors in work, wf, wsw.
 __global__ void __launch_bounds__(256)
 k_cluster_orth(const double* __restrict__ d, const double* __restrict__ e, int m, int nev,
-               const double* __restrict__ evals, double* __restrict__ work, double2* __restrict__ Y, int ldy) {
+               const double* __restrict__ evals, double* work, double* wf, unsigned char* wsw,
+               double2* __restrict__ Y, int ldy) {
     __shared__ double dots[256];
     __shared__ double red[32];
     const int j0 = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (j0 >= nev) return;
-    const double ctol = 1e-5 * tri_ctol(d, e, m);  // every warp computes the same value
+    const double tn = tri_norm(d, e, m), ctol = (m <= 128 ? 1e-3 : 1e-5) * tn;  // every warp computes the same value
     if (j0 > 0 && evals[j0] - evals[j0 - 1] <= ctol) return;  // not a cluster leader
     int j1 = j0 + 1;
     while (j1 < nev && evals[j1] - evals[j1 - 1] <= ctol) ++j1;
     auto X = [&](int q) { return work + ((size_t)q * 4 + 3) * m; };
-    for (int j = j0 + 1; j < j1; ++j) {
-        double* x = X(j);
-        for (int pass = 0; pass < 2; ++pass) {
-            for (int q0 = j0; q0 < j; q0 += 256) {  // coefficients against up to 256 earlier vectors
-                const int nq = min(256, j - q0);
-                for (int q = warp; q < nq; q += 8) {
-                    const double* y = X(q0 + q);
-                    double s = 0.0;
-                    for (int i = lane; i < m; i += 32) s += y[i] * x[i];
-                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                    if (lane == 0) dots[q] = s;
-                }
-                __syncthreads();
-                for (int i = tid; i < m; i += 256) {
-                    double v = x[i];
-                    for (int q = 0; q < nq; ++q) v -= dots[q] * X(q0 + q)[i];
-                    x[i] = v;
-                }
-                __syncthreads();
-            }
-        }
+    auto sum = [&](const double* x) {  // |x|^2, the same value in every thread
         double s = 0.0;
         for (int i = tid; i < m; i += 256) s += x[i] * x[i];
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -527,9 +694,55 @@ k_cluster_orth(const double* __restrict__ d, const double* __restrict__ e, int m
         __syncthreads();
         double t = 0.0;
         for (int w = 0; w < 8; ++w) t += red[w];
-        const double inv = 1.0 / sqrt(t);
-        for (int i = tid; i < m; i += 256) x[i] *= inv;
         __syncthreads();
+        return t;
+    };
+    auto scale_by = [&](double* x, double f) {
+        for (int i = tid; i < m; i += 256) x[i] *= f;
+        __syncthreads();
+    };
+    for (int j = j0 + 1; j < j1; ++j) {
+        double* x = X(j);
+        for (int again = 0;; ++again) {
+            for (int pass = 0; pass < 2; ++pass) {
+                for (int q0 = j0; q0 < j; q0 += 256) {  // coefficients against up to 256 earlier vectors
+                    const int nq = min(256, j - q0);
+                    for (int q = warp; q < nq; q += 8) {
+                        const double* y = X(q0 + q);
+                        double s = 0.0;
+                        for (int i = lane; i < m; i += 32) s += y[i] * x[i];
+                        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                        if (lane == 0) dots[q] = s;
+                    }
+                    __syncthreads();
+                    for (int i = tid; i < m; i += 256) {
+                        double v = x[i];
+                        for (int q = 0; q < nq; ++q) v -= dots[q] * X(q0 + q)[i];
+                        x[i] = v;
+                    }
+                    __syncthreads();
+                }
+            }
+            const double t = sum(x);
+            scale_by(x, t > 0.0 ? 1.0 / sqrt(t) : 0.0);
+            if (t > 1e-2 || again == 8) break;
+            if (!again || t == 0.0)
+                for (int i = tid; i < m; i += 256) x[i] = start_entry(j + nev, i);
+            __syncthreads();
+            if (tid == 0) {
+                double *r = work + (size_t)j * 4 * m, *c = r + m, *c2 = c + m, *f = wf + (size_t)j * m;
+                unsigned char* sw = wsw + (size_t)j * m;
+                const double tiny = 2.2e-16 * fmax(tn, 1e-200);
+                if (!again) tri_factor(d, e, m, evals[j], tiny, tiny, r, c, c2, f, sw);
+                tri_apply(m, r, c, c2, f, sw, x);
+                double xm = 0.0;
+                for (int i = 0; i < m; ++i) xm = fmax(xm, fabs(x[i]));
+                red[0] = (xm > 0.0 && xm < 1e300) ? 1.0 / xm : 1.0;
+            }
+            __syncthreads();
+            scale_by(x, red[0]);
+            scale_by(x, 1.0 / sqrt(sum(x)));
+        }
     }
     for (int j = j0; j < j1; ++j)
         for (int i = tid; i < m; i += 256) Y[(size_t)i * ldy + j] = make_double2(X(j)[i], 0.0);
@@ -565,6 +778,39 @@ k_backtransf(const double2* __restrict__ Vh, const double2* __restrict__ tau, in
     for (int i = tid; i < m; i += bs) Y[(size_t)i * ldy + j] = sy[i];
 }
 
+// the same for m <= 64: one warp per column, the column in registers (rows lane and lane + 32), the next
+// reflector loaded while the present one is applied
+__global__ void __launch_bounds__(32)
+k_backtransf_small(const double2* __restrict__ Vh, const double2* __restrict__ tau, int m, double2* __restrict__ Y, int ldy) {
+    const int j = blockIdx.x, r0 = threadIdx.x, r1 = r0 + 32;
+    const double2 z = make_double2(0.0, 0.0);
+    double2 y0 = r0 < m ? Y[(size_t)r0 * ldy + j] : z, y1 = r1 < m ? Y[(size_t)r1 * ldy + j] : z;
+    auto ref = [&](int k, int r) { return k >= 0 && r > k && r < m ? Vh[(size_t)k * m + r] : z; };
+    double2 v0 = ref(m - 2, r0), v1 = ref(m - 2, r1), t = tau[m - 2];
+    for (int k = m - 2; k >= 0; --k) {
+        const double2 n0 = ref(k - 1, r0), n1 = ref(k - 1, r1), nt = k > 0 ? tau[k - 1] : z;
+        if (t.x != 0.0 || t.y != 0.0) {
+            const double2 c0 = cmulc(v0, y0), c1 = cmulc(v1, y1);
+            double2 sp = make_double2(c0.x + c1.x, c0.y + c1.y);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                sp.x += __shfl_xor_sync(0xffffffffu, sp.x, o);
+                sp.y += __shfl_xor_sync(0xffffffffu, sp.y, o);
+            }
+            const double2 s = cmul(t, sp), u0 = cmul(v0, s), u1 = cmul(v1, s);
+            y0.x -= u0.x;
+            y0.y -= u0.y;
+            y1.x -= u1.x;
+            y1.y -= u1.y;
+        }
+        v0 = n0;
+        v1 = n1;
+        t = nt;
+    }
+    if (r0 < m) Y[(size_t)r0 * ldy + j] = y0;
+    if (r1 < m) Y[(size_t)r1 * ldy + j] = y1;
+}
+
 }  // namespace
 
 size_t heev_work_bytes(int m, int nev) {
@@ -572,8 +818,9 @@ size_t heev_work_bytes(int m, int nev) {
     b += align_up((size_t)m * m * sizeof(double2), 256);      // Vh
     b += align_up((size_t)m * sizeof(double2), 256);          // tau
     b += align_up((size_t)2 * m * sizeof(double2), 256) * 2;  // wbuf, published rows (double-buffered)
-    b += align_up((size_t)m * sizeof(double), 256) * 3;       // d, e, e2
+    b += align_up((size_t)m * sizeof(double), 256) * 2;       // d, e
     b += align_up((size_t)nev * 4 * m * sizeof(double), 256); // inverse-iteration scratch
+    b += align_up((size_t)nev * m * sizeof(double), 256) + align_up((size_t)nev * m, 256);
     return b;
 }
 
@@ -612,8 +859,9 @@ qm_status heev_lowest(double2* A, int lda, int m, int nev, double* evals, double
     double2* prow = (double2*)take((size_t)2 * m * sizeof(double2));
     double* d = (double*)take((size_t)m * sizeof(double));
     double* e = (double*)take((size_t)m * sizeof(double));
-    double* e2 = (double*)take((size_t)m * sizeof(double));
     double* iw = (double*)take((size_t)nev * 4 * m * sizeof(double));
+    double* wf = (double*)take((size_t)nev * m * sizeof(double));  // multipliers and swaps beyond shared memory
+    unsigned char* wsw = (unsigned char*)take((size_t)nev * m);
     qm_status st;
     if (m == 1) {
         // T = (a11): copy the real diagonal, eigenvector 1
@@ -622,7 +870,12 @@ qm_status heev_lowest(double2* A, int lda, int m, int nev, double* evals, double
         cudaMemcpyAsync(Y, &one, sizeof(double2), cudaMemcpyHostToDevice, s);
         return cuda_check(cudaGetLastError(), "heev m=1");
     }
-    {
+    if (m <= kTriSmall) {
+        const size_t smem = ((size_t)m * (m + 1) + 3 * m) * sizeof(double2);
+        if ((st = allow_dynamic_smem((const void*)k_tridiag_small, smem, "heev_lowest: reduction kernel"))) return st;
+        ProfScope pf(PF_TRIDIAG, s);
+        k_tridiag_small<<<1, 256, smem, s>>>(A, lda, m, Vh, tau, d, e);
+    } else {
         int dev = 0, sms = 152;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -684,26 +937,38 @@ qm_status heev_lowest(double2* A, int lda, int m, int nev, double* evals, double
         if (st) return st;
     }
     {
+        const size_t smem = 2 * (size_t)(m + 8) * sizeof(double);
+        if ((st = allow_dynamic_smem((const void*)k_multisect, smem, "heev_lowest: multisection"))) return st;
         ProfScope pf(PF_MULTISECT, s);
-        k_sq<<<(m + 255) / 256, 256, 0, s>>>(e, e2, m - 1);
+        k_multisect<<<nev, 32, smem, s>>>(d, e, m, nev, evals);
     }
     {
-        ProfScope pf(PF_MULTISECT, s);
-        k_multisect<<<nev, 32, 0, s>>>(d, e, e2, m, nev, evals);
+        // shared memory while every eigenvalue's CTA is resident at once (1 KB of it is the system's)
+        int dev = 0, sms = 152;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const size_t per = inviter_smem(m) + 1024;
+        const bool fits = per <= 200 * 1024 && nev <= sms * (int)(224 * 1024 / per);
+        const size_t smem = fits ? inviter_smem(m) : 0;
+        const void* kern = fits ? (const void*)k_inviter<true> : (const void*)k_inviter<false>;
+        if ((st = allow_dynamic_smem(kern, smem, "heev_lowest: inverse iteration"))) return st;
+        ProfScope pf(PF_INVITER, s);
+        (fits ? k_inviter<true> : k_inviter<false>)<<<nev, 32, smem, s>>>(d, e, m, nev, evals, iw, wf, wsw);
     }
     {
         ProfScope pf(PF_INVITER, s);
-        k_inviter<<<nev, 32, 0, s>>>(d, e, m, nev, evals, iw);
-    }
-    {
-        ProfScope pf(PF_INVITER, s);
-        k_cluster_orth<<<nev, 256, 0, s>>>(d, e, m, nev, evals, iw, Y, ldy);
+        k_cluster_orth<<<nev, 256, 0, s>>>(d, e, m, nev, evals, iw, wf, wsw, Y, ldy);
     }
     {
         const size_t smem = (size_t)m * sizeof(double2);
         if ((st = allow_dynamic_smem((const void*)k_backtransf, smem, "heev_lowest: back-transformation"))) return st;
         ProfScope pf(PF_BACKTR, s);
-        k_backtransf<<<nev, 256, smem, s>>>(Vh, tau, m, Y, ldy);
+        if (m <= 64) k_backtransf_small<<<nev, 32, 0, s>>>(Vh, tau, m, Y, ldy);
+        else {
+            // a warp per 64 rows: a CTA's warps repeat every reduction, and FP64 instructions share one pipe
+            const int nt = std::min(256, (m + 63) / 64 * 32);
+            k_backtransf<<<nev, nt, smem, s>>>(Vh, tau, m, Y, ldy);
+        }
     }
     return cuda_check(cudaGetLastError(), "heev launches");
 }
