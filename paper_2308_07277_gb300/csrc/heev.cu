@@ -10,7 +10,7 @@
 //                     (k_tridiag: two barriers per column, for matrices beyond that).
 //                     (k_tridiag_small: one CTA, matrices up to kTriSmall.)
 //   2. k_multisect    the j-th smallest eigenvalue of T by multisection on Sturm counts
-//                     (Sec. 8.4.1): a warp tests 32 points per round, 12 rounds.
+//                     (Sec. 8.4.1): a CTA tests 128 points per round, 8 or 9 rounds.
 //   3. k_inviter      eigenvectors of T by inverse iteration (LU with partial pivoting of the
 //                     tridiagonal, three solves), one warp per eigenvalue; k_cluster_orth
 //                     then orthonormalises the vectors of each cluster of close eigenvalues
@@ -319,12 +319,13 @@ k_tridiag_rows(double2* __restrict__ A, int lda, int m, double2* __restrict__ Vh
 }
 
 // The reduction of a small matrix (m <= kTriSmall) in one CTA, the matrix in shared memory: a column of the
-// grid-wide reduction costs 8 us of barriers and launch-wide latency whatever its length.  The FP64 pipe
-// takes 16 cycles per warp instruction, so the work is laid out to need few of them: four threads per row in
-// the product A v (two shuffle steps instead of five), the rank-2 update on the lower triangle only, the
-// reflector's divisions once.  Warp 0 updates the next column first and builds its reflector (a root, a
-// division and two reductions in a chain) while the others update the rest.  Eight-band solves (m up to 32):
-// 115 us on average, 248 us with the grid-wide kernel.
+// grid-wide reduction costs 8 us of barriers and launch-wide latency whatever its length.  What bounds it is
+// the chain of FP64 instructions: each holds its warp and its partition's pipe for 64 cycles, independent or
+// not, and a root or a division is six to ten of them.  So the reflector stays unscaled (v = x - beta e_1,
+// tau = -1 / (beta conj(v_0))): the product A v needs only the root, and the division for tau runs on the
+// last warp beside it.  v^H A v is real, so the correction of w = tau A v is one real sum.  Warp 0 updates the
+// next column first and builds its reflector while the others update the rest (lower triangle, mirrored).
+// Eight-band solves (m up to 32): 80 us on average, 248 us with the grid-wide kernel.
 constexpr int kTriSmall = 64;
 __global__ void __launch_bounds__(256)
 k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restrict__ Vh, double2* __restrict__ tau,
@@ -332,40 +333,33 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
     extern __shared__ double2 smt[];
     const int ld = m + 1;
     double2 *a = smt, *vb = smt + m * ld, *w = vb + 2 * m;  // [m][ld], reflectors of two columns, product
-    __shared__ double2 s_t[2];
+    __shared__ double s_beta[2], s_half;  // beta (0: no reflection), -|tau|^2 / 2
+    __shared__ double2 s_t;
     const int tid = threadIdx.x, lane = tid & 31;
     for (int i = tid; i < m * m; i += 256) a[(i / m) * ld + i % m] = A[(size_t)(i / m) * lda + i % m];
-    // the reflector of column k (one warp)
+    // the reflector of column k but for tau (one warp)
     auto reflector = [&](int k) {
         const int n = m - k - 1;
         double2* v = vb + (k & 1) * m;
         double part = 0.0;
-        for (int i = 1 + lane; i < n; i += 32) {
+        bool below = false;  // anything to eliminate
+        for (int i = lane; i < n; i += 32) {
             const double2 x = a[(k + 1 + i) * ld + k];
-            part += x.x * x.x + x.y * x.y;
+            part = fma(x.x, x.x, fma(x.y, x.y, part));
+            below = below || x.y != 0.0 || (i > 0 && x.x != 0.0);
         }
         for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
         const double2 alpha = a[(k + 1) * ld + k];
-        double2 t = make_double2(0.0, 0.0), scale = make_double2(0.0, 0.0);
-        double beta = alpha.x;
-        if (part > 0.0 || alpha.y != 0.0) {
-            beta = -copysign(sqrt(alpha.x * alpha.x + alpha.y * alpha.y + part), alpha.x);
-            const double2 den = make_double2(alpha.x - beta, alpha.y);
-            // the two reciprocals on two lanes
-            const double inv = 1.0 / (lane & 1 ? den.x * den.x + den.y * den.y : beta);
-            const double ib = __shfl_sync(0xffffffffu, inv, 0), id = __shfl_sync(0xffffffffu, inv, 1);
-            t = make_double2((beta - alpha.x) * ib, -alpha.y * ib);
-            scale = make_double2(den.x * id, -den.y * id);
-        }
+        double beta = 0.0;
+        if (__any_sync(0xffffffffu, below) && part > 0.0) beta = -copysign(sqrt(part), alpha.x);
         for (int i = lane; i < n; i += 32) {
-            const double2 x = i ? cmul(a[(k + 1 + i) * ld + k], scale) : make_double2(1.0, 0.0);
+            double2 x = a[(k + 1 + i) * ld + k];
+            if (i == 0) x.x -= beta;
             v[i] = x;
-            Vh[(size_t)k * m + k + 1 + i] = x;
         }
         if (lane == 0) {
-            s_t[k & 1] = t;
-            tau[k] = t;
-            e[k] = beta;
+            s_beta[k & 1] = beta;
+            e[k] = beta != 0.0 ? beta : alpha.x;
             d[k] = a[k * ld + k].x;
         }
     };
@@ -375,10 +369,27 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
         __syncthreads();
         const int n = m - k - 1;
         double2* a22 = a + (k + 1) * ld + k + 1;
-        const double2 t = s_t[k & 1], *v = vb + (k & 1) * m;
-        const bool any = t.x != 0.0 || t.y != 0.0;  // (uniform)
+        const double2* v = vb + (k & 1) * m;
+        const double beta = s_beta[k & 1];
+        const bool any = beta != 0.0;  // (uniform)
+        if (tid >= 224) {
+            const double2 v0 = v[0];
+            double2 t = make_double2(0.0, 0.0);
+            if (any) {
+                // the two reciprocals on two lanes
+                const double inv = 1.0 / (lane & 1 ? fma(v0.x, v0.x, v0.y * v0.y) : beta);
+                const double ib = __shfl_sync(0xffffffffu, inv, 0), in = __shfl_sync(0xffffffffu, inv, 1);
+                t = make_double2(-(v0.x * in) * ib, -(v0.y * in) * ib);
+                if (lane == 0) {
+                    s_t = t;
+                    s_half = -0.5 * ib * (ib * in);
+                }
+            }
+            if (lane == 0) tau[k] = t;
+            for (int i = lane; i < n; i += 32) Vh[(size_t)k * m + k + 1 + i] = v[i];
+        }
         if (any) {
-            // w = t A22 v
+            // w = A22 v, four lanes a row; the pairs of lanes sum a component each
             for (int r0 = 0; r0 < n; r0 += 64) {
                 const int r = r0 + (tid >> 2);
                 double2 acc = make_double2(0.0, 0.0);
@@ -388,35 +399,28 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
                         acc.x = fma(x.x, y.x, fma(-x.y, y.y, acc.x));
                         acc.y = fma(x.x, y.y, fma(x.y, y.x, acc.y));
                     }
-#pragma unroll
-                for (int o = 1; o < 4; o <<= 1) {
-                    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-                    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+                if (r0 + ((tid & ~31) >> 2) < n) {  // (warps without a row skip the sums)
+                    const bool up = tid & 1;
+                    double h = (up ? acc.y : acc.x) + __shfl_xor_sync(0xffffffffu, up ? acc.x : acc.y, 1);
+                    h += __shfl_xor_sync(0xffffffffu, h, 2);
+                    if (r < n && (tid & 3) < 2) reinterpret_cast<double*>(w + r)[tid & 1] = h;
                 }
-                if (r < n && (tid & 3) == 0) w[r] = cmul(t, acc);
             }
             __syncthreads();
-            if (tid < 32) {  // w -= t (w^H v) / 2 v
-                double2 dp = make_double2(0.0, 0.0);
+            if (tid < 32) {  // w <- tau w - |tau|^2 (v^H w) / 2 v
+                double dp = 0.0;
+                for (int i = lane; i < n; i += 32) dp = fma(w[i].x, v[i].x, fma(w[i].y, v[i].y, dp));
+                for (int o = 16; o > 0; o >>= 1) dp += __shfl_xor_sync(0xffffffffu, dp, o);
+                const double g = s_half * dp;
+                const double2 t = s_t;
                 for (int i = lane; i < n; i += 32) {
-                    const double2 c = cmulc(w[i], v[i]);
-                    dp.x += c.x;
-                    dp.y += c.y;
-                }
-                for (int o = 16; o > 0; o >>= 1) {
-                    dp.x += __shfl_xor_sync(0xffffffffu, dp.x, o);
-                    dp.y += __shfl_xor_sync(0xffffffffu, dp.y, o);
-                }
-                const double2 a2 = cmul(make_double2(-0.5 * t.x, -0.5 * t.y), dp);
-                for (int i = lane; i < n; i += 32) {
-                    const double2 c = cmul(a2, v[i]);
-                    w[i].x += c.x;
-                    w[i].y += c.y;
+                    const double2 x = w[i], y = v[i];
+                    w[i] = make_double2(fma(t.x, x.x, fma(-t.y, x.y, g * y.x)), fma(t.x, x.y, fma(t.y, x.x, g * y.y)));
                 }
             }
             __syncthreads();
         }
-        // A22 -= v w^H + w v^H: lower triangle, mirrored
+        // A22 -= v w^H + w v^H
         auto update = [&](int i, int j) {
             const double2 vi = v[i], wi = w[i], vj = v[j], wj = w[j];
             double2 x = a22[i * ld + j];
@@ -446,11 +450,13 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
 
 // number of eigenvalues of T smaller than x: sign changes of the leading minors' determinants by their
 // three-term recurrence p_i = (d_i - x) p_(i-1) - e_(i-1)^2 p_(i-2) (Wilkinson, The Algebraic Eigenvalue
-// Problem, Ch. 5, Sec. 37), T scaled below 2 in magnitude.  (Eight-band solves: 66 us, 150 us with quotients.)  A ratio p_i / p_(i-1) below 2^-100 is replaced
+// Problem, Ch. 5, Sec. 37), T scaled below 2 in magnitude.
+// (Eight-band solves: 41 us, 150 us with
+// quotients and one warp.)  A ratio p_i / p_(i-1) below 2^-100 is replaced
 // by -2^-100 (a shift of d_i by less than 2^-99, and a zero counts as negative), so eight rows change the
 // pair by factors between 2^-900 and 2^40 and its rescaling every eight rows keeps it in range.  The
-// quotient form has a division in the chain of every row, about 450 cycles on this GPU's FP64 pipe; a
-// multiply-add is 45, and eight unrolled rows keep the loads and differences off the chain.
+// quotient form has a division in the chain of every row, about 430 cycles on this GPU; a
+// multiply-add is 64, and eight unrolled rows keep the loads and differences off the chain.
 __device__ __forceinline__ int sturm_count(const double* __restrict__ d, const double* __restrict__ e2, int m, double x) {
     int c = 0;
     double p0 = 1.0, p1 = d[0] - x;
@@ -462,7 +468,8 @@ __device__ __forceinline__ int sturm_count(const double* __restrict__ d, const d
             const int i = i0 + q;
             double p = fma(d[i] - x, p1, -e2[i - 1] * p0);
             const int hp = __double2hiint(p), h1 = __double2hiint(p1);
-            if ((hp & 0x7FF00000) < (h1 & 0x7FF00000) - (100 << 20)) p = -0x1p-100 * p1;
+            if ((hp & 0x7FF00000) < (h1 & 0x7FF00000) - (100 << 20))  // -2^-100 p1, without the FP64 pipe
+                p = __hiloint2double((h1 - (100 << 20)) ^ (int)0x80000000, __double2loint(p1));
             c += (int)((unsigned)(__double2hiint(p) ^ h1) >> 31);
             p0 = p1;
             p1 = p;
@@ -476,14 +483,17 @@ __device__ __forceinline__ int sturm_count(const double* __restrict__ d, const d
     return c;
 }
 
-// one warp (CTA) per wanted eigenvalue j < nev; d and e^2, scaled, in shared memory (2 (m + 8) doubles)
-__global__ void __launch_bounds__(32) k_multisect(const double* __restrict__ d, const double* __restrict__ e, int m, int nev,
+// one CTA per wanted eigenvalue j < nev, 128 points per round: a warp on each of the SM's four partitions (an
+// FP64 instruction holds a partition for 64 cycles, whatever its warp's lanes do); d and e^2, scaled, in
+// shared memory (2 (m + 8) doubles)
+__global__ void __launch_bounds__(128) k_multisect(const double* __restrict__ d, const double* __restrict__ e, int m, int nev,
                                                   double* __restrict__ evals) {
     extern __shared__ double sms[];
     double *sd = sms, *se = sms + m + 8;
-    const int j = blockIdx.x, lane = threadIdx.x;
+    const int j = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     if (j >= nev) return;
-    // Gershgorin interval
+    __shared__ int first[2][4];  // each warp's first point above eigenvalue j, rounds alternating
+    // Gershgorin interval (every warp)
     double lo = 1e300, hi = -1e300;
     for (int i = lane; i < m; i += 32) {
         const double r = (i > 0 ? fabs(e[i - 1]) : 0.0) + (i < m - 1 ? fabs(e[i]) : 0.0);
@@ -501,35 +511,31 @@ __global__ void __launch_bounds__(32) k_multisect(const double* __restrict__ d, 
     int ex = 0;
     frexp(fmax(fabs(lo), fabs(hi)), &ex);
     const double scale = ldexp(1.0, -ex), back = ldexp(1.0, ex);
-    for (int i = lane; i < m; i += 32) {
+    for (int i = tid; i < m; i += 128) {
         sd[i] = d[i] * scale;
         const double t = i < m - 1 ? e[i] * scale : 0.0;
         se[i] = t * t;
     }
-    if (lane < 8) {
-        sd[m + lane] = 4.0;
-        se[m + lane] = 0.0;
+    if (tid < 8) {
+        sd[m + tid] = 4.0;
+        se[m + tid] = 0.0;
     }
     lo *= scale;
     hi *= scale;
-    __syncwarp();
-    for (int round = 0; round < 14; ++round) {
-        const double x = lo + (hi - lo) * (double)(lane + 1) / 33.0;
-        const int c = sturm_count(sd, se, m, x);
+    __syncthreads();
+    for (int round = 0; round < 11; ++round) {
+        const auto point = [&](int q) { return fma(hi - lo, (double)(q + 1) * (1.0 / 129.0), lo); };
+        const int c = sturm_count(sd, se, m, point(tid));
         const unsigned above = __ballot_sync(0xffffffffu, c > j);
-        double nlo = lo, nhi = hi;
-        if (above) {
-            const int f = __ffs(above) - 1;
-            nhi = __shfl_sync(0xffffffffu, x, f);
-            if (f > 0) nlo = __shfl_sync(0xffffffffu, x, f - 1);
-        } else {
-            nlo = __shfl_sync(0xffffffffu, x, 31);
-        }
+        if (lane == 0) first[round & 1][tid >> 5] = above ? (tid & ~31) + __ffs(above) - 1 : 128;
+        __syncthreads();
+        const int *fr = first[round & 1], f = min(min(fr[0], fr[1]), min(fr[2], fr[3]));
+        const double nlo = f > 0 ? point(f - 1) : lo;
+        if (f < 128) hi = point(f);
         lo = nlo;
-        hi = nhi;
         if (hi - lo <= 4.0e-16 * fmax(fabs(lo), fabs(hi)) + 1e-300) break;
     }
-    if (lane == 0) evals[j] = 0.5 * (lo + hi) * back;
+    if (tid == 0) evals[j] = 0.5 * (lo + hi) * back;
 }
 
 // LU with partial pivoting of T - lam, T = tridiag(e, d, e): row i of U is (1 / r[i], c[i], c2[i]), the
@@ -778,37 +784,56 @@ k_backtransf(const double2* __restrict__ Vh, const double2* __restrict__ tau, in
     for (int i = tid; i < m; i += bs) Y[(size_t)i * ldy + j] = sy[i];
 }
 
-// the same for m <= 64: one warp per column, the column in registers (rows lane and lane + 32), the next
-// reflector loaded while the present one is applied
+// the same for m <= 32 kRows: one warp per column, the column in registers (rows lane, lane + 32), the next
+// reflector loaded while the present one is applied.  Bound by the chain of FP64 instructions, 64 cycles
+// each: the two components of the dot product are summed by half a warp each.  Eight-band solves: 21 us, 74 us
+// with the general kernel.
+template <int kRows>
 __global__ void __launch_bounds__(32)
 k_backtransf_small(const double2* __restrict__ Vh, const double2* __restrict__ tau, int m, double2* __restrict__ Y, int ldy) {
-    const int j = blockIdx.x, r0 = threadIdx.x, r1 = r0 + 32;
+    const int j = blockIdx.x, lane = threadIdx.x;
+    const bool upper = lane >= 16;
     const double2 z = make_double2(0.0, 0.0);
-    double2 y0 = r0 < m ? Y[(size_t)r0 * ldy + j] : z, y1 = r1 < m ? Y[(size_t)r1 * ldy + j] : z;
-    auto ref = [&](int k, int r) { return k >= 0 && r > k && r < m ? Vh[(size_t)k * m + r] : z; };
-    double2 v0 = ref(m - 2, r0), v1 = ref(m - 2, r1), t = tau[m - 2];
-    for (int k = m - 2; k >= 0; --k) {
-        const double2 n0 = ref(k - 1, r0), n1 = ref(k - 1, r1), nt = k > 0 ? tau[k - 1] : z;
-        if (t.x != 0.0 || t.y != 0.0) {
-            const double2 c0 = cmulc(v0, y0), c1 = cmulc(v1, y1);
-            double2 sp = make_double2(c0.x + c1.x, c0.y + c1.y);
+    double2 y[kRows], v[kRows], nv[kRows];
+    const auto ref = [&](int k, int r) { return k >= 0 && r > k && r < m ? Vh[(size_t)k * m + r] : z; };
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                sp.x += __shfl_xor_sync(0xffffffffu, sp.x, o);
-                sp.y += __shfl_xor_sync(0xffffffffu, sp.y, o);
+    for (int q = 0; q < kRows; ++q) {
+        const int r = lane + 32 * q;
+        y[q] = r < m ? Y[(size_t)r * ldy + j] : z;
+        v[q] = ref(m - 2, r);
+    }
+    double2 t = tau[m - 2];
+    for (int k = m - 2; k >= 0; --k) {
+#pragma unroll
+        for (int q = 0; q < kRows; ++q) nv[q] = ref(k - 1, lane + 32 * q);
+        const double2 nt = k > 0 ? tau[k - 1] : z;
+        if (t.x != 0.0 || t.y != 0.0) {
+            double2 sp = cmulc(v[0], y[0]);
+#pragma unroll
+            for (int q = 1; q < kRows; ++q) {
+                sp.x = fma(v[q].x, y[q].x, fma(v[q].y, y[q].y, sp.x));
+                sp.y = fma(v[q].x, y[q].y, fma(-v[q].y, y[q].x, sp.y));
             }
-            const double2 s = cmul(t, sp), u0 = cmul(v0, s), u1 = cmul(v1, s);
-            y0.x -= u0.x;
-            y0.y -= u0.y;
-            y1.x -= u1.x;
-            y1.y -= u1.y;
+            double h = (upper ? sp.y : sp.x) + __shfl_xor_sync(0xffffffffu, upper ? sp.x : sp.y, 16);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+            // s = t (v^H y), a component per half
+            const double other = __shfl_xor_sync(0xffffffffu, h, 16);
+            const double sh = fma(t.x, h, (upper ? t.y : -t.y) * other);
+            const double2 s = make_double2(__shfl_sync(0xffffffffu, sh, 0), __shfl_sync(0xffffffffu, sh, 16));
+#pragma unroll
+            for (int q = 0; q < kRows; ++q) {
+                y[q].x = fma(-v[q].x, s.x, fma(v[q].y, s.y, y[q].x));
+                y[q].y = fma(-v[q].x, s.y, fma(-v[q].y, s.x, y[q].y));
+            }
         }
-        v0 = n0;
-        v1 = n1;
+#pragma unroll
+        for (int q = 0; q < kRows; ++q) v[q] = nv[q];
         t = nt;
     }
-    if (r0 < m) Y[(size_t)r0 * ldy + j] = y0;
-    if (r1 < m) Y[(size_t)r1 * ldy + j] = y1;
+#pragma unroll
+    for (int q = 0; q < kRows; ++q)
+        if (lane + 32 * q < m) Y[(size_t)(lane + 32 * q) * ldy + j] = y[q];
 }
 
 }  // namespace
@@ -940,7 +965,7 @@ qm_status heev_lowest(double2* A, int lda, int m, int nev, double* evals, double
         const size_t smem = 2 * (size_t)(m + 8) * sizeof(double);
         if ((st = allow_dynamic_smem((const void*)k_multisect, smem, "heev_lowest: multisection"))) return st;
         ProfScope pf(PF_MULTISECT, s);
-        k_multisect<<<nev, 32, smem, s>>>(d, e, m, nev, evals);
+        k_multisect<<<nev, 128, smem, s>>>(d, e, m, nev, evals);
     }
     {
         // shared memory while every eigenvalue's CTA is resident at once (1 KB of it is the system's)
@@ -963,7 +988,8 @@ qm_status heev_lowest(double2* A, int lda, int m, int nev, double* evals, double
         const size_t smem = (size_t)m * sizeof(double2);
         if ((st = allow_dynamic_smem((const void*)k_backtransf, smem, "heev_lowest: back-transformation"))) return st;
         ProfScope pf(PF_BACKTR, s);
-        if (m <= 64) k_backtransf_small<<<nev, 32, 0, s>>>(Vh, tau, m, Y, ldy);
+        if (m <= 32) k_backtransf_small<1><<<nev, 32, 0, s>>>(Vh, tau, m, Y, ldy);
+        else if (m <= 64) k_backtransf_small<2><<<nev, 32, 0, s>>>(Vh, tau, m, Y, ldy);
         else {
             // a warp per 64 rows: a CTA's warps repeat every reduction, and FP64 instructions share one pipe
             const int nt = std::min(256, (m + 63) / 64 * 32);

@@ -268,9 +268,9 @@ k_cn(int M, int N, int K, const C* __restrict__ A, int lda, const C* __restrict_
     }
 }
 
-constexpr int kTnM = 8, kTnN = 32, kTnK = 16;
-template <class T>
-__global__ void __launch_bounds__(NTH)
+constexpr int kTnN = 32, kTnK = 16;
+template <class T, int kTnM>  // a warp per row
+__global__ void __launch_bounds__(32 * kTnM)
 k_tn(int M, int N, int K, const T* __restrict__ A, int lda, const double* __restrict__ d, double alpha,
      const T* __restrict__ B, int ldb, T* __restrict__ C, int ldc, int accumulate, const GemmFlags f) {
     if (f.any && !*f.any) return;
@@ -291,12 +291,12 @@ k_tn(int M, int N, int K, const T* __restrict__ A, int lda, const double* __rest
             As[kk][tid % kTnM] = v;
         }
 #pragma unroll
-        for (int q = 0; q < kTnK * kTnN / NTH; ++q) {
-            const int kk = ty + q * (NTH / kTnN), k = k0 + kk, n = n0 + tx;
+        for (int q = 0; q < kTnK / kTnM; ++q) {
+            const int kk = ty + q * kTnM, k = k0 + kk, n = n0 + tx;
             Bs[kk][tx] = (k < K && n < N) ? B[(size_t)k * ldb + n] : czero<T>();
         }
         __syncthreads();
-        const int kn = min(kTnK, K - k0);
+        const int kn = m0 + ty < M ? min(kTnK, K - k0) : 0;  // (warps past the last row leave the FP64 pipe alone)
         for (int kk = 0; kk < kn; ++kk) {
             const T a = As[kk][ty], b = Bs[kk][tx];
             acc.x = fma(a.x, b.x, fma(-a.y, b.y, acc.x));
@@ -357,8 +357,15 @@ template <class T>
 qm_status tn_small(int M, int N, int K, const T* A, int lda, const double* d, double alpha, const T* B, int ldb, T* C,
                    int ldc, bool accumulate, const GemmFlags& f, cudaStream_t s) {
     ProfScope pf(PF_GEMM_TN, s);
-    const dim3 grid((N + kTnN - 1) / kTnN, (M + kTnM - 1) / kTnM);
-    k_tn<T><<<grid, NTH, 0, s>>>(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate ? 1 : 0, f);
+    // Rows per CTA, 8 or 4, in FP64: a warp's FP64 instruction holds one of the SM's four partitions, so eight
+    // rows take twice the time of four and are worth it only where the tiles fill the SMs that often anyway
+    // (8 x 1500 outputs, K up to 32: 5.2 us with 4 rows on 94 SMs, 6.9 us with 8 on 47)
+    const auto tiles = [&](int rows) { return (long)((N + kTnN - 1) / kTnN) * ((M + rows - 1) / rows); };
+    const long sms = device_sms(), load8 = (tiles(8) + sms - 1) / sms * 2, load4 = (tiles(4) + sms - 1) / sms;
+    const int rows = sizeof(T) == sizeof(double2) && load4 < load8 ? 4 : 8;
+    const dim3 grid((N + kTnN - 1) / kTnN, (M + rows - 1) / rows);
+    if (rows == 4) k_tn<T, 4><<<grid, 128, 0, s>>>(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate ? 1 : 0, f);
+    else k_tn<T, 8><<<grid, 256, 0, s>>>(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate ? 1 : 0, f);
     return cuda_check(cudaGetLastError(), "gemm_tn launch");
 }
 
