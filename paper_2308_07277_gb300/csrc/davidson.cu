@@ -131,34 +131,25 @@ __global__ void __launch_bounds__(256) k_hdiag(const double* __restrict__ kin, i
     hdiag[g] = kin[g] + vmean + nl;
 }
 
-// Hermitian completion after new columns [m0, m) of H were computed for rows [0, m):
-// H[j][i] = conj(H[i][j]) for i < m0 <= j; the new diagonal block is symmetrised.
-__global__ void k_herm_fill(double2* __restrict__ H, int ld, int m0, int m) {
-    const int nn = m - m0;
-    const long total = (long)m * nn;
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
-        const int i = (int)(e / nn), j = m0 + (int)(e % nn);
-        if (i < m0) {
-            double2 v = H[(size_t)i * ld + j];
-            H[(size_t)j * ld + i] = make_double2(v.x, -v.y);
-        } else if (i < j) {
-            double2 a = H[(size_t)i * ld + j], b = H[(size_t)j * ld + i];
-            double2 h = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
-            H[(size_t)i * ld + j] = h;
-            H[(size_t)j * ld + i] = make_double2(h.x, -h.y);
-        } else if (i == j) {
-            H[(size_t)i * ld + i].y = 0.0;
-        }
-    }
-}
-
-// A[i][j] = Hermitian part of H (m x m)
-__global__ void k_herm_copy(const double2* __restrict__ H, int ldh, int m, double2* __restrict__ A, int lda) {
+// the new columns j >= m0 of the Hermitian H (m x m): column part below m0 mirrored, the square beyond
+// averaged with its mirror, the diagonal real; and a copy of the whole of H for the eigensolver
+__global__ void k_herm_fill(double2* __restrict__ H, int ld, int m0, int m, double2* __restrict__ A, int lda) {
     const long total = (long)m * m;
     for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
         const int i = (int)(e / m), j = (int)(e % m);
-        const double2 a = H[(size_t)i * ldh + j], b = H[(size_t)j * ldh + i];
-        A[(size_t)i * lda + j] = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
+        if (i > j) continue;
+        double2 h = H[(size_t)i * ld + j];
+        if (i >= m0 || j < m0) {
+            const double2 b = H[(size_t)j * ld + i];
+            h = make_double2(0.5 * (h.x + b.x), 0.5 * (h.y - b.y));
+        }
+        const double2 c = make_double2(h.x, -h.y);
+        if (j >= m0) {
+            H[(size_t)i * ld + j] = h;
+            H[(size_t)j * ld + i] = c;
+        }
+        A[(size_t)i * lda + j] = h;
+        A[(size_t)j * lda + i] = c;
     }
 }
 
@@ -534,8 +525,8 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
                  oQT = take(thick ? sqb : 0), oY = take(thick ? big * nb : 0), oHY = take(thick ? big * nb : 0);
     const size_t part_bytes = std::max(gemm_cn_partial_bytes(false), std::max(zgemm_cn_bytes(nvx, nvx, npw), zgemm_tn_bytes(nvx, npw, nvx)));
     const size_t oPart = take(part_bytes);
-    const size_t oEval = take(sizeof(double) * nsq), oEps = take(sizeof(double) * nsq),
-                 oRn = take(sizeof(double) * nsq), oTk = take(sizeof(double) * nsq),
+    const size_t oEval = take(sizeof(double) * nsq), oEps = take(sizeof(double) * (nsq + nb)),
+                 oTk = take(sizeof(double) * nsq),
                  oSel = take(sizeof(int) * nsq), oRank = take(sizeof(int) * nsq), oInfo = take(sizeof(int) * 4),
                  oHeev = take(heev_work_bytes(nsq, nsq));
     const size_t oHd = take(o.precond == 1 ? sizeof(double) * npw : 0),
@@ -581,7 +572,7 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
     }
     w.eval = (double*)(base + oEval);
     w.eps = (double*)(base + oEps);
-    w.rn2 = (double*)(base + oRn);
+    w.rn2 = w.eps + nsq;  // beside the Ritz values: one copy brings both back
     w.tk = (double*)(base + oTk);
     w.sel = (int*)(base + oSel);
     w.rank = (int*)(base + oRank);
@@ -620,7 +611,8 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
     // the network's features need the Hamiltonian's diagonal (once per solve)
     if (use_mlp && (st = hamiltonian_diag(g, ik, vloc_r, nproj, (const double2*)beta, ld_beta, D, w.hdiag, w.vpart, s)))
         return st;
-    std::vector<double> rn2(nb), eps(nb);
+    std::vector<double> back(nsq + nb);
+    const double *eps = back.data(), *rn2 = eps + nsq;
     int it = 0, it_mixed = 0, restarts = 0;
     long long prev_kept = 0;
     std::vector<double> hist_mixed;
@@ -664,10 +656,8 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
             ProfScope pf(PF_OTHER, s);
             k_residual<<<nb, 256, 0, s>>>(w.X, w.HX, ld, npw, w.eps, kin, w.R, w.rn2, w.tk);
         }
-        if ((st2 = cuda_check(cudaMemcpyAsync(rn2.data(), w.rn2, sizeof(double) * nb, cudaMemcpyDeviceToHost, s),
-                              "D2H residual norms")) ||
-            (st2 = cuda_check(cudaMemcpyAsync(eps.data(), w.eps, sizeof(double) * nb, cudaMemcpyDeviceToHost, s),
-                              "D2H Ritz values")) ||
+        if ((st2 = cuda_check(cudaMemcpyAsync(back.data(), w.eps, sizeof(double) * back.size(), cudaMemcpyDeviceToHost, s),
+                              "D2H Ritz values, residual norms")) ||
             (st2 = cuda_check(cudaStreamSynchronize(s), "stream sync")))
             return st2;
         for (int n = 0; n < nb; ++n)
@@ -698,11 +688,7 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
         }
         {
             ProfScope pf(PF_OTHER, s);
-            k_herm_fill<<<grid_for((long)m * (m - m0)), 256, 0, s>>>(w.Hs, nsq, m0, m);
-        }
-        {
-            ProfScope pf(PF_OTHER, s);
-            k_herm_copy<<<grid_for((long)m * m), 256, 0, s>>>(w.Hs, nsq, m, w.A, m);
+            k_herm_fill<<<grid_for((long)m * m), 256, 0, s>>>(w.Hs, nsq, m0, m, w.A, m);
         }
         // lowest nb eigenpairs: values -> eps (device, increasing), vectors -> Cs [m][nb]
         if ((st = heev_lowest(w.A, m, m, nb, w.eps, w.Cs, nb, w.heev, s))) return st;

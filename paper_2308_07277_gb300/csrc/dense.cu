@@ -36,7 +36,8 @@ k_chol_diag(double2* __restrict__ S, int lds, int k0, int nb, const double* __re
     if (ty < nb && tx <= ty) a[ty][tx] = S[(size_t)(k0 + ty) * lds + k0 + tx];
     __syncthreads();
     // (the pivot's root and reciprocal are taken by one warp: a warp's FP64 instruction holds
-    // its partition's pipe for 64 cycles, and a square root and a division are about 16 of them; 8 columns: 7 us, 35 us with every warp's own)
+    // its partition's pipe for 64 cycles, and a square root and a division are about 16 of them; 8 columns: 7 us,
+    // 35 us with every warp's own)
     for (int j = 0; j < nb; ++j) {
         if (ty == j) {
             const double piv = a[j][j].x;
@@ -208,6 +209,69 @@ k_trinv_small(const double2* __restrict__ L, int lds, int nd, const int* __restr
     if (kept) W[(size_t)c * ldw + rank[i]] = i < c ? make_double2(0.0, 0.0) : make_double2(x.x, -x.y);
 }
 
+// factor, ranks and transform of a block of nd <= kFused in one launch, everything in shared memory: warp i
+// holds row i for the factorisation (as k_chol_diag) and column i of L^-1 after it (as k_trinv_small).
+// Beyond 16 the columns' instructions on one SM take longer than a launch each (nd^2 / 4 x 6 of 64 cycles on
+// each of the four partitions: 6 us at 16, against 3 us and the gap of a launch on many SMs).  With nothing
+// kept, W is not written.  8 rows: 9 us for one launch, 14.5 us for four.
+constexpr int kFused = 16;
+__global__ void __launch_bounds__(32 * kFused)
+k_chol_small(const double2* __restrict__ S, int lds, int nd, double drop_rel, int* __restrict__ keep, int* __restrict__ rank,
+             int* __restrict__ kept_dev, double2* __restrict__ W) {
+    __shared__ double2 a[kFused][kFused + 1];
+    __shared__ double orig[kFused];
+    __shared__ int skeep[kFused];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // column, row
+    if (tx <= ty) {
+        a[ty][tx] = S[(size_t)ty * lds + tx];
+        if (tx == ty) orig[ty] = a[ty][ty].x;
+    }
+    __syncthreads();
+    for (int j = 0; j < nd; ++j) {
+        if (ty == j) {
+            const double piv = a[j][j].x;
+            const bool ok = piv > drop_rel * orig[j] && piv > 0.0 && isfinite(piv);
+            const double root = ok ? sqrt(piv) : 0.0, il = ok ? 1.0 / root : 0.0;
+            __syncwarp();
+            if (tx == 0) {
+                a[j][j] = make_double2(root, 0.0);
+                skeep[j] = ok ? 1 : 0;
+            }
+            const int i = j + 1 + tx;
+            if (i < nd) a[i][j] = make_double2(a[i][j].x * il, a[i][j].y * il);
+        }
+        __syncthreads();
+        if (ty > j && tx > j && tx <= ty) {
+            const double2 p = a[ty][j], q = a[tx][j];
+            a[ty][tx].x -= p.x * q.x + p.y * q.y;
+            a[ty][tx].y -= p.y * q.x - p.x * q.y;
+        }
+        __syncthreads();
+    }
+    const bool mine = tx < nd && skeep[tx];
+    const unsigned mask = __ballot_sync(0xffffffffu, mine);
+    const int ldw = __popc(mask), rk = __popc(mask & ((1u << tx) - 1u));
+    if (ty == 0 && tx < nd) {
+        keep[tx] = mine ? 1 : 0;
+        rank[tx] = mine ? rk : -1;
+        if (tx == 0) *kept_dev = ldw;
+    }
+    const int c = ty;
+    const double inv = mine && tx >= c ? 1.0 / a[tx][tx].x : 0.0;
+    double2 x = make_double2(tx == c ? 1.0 : 0.0, 0.0);
+    for (int j = c; j < nd; ++j) {
+        const double f = __shfl_sync(0xffffffffu, inv, j);
+        const double2 xj = make_double2(__shfl_sync(0xffffffffu, x.x, j) * f, __shfl_sync(0xffffffffu, x.y, j) * f);
+        if (tx == j) x = xj;
+        if (tx > j && tx < nd) {
+            const double2 l = a[tx][j];
+            x.x = fma(-l.x, xj.x, fma(l.y, xj.y, x.x));
+            x.y = fma(-l.x, xj.y, fma(-l.y, xj.x, x.y));
+        }
+    }
+    if (mine) W[(size_t)c * ldw + rk] = tx < c ? make_double2(0.0, 0.0) : make_double2(x.x, -x.y);
+}
+
 __global__ void k_rank(const int* __restrict__ keep, int nd, int* __restrict__ rank, int* __restrict__ kept) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         int r = 0;
@@ -228,6 +292,11 @@ __global__ void k_rank(const int* __restrict__ keep, int nd, int* __restrict__ r
 qm_status chol_transform(double2* S, int lds, int nd, double drop_rel, int* keep, int* rank, int* kept_dev,
                          double2* X, double2* W, int ldw_max, cudaStream_t s) {
     (void)ldw_max;
+    if (nd <= kFused) {
+        ProfScope pf(PF_CHOL, s);
+        k_chol_small<<<1, 32 * nd, 0, s>>>(S, lds, nd, drop_rel, keep, rank, kept_dev, W);
+        return cuda_check(cudaGetLastError(), "k_chol_small launch");
+    }
     double* orig = reinterpret_cast<double*>(X);  // the scratch X is free until chol_transform_rows
     {
         ProfScope pf(PF_CHOL, s);
@@ -261,6 +330,7 @@ qm_status chol_transform(double2* S, int lds, int nd, double drop_rel, int* keep
 // second half, once kept is known on the host: W (nd x kept)
 qm_status chol_transform_rows(const double2* L, int lds, int nd, const int* keep, const int* rank, int kept,
                               double2* X, double2* W, cudaStream_t s) {
+    if (nd <= kFused) return QM_OK;  // W is there already
     ProfScope pf(PF_CHOL, s);
     if (nd <= 32) k_trinv_small<<<nd, 32, 0, s>>>(L, lds, nd, keep, rank, W, kept);
     else k_trinv_rows<<<nd, 32, 0, s>>>(L, lds, nd, keep, rank, kept, X, nd, W, kept);
