@@ -62,7 +62,7 @@ struct Workspace {
 };
 
 // Projectors of one k-point prepared for the precision form's tensor-core nonlocal part
-// (qm_hpsi_prepare): the BF16 planes of beta in both GEMM layouts, for calls that pass the same
+// (qm_hpsi_prepare): the FP16 planes of beta in both GEMM layouts, for calls that pass the same
 // (beta, ld, nproj).
 struct NlPrep {
     const void* beta = nullptr;
