@@ -45,10 +45,6 @@ constexpr long kSpin = 1L << 26;
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 __device__ __forceinline__ float sigm(float z) { return 1.f / (1.f + expf(-z)); }
 __device__ __forceinline__ float silu(float z) { return z * sigm(z); }
-__device__ __forceinline__ float silu_d(float z) {
-    const float s = sigm(z);
-    return s * (1.f + z * (1.f - s));
-}
 __device__ __forceinline__ float softplus(float z) { return fmaxf(z, 0.f) + log1pf(expf(-fabsf(z))); }
 constexpr float kInvLog2 = 1.44269504088896340736f;  // 1 / log 2
 // Teter-Payne-Allan factor (27+18x+12x^2+8x^3)/(27+18x+12x^2+8x^3+16x^4) (Phys. Rev. B 40, 12255)
@@ -250,10 +246,15 @@ int infer_grid(long ntiles) {
 // dw3 and db3 are per-tile column sums on the CUDA cores.  dz2 and dz1 are rounded to BF16
 // before their products, like every other operand.
 constexpr int kGN3 = 80;                             // N of MMA3
-constexpr int kGStride = kH + 1;                     // padded row of h2 (floats, odd: no bank conflicts)
+constexpr int kGStride = kH + 2;                     // padded row of h2 (BF16; 33 words: no bank conflicts)
 constexpr uint32_t kIdesc3 = tc::idesc_bf16(128, kGN3);
-constexpr size_t kGradSmem = 2 * 16384 + 2 * 8192 + 32768 + 20480 + sizeof(float) * (kMT * kGStride + kMT + kH * 3 +
-                                                                                    3 * kH + 4);
+// A CTA's four warps are one per scheduler and wait on each other's chains (activations, three products and
+// six barriers a tile); two CTAs per SM, 104 KB and half of the tensor memory each, fill the gaps.  To fit,
+// h1 and dz2 share one operand buffer (the first product is complete before dz2 is written) and h2 is kept in
+// the BF16 that it is rounded to.  The derivatives of both activations are taken with their values (one
+// exponential and one division instead of two) and stay in registers.  300k samples: GRADUS us, 469 us with one
+// CTA per SM and separate derivatives.
+constexpr size_t kGradSmem = 16384 + 2 * 8192 + 32768 + 20480 + 2 * kMT * kGStride + sizeof(float) * (kMT + kH * 3 + 3 * kH + 4);
 
 // byte offset of element (row, k) of a K-major no-swizzle operand with 128 K columns
 __device__ __forceinline__ int cm_off128(int row, int k) {
@@ -301,19 +302,18 @@ __device__ __forceinline__ void to_async_proxy_and_sync() {
 // Cosine-loss gradient of every tile of the CTA (grid-stride), given per-band coefficients:
 // per-CTA partials to gpart[blockIdx.x][kNP].  128 threads; a bounded wait that expires sets
 // *err and ends the CTA (its partials are then not written).
-__global__ void __launch_bounds__(kMT, 1)
+__global__ void __launch_bounds__(kMT, 2)
 k_mlp_grad(long n, const float* __restrict__ feats, const float* __restrict__ theta, const int* __restrict__ band_of,
            const float* __restrict__ r2, const float* __restrict__ cc, const float* __restrict__ coef,
            const float* __restrict__ ratio, float* __restrict__ gpart, int* __restrict__ err) {
     extern __shared__ __align__(1024) unsigned char dsm[];
-    unsigned char* sA1 = dsm;              // h1, 128 x 64
-    unsigned char* sA2 = sA1 + 16384;      // dz2, 128 x 64
-    unsigned char* sW2 = sA2 + 16384;      // W2 as the B operand of MMA1 (rows j, K = i)
+    unsigned char* sA = dsm;               // h1, then dz2, 128 x 64
+    unsigned char* sW2 = sA + 16384;       // W2 as the B operand of MMA1 (rows j, K = i)
     unsigned char* sW2t = sW2 + 8192;      // W2^T as the B operand of MMA2 (rows i, K = j)
     unsigned char* sA3 = sW2t + 8192;      // Amat of MMA3, 128 x 128
     unsigned char* sB3 = sA3 + 32768;      // Bmat of MMA3, 80 x 128
-    float* sH2 = reinterpret_cast<float*>(sB3 + 20480);  // h2 [sample][kGStride]
-    float* sDz3 = sH2 + kMT * kGStride;
+    __nv_bfloat16* sH2 = reinterpret_cast<__nv_bfloat16*>(sB3 + 20480);  // h2 [sample][kGStride]
+    float* sDz3 = reinterpret_cast<float*>(sH2 + kMT * kGStride);
     float* sW1 = sDz3 + kMT;
     float* sb1 = sW1 + kH * 3;
     float* sb2 = sb1 + kH;
@@ -352,7 +352,7 @@ k_mlp_grad(long n, const float* __restrict__ feats, const float* __restrict__ th
     const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
     const uint32_t mb = tc::smem_u32(&mbar);
     uint32_t phase = 0;
-    float gw3 = 0.f;  // thread j < 64: dw3[j]; thread 64: db3
+    float gw3 = 0.f, gb3 = 0.f;  // thread: dw3[tid & 63] of half of each tile's samples; db3 of its own samples
     bool aborted = false;
     int tiles = 0;
     const long nt = (n + kMT - 1) / kMT;
@@ -370,22 +370,25 @@ k_mlp_grad(long n, const float* __restrict__ feats, const float* __restrict__ th
         f[1] = bf16r(f[1]);
         f[2] = bf16r(f[2]);
         // layer 1: h1 row of this sample into MMA1's A operand and column `tid` of Bmat
+        float g1[kH];  // silu'(z1)
 #pragma unroll
         for (int kc = 0; kc < kH / 8; ++kc) {
             float h[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 const int j = kc * 8 + q;
-                h[q] = bf16r(silu(sb1[j] + sW1[3 * j] * f[0] + sW1[3 * j + 1] * f[1] + sW1[3 * j + 2] * f[2]));
+                const float z = sb1[j] + sW1[3 * j] * f[0] + sW1[3 * j + 1] * f[1] + sW1[3 * j + 2] * f[2], sg = sigm(z);
+                h[q] = bf16r(z * sg);
+                g1[j] = sg * (1.f + z * (1.f - sg));
                 put_bf16(sB3, cm_off128(j, tid), h[q]);
             }
-            *reinterpret_cast<uint4*>(sA1 + cm_off(tid, kc * 8)) =
+            *reinterpret_cast<uint4*>(sA + cm_off(tid, kc * 8)) =
                 make_uint4(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]), pack_bf16(h[4], h[5]), pack_bf16(h[6], h[7]));
         }
 #pragma unroll
         for (int k = 0; k < 3; ++k) put_bf16(sB3, cm_off128(65 + k, tid), f[k]);
         to_async_proxy_and_sync();
-        if (tid == 0) mma_issue(tmem, tc::smem_u32(sA1), tc::smem_u32(sW2), 1024, kH / 16, kIdesc, false, mb);
+        if (tid == 0) mma_issue(tmem, tc::smem_u32(sA), tc::smem_u32(sW2), 1024, kH / 16, kIdesc, false, mb);
         bool ok = tc::mbar_wait(mb, phase, kSpin);
         phase ^= 1u;
         if (!__syncthreads_and(ok)) {
@@ -394,16 +397,22 @@ k_mlp_grad(long n, const float* __restrict__ feats, const float* __restrict__ th
         }
         asm volatile("tcgen05.fence::after_thread_sync;\n");
         // layer 2 and output from z2 - b2 (tensor memory columns 0..63)
-        float z3 = *sb3;
+        float z3 = *sb3, g2[kH];  // silu'(z2)
 #pragma unroll
         for (int c0 = 0; c0 < kH; c0 += 16) {
             uint32_t v[16];
             tmem_ld16(tmem + lane_off + (uint32_t)c0, v);
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const float h2 = bf16r(silu(__uint_as_float(v[q]) + sb2[c0 + q]));
-                sH2[tid * kGStride + c0 + q] = h2;
-                z3 += sw3[c0 + q] * h2;
+            for (int q = 0; q < 16; q += 2) {
+                float h2[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const float z = __uint_as_float(v[q + u]) + sb2[c0 + q + u], sg = sigm(z);
+                    h2[u] = bf16r(z * sg);
+                    g2[c0 + q + u] = sg * (1.f + z * (1.f - sg));
+                    z3 += sw3[c0 + q + u] * h2[u];
+                }
+                *reinterpret_cast<uint32_t*>(sH2 + tid * kGStride + c0 + q) = pack_bf16(h2[0], h2[1]);
             }
         }
         float dz3 = 0.f;
@@ -413,33 +422,30 @@ k_mlp_grad(long n, const float* __restrict__ feats, const float* __restrict__ th
             dz3 = coef[b] * (ratio[b] * K * r2[s] - cc[s]) * t * sigm(z3);
         }
         sDz3[tid] = dz3;
+        gb3 += dz3;
         // dz2 = dz3 w3 silu'(z2): A operand of MMA2 (row tid) and rows 0..63 of Amat (column tid)
 #pragma unroll
         for (int c0 = 0; c0 < kH; c0 += 16) {
-            uint32_t v[16];
-            tmem_ld16(tmem + lane_off + (uint32_t)c0, v);
             float d[16];
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
-                d[q] = bf16r(dz3 * sw3[c0 + q] * silu_d(__uint_as_float(v[q]) + sb2[c0 + q]));
+                d[q] = bf16r(dz3 * sw3[c0 + q] * g2[c0 + q]);
                 put_bf16(sA3, cm_off128(c0 + q, tid), d[q]);
             }
 #pragma unroll
             for (int h = 0; h < 2; ++h)
-                *reinterpret_cast<uint4*>(sA2 + cm_off(tid, c0 + 8 * h)) =
+                *reinterpret_cast<uint4*>(sA + cm_off(tid, c0 + 8 * h)) =
                     make_uint4(pack_bf16(d[8 * h], d[8 * h + 1]), pack_bf16(d[8 * h + 2], d[8 * h + 3]),
                                pack_bf16(d[8 * h + 4], d[8 * h + 5]), pack_bf16(d[8 * h + 6], d[8 * h + 7]));
         }
         to_async_proxy_and_sync();
-        if (tid == 0) mma_issue(tmem + 64, tc::smem_u32(sA2), tc::smem_u32(sW2t), 1024, kH / 16, kIdesc, false, mb);
-        // dw3, db3 of this tile while the tensor core works (h2 and dz3 are complete)
-        if (tid < kH) {
+        if (tid == 0) mma_issue(tmem + 64, tc::smem_u32(sA), tc::smem_u32(sW2t), 1024, kH / 16, kIdesc, false, mb);
+        // dw3 of this tile while the tensor core works (h2 and dz3 are complete)
+        {
+            const int j = tid & 63, q0 = tid & 64;
             float a = 0.f;
-            for (int q = 0; q < kMT; ++q) a += sDz3[q] * sH2[q * kGStride + tid];
-            gw3 += a;
-        } else if (tid == kH) {
-            float a = 0.f;
-            for (int q = 0; q < kMT; ++q) a += sDz3[q];
+#pragma unroll 8
+            for (int q = q0; q < q0 + 64; ++q) a += sDz3[q] * __bfloat162float(sH2[q * kGStride + j]);
             gw3 += a;
         }
         ok = tc::mbar_wait(mb, phase, kSpin);
@@ -457,8 +463,7 @@ k_mlp_grad(long n, const float* __restrict__ feats, const float* __restrict__ th
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
                 const int i = c0 + q;
-                const float z1 = sb1[i] + sW1[3 * i] * f[0] + sW1[3 * i + 1] * f[1] + sW1[3 * i + 2] * f[2];
-                put_bf16(sA3, cm_off128(64 + i, tid), __uint_as_float(v[q]) * silu_d(z1));
+                put_bf16(sA3, cm_off128(64 + i, tid), __uint_as_float(v[q]) * g1[i]);
             }
         }
         to_async_proxy_and_sync();
@@ -499,8 +504,13 @@ k_mlp_grad(long n, const float* __restrict__ feats, const float* __restrict__ th
                     }
                 }
             }
-            if (tid < kH) g[kOffW3 + tid] = gw3;
-            if (tid == kH) g[kOffB3] = gw3;
+            // the halves of dw3 and the threads' db3 (every warp is past its reads of sDz3)
+            if (tid >= kH) sDz3[tid] = gw3;
+            for (int o = 16; o > 0; o >>= 1) gb3 += __shfl_xor_sync(0xffffffffu, gb3, o);
+            if ((tid & 31) == 0) sDz3[warp] = gb3;
+            __syncthreads();
+            if (tid < kH) g[kOffW3 + tid] = gw3 + sDz3[kH + tid];
+            if (tid == kH) g[kOffB3] = sDz3[0] + sDz3[1] + sDz3[2] + sDz3[3];
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
@@ -585,12 +595,21 @@ __global__ void k_mlp_wnorm(int n, const float* __restrict__ D, float* __restric
     for (int b = threadIdx.x; b < n; b += blockDim.x) W[b] = (D[b] > 0.f && tot > 0.0) ? (float)(W[b] / tot) : 0.f;
 }
 
-__global__ void k_mlp_reduce_grad(const float* __restrict__ gpart, int nblk, float* __restrict__ grad) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= kNP) return;
+// sum of the CTAs' partials: 32 outputs x 8 parts of the CTAs per block (one thread per output is a chain of
+// loads on 18 SMs)
+__global__ void __launch_bounds__(256) k_mlp_reduce_grad(const float* __restrict__ gpart, int nblk, float* __restrict__ grad) {
+    __shared__ float red[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
     float a = 0.f;
-    for (int b = 0; b < nblk; ++b) a += gpart[(size_t)b * kNP + e];
-    grad[e] = a;
+    if (e < kNP)
+#pragma unroll 8
+        for (int b = w; b < nblk; b += 8) a += gpart[(size_t)b * kNP + e];
+    red[w][lane] = a;
+    __syncthreads();
+    if (w == 0 && e < kNP) {
+        for (int i = 1; i < 8; ++i) a += red[i][lane];
+        grad[e] = a;
+    }
 }
 
 __global__ void k_mlp_band_of(const long long* __restrict__ off, int nband, int* __restrict__ band_of) {
@@ -724,11 +743,11 @@ struct DevBuf {
     }
 };
 
-int train_grid() {  // one gradient CTA per SM (its shared memory allows one)
+int train_grid(long n) {  // two gradient CTAs per SM, at most one per tile
     int dev = 0, nsm = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    return nsm;
+    return (int)std::max<long>(1, std::min<long>(2L * nsm, (n + kMT - 1) / kMT));
 }
 
 // loss (device) and gradient (device) for one parameter vector
@@ -757,7 +776,7 @@ qm_status loss_grad_dev(int nband, const long long* off, const int* band_of, lon
     }
     {
         ProfScope pf(PF_MLP, s);
-        k_mlp_reduce_grad<<<(kNP + 255) / 256, 256, 0, s>>>(gpart, nblk, grad);
+        k_mlp_reduce_grad<<<(kNP + 31) / 32, 256, 0, s>>>(gpart, nblk, grad);
     }
     return cuda_check(cudaGetLastError(), "learned preconditioner training launch");
 }
@@ -862,7 +881,7 @@ extern "C" qm_status qm_mlp_loss_grad(int nband, const long long* band_off, cons
         return st;
     const long n = (long)last;
     if (n < 1) return fail(QM_ERR_ARG, "qm_mlp_loss_grad: no samples");
-    const int nblk = train_grid();
+    const int nblk = train_grid(n);
     DevBuf K(s), bo(s), A(s), B(s), co(s), ra(s), ld(s), gp(s), er(s);
     if ((st = K.get(sizeof(float) * n)) || (st = bo.get(sizeof(int) * n)) || (st = A.get(sizeof(double) * nband)) ||
         (st = B.get(sizeof(double) * nband)) || (st = co.get(sizeof(float) * nband)) ||
@@ -896,7 +915,7 @@ extern "C" qm_status qm_mlp_train(int nband, const long long* band_off, const fl
         return st;
     const long n = (long)last;
     if (n < 1) return fail(QM_ERR_ARG, "qm_mlp_train: no samples");
-    const int nblk = train_grid();
+    const int nblk = train_grid(n);
     DevBuf K(s), bo(s), A(s), B(s), co(s), ra(s), lh(s), gp(s), gr(s), m(s), v(s), er(s);
     if ((st = K.get(sizeof(float) * n)) || (st = bo.get(sizeof(int) * n)) || (st = A.get(sizeof(double) * nband)) ||
         (st = B.get(sizeof(double) * nband)) || (st = co.get(sizeof(float) * nband)) ||
