@@ -56,5 +56,16 @@ def test_decoupled_tridiagonal(Q, m):
     _check(Q, H.astype(complex), m)
 
 
+@pytest.mark.parametrize("m", [66, 127, 128, 129, 256, 257, 512, 513, 768, 769])
+def test_back_transformation_rows(Q, m):
+    """The register rows of the back-transformation at their edges, with reflectors that are the identity
+    (a block that is already diagonal) between the others."""
+    H = _herm(np.random.default_rng(m), m)
+    H[m // 3: m // 2, :] = 0.0
+    H[:, m // 3: m // 2] = 0.0
+    H[np.arange(m // 3, m // 2), np.arange(m // 3, m // 2)] = 200.0 + np.arange(m // 2 - m // 3)
+    _check(Q, H, 9)
+
+
 def test_inverse_iteration_past_shared_memory(Q):
     _check(Q, _herm(np.random.default_rng(3), 1216), 470)
