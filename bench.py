@@ -4,7 +4,7 @@ Headline workload: the 255-atom Si-like cell with one vacancy (41.04 x 41.04 x 2
 30 Ry, the stated FFT grid 96x96x48, 4 shifted k-points, 288 bands, 1020 projectors, 95,885
 plane waves per k), the largest single-GPU workload of the method.  One step = H psi applied
 to every band at every k-point (1152 band-applies) through the C ABI (qm_hpsi).  The headline
-`value` is the precision form (QM_MIXED: FP32 FFT path, BF16x3 tensor-core nonlocal GEMMs);
+`value` is the precision form (QM_MIXED: FP32 FFT path, FP16-pair tensor-core nonlocal GEMMs);
 the plain FP64 form is measured on the same cell under `forms.fp64`.  Secondary objects: the
 64-atom cell (72^3, 4 k, 160 bands) in both forms, block Davidson to 1e-8 Ha on it, the batched
 form (256 uneven cells, one persistent launch) and the 216-atom cell.  Prints one JSON line.
@@ -45,10 +45,8 @@ FLOP_PER_CLK_SM = {"fp64": 4, "mixed": 256}
 
 # DRAM bytes per launch of a dominant kernel, from one ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum) of the current kernel, keyed by (kernel family, precision, workload);
-# None where no capture of the current kernel exists.  The tensor-core nonlocal family launches
-# the projection and the application GEMM once per k-point: its figure is their mean over one
-# k-point of the 255-atom cell (1.844 GB and 1.479 GB; every k-point has the same shapes).
-TRAFFIC_PER_LAUNCH = {("k_umma_bf16x3", "mixed", "si255_vac"): (1844459520 + 1478849536) // 2}
+# None where no capture of the current kernel exists.
+TRAFFIC_PER_LAUNCH = {}
 
 
 def parse():
@@ -390,16 +388,25 @@ def measure_hpsi(steps, warmup, Q, lib, g, cell, wl, v, D, world, dev, peaks, sa
         if name == "k_plane":
             fl = sum(nb * cell.grid[0] * fft_flops_per_plane(cell.grid, wl.nrow[ik]) for ik in range(nk))
         elif name in ("k_gemm_tn", "k_gemm_cn"):
-            fl = 8.0 * nproj * nb * sum(g.npw)   # 8 flops per complex multiply-add, all k
+            useful = 8.0 * nproj * nb * sum(g.npw)   # 8 flops per complex multiply-add, all k
+            fl = useful
+            if wl.prec == "fp64":
+                # exact digit products on the tensor cores: 34 BF16 products per FP64 one
+                fl = 34 * useful
+                bound = "tensor"
+                fl_pk = float(peaks.get("bf16_tflops_sustained", 1742.0))
+                extra = {"useful_tflops": useful / per_step / (avg_ms * 1e-3) / 1e12,
+                         "flops_counted": "BF16 digit products (34 per FP64 product); useful_tflops counts each "
+                                          "complex multiply-add once (8 flops)"}
         elif name == "k_umma_bf16x3":
-            # projection + application: 8 flops per complex multiply-add each; the method (3-term
-            # BF16 split) issues 6 BF16 products per FP32-accurate one, all on the tensor pipe
+            # projection + application: 8 flops per complex multiply-add each; the method (FP16
+            # pairs) issues 3 FP16 products per FP32-accurate one, all on the tensor pipe
             useful = 2 * 8.0 * nproj * nb * sum(g.npw)
-            fl = 6 * useful
+            fl = 3 * useful
             bound = "tensor"
             fl_pk = float(peaks.get("bf16_tflops_sustained", 1742.0))
             extra = {"useful_tflops": useful / per_step / (avg_ms * 1e-3) / 1e12,
-                     "flops_counted": "BF16 products of the 3-term split (6 per FP32-accurate product); "
+                     "flops_counted": "FP16 products of the pair split (3 per FP32-accurate product); "
                                       "useful_tflops counts each complex multiply-add once (8 flops)"}
         if fl is None:
             return {"bound": "hbm", "achieved": None, "peak": peaks.get("hbm_gbs"), "unit": "GB/s", "frac": None,
@@ -996,9 +1003,9 @@ def run_ours(args):
         keep = ("value", "ms_per_step", "steps", "roofline", "roofline_other", "kernels", "gpu_launches")
         line = {"metric": METRIC, "value": head["value"], "unit": UNIT, "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": head["ms_per_step"], "higher_is_better": True,
-                "scaling": "weak", "vs_baseline": None, "dtype": "f32+bf16x3", "data": "synthetic",
+                "scaling": "weak", "vs_baseline": None, "dtype": "f32+f16x2", "data": "synthetic",
                 "config": {"workload": WORKLOAD,
-                           "precision": "mixed (FP32 FFT path, BF16x3-split tensor-core nonlocal GEMMs)",
+                           "precision": "mixed (FP32 FFT path, FP16-pair tensor-core nonlocal GEMMs)",
                            "projectors": "prepared once per k-point (qm_hpsi_prepare, %.3f s, outside the timed "
                                          "steps); per-call splitting under forms.mixed_per_call" % head["prepare_seconds"],
                            "band_applies_per_step": cell.nbnd * len(cell.kpts), "npw": npw5,

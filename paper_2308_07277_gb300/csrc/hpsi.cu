@@ -28,7 +28,8 @@ constexpr size_t kStickBudgetOverlap = 1ull << 30;
 // caller's stream: the tensor-core chain is five or six launches (nine where the projectors are split on
 // the call) behind a fork and before a join.  Whole call, CUDA cores / tensor cores, us: prepared 1.3e6
 // (nproj nb npw) 41 / 47, 3.4e6 54 / 56, 1.0e7 77 / 60; split per call 3.4e6 54 / 72, 1.7e7 75 / 83,
-// 5.3e7 130 / 112.  One line for both, so that preparing the projectors does not change the result.
+// 5.3e7 130 / 112 (the chain's early launches have since taken 6 to 9 us off the tensor-core side above the line).
+// One line for both, so that preparing the projectors does not change the result.
 static bool small_nonlocal(int nproj, int nb, int npw) { return (double)nproj * nb * npw <= 3.5e6; }
 
 struct HpsiLayout {
