@@ -26,11 +26,11 @@ constexpr size_t kStickBudgetOverlap = 1ull << 30;
 
 // Whether the precision form's nonlocal part is small enough for FP32 products on the CUDA cores, on the
 // caller's stream: the tensor-core chain is five or six launches (nine where the projectors are split on
-// the call) behind a fork and before a join.  Whole call, CUDA cores / tensor cores, us: prepared 1.3e6
-// (nproj nb npw) 41 / 47, 3.4e6 54 / 56, 1.0e7 77 / 60; split per call 3.4e6 54 / 72, 1.7e7 75 / 83,
-// 5.3e7 130 / 112 (the chain's early launches have since taken 6 to 9 us off the tensor-core side above the line).
-// One line for both, so that preparing the projectors does not change the result.
-static bool small_nonlocal(int nproj, int nb, int npw) { return (double)nproj * nb * npw <= 3.5e6; }
+// the call) behind a fork and before a join.  With the chain's early launches the tensor cores win from about
+// 1.5e6 (nproj nb npw) on: whole call, CUDA cores / tensor cores, us: 1.3e6 41 / about 40, 3.4e6 54 / 48; a
+// propagation step of 16 atoms with 10 bands (3.1e6, four H psi) 269 / 189.  One line for prepared and split
+// projectors, so that preparing them does not change the result.
+static bool small_nonlocal(int nproj, int nb, int npw) { return (double)nproj * nb * npw <= 1.5e6; }
 
 struct HpsiLayout {
     size_t vt_off, p_off, part_off, part_bytes, t_off, nl_off, err_off, total, t_bytes;
