@@ -326,7 +326,12 @@ k_tridiag_rows(double2* __restrict__ A, int lda, int m, double2* __restrict__ Vh
 // last warp beside it.  v^H A v is real, so the correction of w = tau A v is one real sum.  Warp 0 updates the
 // next column first and builds its reflector while the others update the rest (lower triangle, mirrored).
 // Eight-band solves (m up to 32): 80 us on average, 248 us with the grid-wide kernel.
+// Unscaled, |tau|^2 is of the order of |x|^-4, so the range of x has to be bounded: a matrix whose largest
+// component lies outside 2^-50 ... 2^50 is scaled by a power of two into it (T is scaled back; v and tau belong
+// together at either scale), and a column whose norm is below 2^-120 of that component counts as eliminated
+// (its coupling is zero: a change of 1e-36 |A|).  Then |x| is within 2^-171 ... 2^57, |tau|^2 below 2^685.
 constexpr int kTriSmall = 64;
+constexpr int kTriRange = 50, kTriDrop = 120;
 __global__ void __launch_bounds__(256)
 k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restrict__ Vh, double2* __restrict__ tau,
                 double* __restrict__ d, double* __restrict__ e) {
@@ -335,8 +340,32 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
     double2 *a = smt, *vb = smt + m * ld, *w = vb + 2 * m;  // [m][ld], reflectors of two columns, product
     __shared__ double s_beta[2], s_half;  // beta (0: no reflection), -|tau|^2 / 2
     __shared__ double2 s_t;
+    __shared__ int s_max;
     const int tid = threadIdx.x, lane = tid & 31;
-    for (int i = tid; i < m * m; i += 256) a[(i / m) * ld + i % m] = A[(size_t)(i / m) * lda + i % m];
+    if (tid == 0) s_max = 0;
+    __syncthreads();
+    int h = 0;  // largest high word of a component, compared as integers
+    for (int i = tid; i < m * m; i += 256) {
+        const double2 x = A[(size_t)(i / m) * lda + i % m];
+        h = max(h, max(__double2hiint(x.x) & 0x7FFFFFFF, __double2hiint(x.y) & 0x7FFFFFFF));
+        a[(i / m) * ld + i % m] = x;
+    }
+    h = __reduce_max_sync(0xffffffffu, h);
+    if (lane == 0) atomicMax(&s_max, h);
+    __syncthreads();
+    // (a non-finite matrix is left as it is; a zero one has nothing to scale)
+    int ex = (s_max >> 20) - 1023;  // the largest component is in [2^ex, 2^(ex+1))
+    const bool scaled = (ex < -kTriRange || ex > kTriRange) && ex < 1024 && s_max > 0;
+    const double up = scaled ? ldexp(1.0, max(-1000, min(1000, -ex))) : 1.0, back = scaled ? 1.0 / up : 1.0;
+    if (scaled) {
+        for (int i = tid; i < m * m; i += 256) {
+            double2& x = a[(i / m) * ld + i % m];
+            x.x *= up;
+            x.y *= up;
+        }
+        ex = 0;
+    }
+    const double drop = ldexp(1.0, 2 * (ex - kTriDrop));  // on the square of a column's norm
     // the reflector of column k but for tau (one warp)
     auto reflector = [&](int k) {
         const int n = m - k - 1;
@@ -350,8 +379,9 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
         }
         for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
         const double2 alpha = a[(k + 1) * ld + k];
+        const bool none = part < drop;
         double beta = 0.0;
-        if (__any_sync(0xffffffffu, below) && part > 0.0) beta = -copysign(sqrt(part), alpha.x);
+        if (__any_sync(0xffffffffu, below) && !none) beta = -copysign(sqrt(part), alpha.x);
         for (int i = lane; i < n; i += 32) {
             double2 x = a[(k + 1 + i) * ld + k];
             if (i == 0) x.x -= beta;
@@ -359,8 +389,9 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
         }
         if (lane == 0) {
             s_beta[k & 1] = beta;
-            e[k] = beta != 0.0 ? beta : alpha.x;
-            d[k] = a[k * ld + k].x;
+            const double ek = none ? 0.0 : beta != 0.0 ? beta : alpha.x, dk = a[k * ld + k].x;
+            e[k] = scaled ? ek * back : ek;
+            d[k] = scaled ? dk * back : dk;
         }
     };
     __syncthreads();
@@ -445,7 +476,7 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
         }
     }
     __syncthreads();
-    if (tid == 0) d[m - 1] = a[(m - 1) * ld + m - 1].x;
+    if (tid == 0) d[m - 1] = a[(m - 1) * ld + m - 1].x * back;
 }
 
 // number of eigenvalues of T smaller than x: sign changes of the leading minors' determinants by their
