@@ -551,6 +551,15 @@ qm_status qm_eigh_lowest(int m, int nev, const void* A, int lda, double* evals, 
 qm_status qm_zgemm(int op, int arith, int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C,
                    int ldc, void* stream);
 
+/* qm_zgemm_hold - qm_zgemm (arith 0) with a given amount of device scratch, and failure-detection test hook of
+ * its bounded tensor-core waits (not part of the method).  scratch: bytes (0: none); with less than qm_zgemm
+ * takes the product runs in more panels of K (op 0) or of columns (op 1), or in FP64 multiply-adds.  panel >= 0:
+ * the waits of that panel give up after `polls` polls; what they leave incomplete is recomputed in FP64
+ * multiply-adds, so the result is whole all the same.  panels: host, receives the number of panels (0: the
+ * product ran in multiply-adds).  Errors as qm_zgemm. */
+qm_status qm_zgemm_hold(int op, int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C, int ldc,
+                        size_t scratch, int panel, long long polls, int* panels, void* stream);
+
 /*
  * qm_tddft_taylor - real-time propagation by the truncated Taylor series of the propagator
  * (Sec. 5, "tddft" module, expoper submodule):

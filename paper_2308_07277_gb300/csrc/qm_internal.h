@@ -223,11 +223,14 @@ qm_status launch_local_kinetic_tab(const DevTables& t, int nb, const void* psi, 
 // least as large in every dimension) serve it best; with less (none: ptr NULL) it runs with fewer
 // splits and without the digit products.  digits = false: FP64 multiply-adds at every size.
 // err (may be NULL): device word set when a bounded wait of the digit products expired.
+// hold_panel, hold_polls: the waits of that panel's product give up after so many polls (failure test).
 struct GemmWork {
     void* ptr = nullptr;
     size_t bytes = 0;
     int* err = nullptr;
     bool digits = true;
+    int hold_panel = -1;
+    long hold_polls = 0;
 };
 // Rows of a product that the digit products leave to the FP64 kernels: *any != 0 if there are some,
 // output (m, n) is one if em[m] or en[n] equals `flag`.  any = NULL: every output.
@@ -255,6 +258,7 @@ qm_status zdigits_tn(int M, int N, int K, const double2* A, int lda, const doubl
                      int ldb, double2* C, int ldc, bool accumulate, const GemmWork& w, cudaStream_t s, GemmFlags* flags,
                      bool* done);
 size_t zdigits_bytes(bool cn, int M, int N, int K);
+int zdigits_panels(bool cn, int M, int N, int K, size_t bytes);  // panels with that much scratch, 0: not served
 // ---- tensor-core nonlocal step of the precision form (nonlocal_tc.cu) ----
 constexpr int kMaxUmmaSplits = 64;
 // out[b][g] (+)= sum_p beta[p][g] D_p <beta_p|psi_b> (FP32 complex in/out) as FP16-pair split

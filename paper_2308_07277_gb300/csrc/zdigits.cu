@@ -192,7 +192,9 @@ __global__ void __launch_bounds__(256) k_dg_colmax(const double2* __restrict__ s
 }
 
 // rows of src (complex columns [0, cols)) -> digit planes; expanded: output row 2r + t.  CTA: 8
-// output rows (one core-matrix row group) x 32 chunks of 8 real values.  eout: the rows' exponents
+// output rows (one core-matrix row group) x 32 chunks of 8 real values.  eout: the rows' exponents, written
+// for the first panel of K only (NULL later): a product that gives up marks its rows there, and a later panel
+// must not take the mark off
 __global__ void __launch_bounds__(256) k_dg_rows(const double2* __restrict__ src, int ld, int rows, int cols, int expand,
                                                  int R, int nkt, const int* __restrict__ emax, int* __restrict__ eout,
                                                  int* __restrict__ any, unsigned char* __restrict__ blk) {
@@ -200,7 +202,7 @@ __global__ void __launch_bounds__(256) k_dg_rows(const double2* __restrict__ src
     const int ch = blockIdx.x * 32 + (threadIdx.x >> 3);
     const int b = expand ? (r >> 1) : r;
     const int e = b < rows ? reduce_segs(emax, rows, b) : 0;
-    if (ch == 0 && b < rows && !(expand && (r & 1))) {
+    if (eout && ch == 0 && b < rows && !(expand && (r & 1))) {
         eout[b] = e;
         if (e == kDgFlag) *any = 1;
     }
@@ -289,8 +291,8 @@ __device__ __forceinline__ double dg_value(long long hi, long long lo, int ex) {
 // exponent of the integer unit of a product of rows with exponents ea, eb
 __device__ __forceinline__ int dg_unit(int ea, int eb) { return ea + eb - 2 * 1022 - 70; }
 
-__device__ __forceinline__ bool dg_wait(uint32_t bar, uint32_t parity, volatile int* abort) {
-    for (long i = 0; i < kDgSpin; ++i) {
+__device__ __forceinline__ bool dg_wait(uint32_t bar, uint32_t parity, volatile int* abort, long polls = kDgSpin) {
+    for (long i = 0; i < polls; ++i) {
         uint32_t done;
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
@@ -313,7 +315,7 @@ __global__ void __launch_bounds__(kDgThreads, 1)
 k_dg_gemm(const unsigned char* __restrict__ P, const unsigned char* __restrict__ X, int nkt, int kt_per_split,
           longlong2* __restrict__ part, int mpad, int npad, int add, int* __restrict__ ep,
           const int* __restrict__ ex, int* __restrict__ any, int nplain, int nexp, double2* __restrict__ C, int ldc, int accumulate,
-          int* __restrict__ err) {
+          int* __restrict__ err, long polls) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t full[kDgStages], empty[kDgStages], acc_full, acc_empty, done;
     __shared__ uint32_t tmem_base;
@@ -352,7 +354,7 @@ k_dg_gemm(const unsigned char* __restrict__ P, const unsigned char* __restrict__
             int it = 0;
             for (; it < nk; ++it) {
                 const int s = it % kDgStages;
-                if (it >= kDgStages && !dg_wait(tc::smem_u32(&empty[s]), ((it / kDgStages) & 1) ^ 1, abort)) {
+                if (it >= kDgStages && !dg_wait(tc::smem_u32(&empty[s]), ((it / kDgStages) & 1) ^ 1, abort, polls)) {
                     *abort = 1;
                     break;
                 }
@@ -376,11 +378,11 @@ k_dg_gemm(const unsigned char* __restrict__ P, const unsigned char* __restrict__
             for (; it < nk; ++it) {
                 const int s = it % kDgStages, c = it / kDgChunk;
                 // the drains of the previous chunk must have read the accumulators
-                if (it % kDgChunk == 0 && c > 0 && !dg_wait(tc::smem_u32(&acc_empty), (c - 1) & 1, abort)) {
+                if (it % kDgChunk == 0 && c > 0 && !dg_wait(tc::smem_u32(&acc_empty), (c - 1) & 1, abort, polls)) {
                     *abort = 1;
                     break;
                 }
-                if (!dg_wait(tc::smem_u32(&full[s]), (it / kDgStages) & 1, abort)) {
+                if (!dg_wait(tc::smem_u32(&full[s]), (it / kDgStages) & 1, abort, polls)) {
                     *abort = 1;
                     break;
                 }
@@ -422,7 +424,7 @@ k_dg_gemm(const unsigned char* __restrict__ P, const unsigned char* __restrict__
         for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
         bool ok = true;
         for (int c = 0; c < nchunk; ++c) {
-            ok = dg_wait(tc::smem_u32(&acc_full), c & 1, abort);
+            ok = dg_wait(tc::smem_u32(&acc_full), c & 1, abort, polls);
             if (!ok) *abort = 1;
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -627,13 +629,13 @@ bool dg_serves(bool cn, int M, int N, int K) {
 template <int EPI>
 qm_status dg_gemm(const unsigned char* P, const unsigned char* X, int nkt, int splits, int pt, int xt, longlong2* part, int mpad,
                   int npad, bool add, int* ep, const int* ex, int* any, int nplain, int nexp, double2* C, int ldc, bool accumulate,
-                  int* err, cudaStream_t s) {
+                  int* err, long polls, cudaStream_t s) {
     const size_t smem = (size_t)kDgStages * (dg_block(kDgM) + dg_block(kDgN));
     qm_status st = allow_dynamic_smem((const void*)k_dg_gemm<EPI>, smem, "digit products: shared memory");
     if (st) return st;
     ProfScope pf(EPI ? PF_GEMM_TN : PF_GEMM_CN, s);
     k_dg_gemm<EPI><<<dim3(xt, pt, splits), kDgThreads, smem, s>>>(P, X, nkt, cdiv(nkt, splits), part, mpad, npad, add ? 1 : 0, ep, ex,
-                                                                any, nplain, nexp, C, ldc, accumulate ? 1 : 0, err);
+                                                                any, nplain, nexp, C, ldc, accumulate ? 1 : 0, err, polls);
     return cuda_check(cudaGetLastError(), "k_dg_gemm launch");
 }
 
@@ -643,6 +645,11 @@ size_t zdigits_bytes(bool cn, int M, int N, int K) {
     if (!dg_serves(cn, M, N, K)) return 0;
     DgLayout L;
     return dg_layout(cn, cn ? M : N, cn ? N : M, K, 0, L) ? L.total : 0;
+}
+
+int zdigits_panels(bool cn, int M, int N, int K, size_t bytes) {
+    DgLayout L;
+    return dg_serves(cn, M, N, K) && dg_layout(cn, cn ? M : N, cn ? N : M, K, bytes, L) ? L.npanel : 0;
 }
 
 // Both return false in *done when the product is left to the FP64 kernels (small, or not enough
@@ -677,14 +684,14 @@ qm_status zdigits_cn(int M, int N, int K, const double2* A, int lda, const doubl
         if (p == 0) Z = splits;
         {
             ProfScope pf(PF_SPLIT, s);
-            k_dg_rows<<<dim3(cdiv(nkt * 2, 32), mpad / 8), 256, 0, s>>>(A + c0, lda, M, cols, 0, kDgM, nkt, ma, ea, any, P);
+            k_dg_rows<<<dim3(cdiv(nkt * 2, 32), mpad / 8), 256, 0, s>>>(A + c0, lda, M, cols, 0, kDgM, nkt, ma, p ? nullptr : ea, any, P);
         }
         {
             ProfScope pf(PF_SPLIT, s);
-            k_dg_rows<<<dim3(cdiv(nkt * 2, 32), npad / 8), 256, 0, s>>>(B + c0, ldb, N, cols, 1, kDgN, nkt, mb, eb, any, X);
+            k_dg_rows<<<dim3(cdiv(nkt * 2, 32), npad / 8), 256, 0, s>>>(B + c0, ldb, N, cols, 1, kDgN, nkt, mb, p ? nullptr : eb, any, X);
         }
         qm_status st = dg_gemm<0>(P, X, nkt, splits, L.ptiles, L.xtiles, part, mpad, npad, p > 0, ea, eb, any, M, N, nullptr, 0, false,
-                                  w.err, s);
+                                  w.err, p == w.hold_panel ? w.hold_polls : kDgSpin, s);
         if (st) return st;
     }
     {
@@ -728,7 +735,7 @@ qm_status zdigits_tn(int M, int N, int K, const double2* A, int lda, const doubl
                                                                         N, eb + r0, any, P);
         }
         qm_status st = dg_gemm<1>(P, X, L.nkt, 1, pt, L.xtiles, nullptr, 0, 0, false, eb + r0, ea, any, rows, M, C + r0, ldc, accumulate,
-                                  w.err, s);
+                                  w.err, p == w.hold_panel ? w.hold_polls : kDgSpin, s);
         if (st) return st;
     }
     *flags = GemmFlags{any, ea, eb, kDgFlag};

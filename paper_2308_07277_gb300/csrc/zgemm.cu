@@ -540,13 +540,19 @@ qm_status cgemm_tn(int M, int N, int K, const float2* A, int lda, const double* 
 
 using namespace qm;
 
+static qm_status check_zgemm(int op, int M, int N, int K, const void* A, int lda, const void* B, int ldb, const void* C,
+                             int ldc) {
+    if (M < 1 || N < 1 || K < 1 || !A || !B || !C) return fail(QM_ERR_ARG, "qm_zgemm: bad sizes or NULL operand");
+    if (op == 0 ? (lda < K || ldb < K || ldc < N) : (lda < M || ldb < N || ldc < N))
+        return fail(QM_ERR_ARG, "qm_zgemm: leading dimension too small");
+    return QM_OK;
+}
+
 extern "C" qm_status qm_zgemm(int op, int arith, int M, int N, int K, const void* A, int lda, const void* B, int ldb,
                               void* C, int ldc, void* stream) {
     clear_error();
     if ((op != 0 && op != 1) || arith < 0 || arith > 2) return fail(QM_ERR_ARG, "qm_zgemm: op not 0/1 or arith not 0..2");
-    if (M < 1 || N < 1 || K < 1 || !A || !B || !C) return fail(QM_ERR_ARG, "qm_zgemm: bad sizes or NULL operand");
-    if (op == 0 ? (lda < K || ldb < K || ldc < N) : (lda < M || ldb < N || ldc < N))
-        return fail(QM_ERR_ARG, "qm_zgemm: leading dimension too small");
+    if (qm_status st = check_zgemm(op, M, N, K, A, lda, B, ldb, C, ldc)) return st;
     cudaStream_t s = (cudaStream_t)stream;
     const double2* a = (const double2*)A;
     const double2* b = (const double2*)B;
@@ -582,6 +588,27 @@ extern "C" qm_status qm_zgemm(int op, int arith, int M, int N, int K, const void
     }
     qm_status st = op == 0 ? zgemm_cn(M, N, K, a, lda, b, ldb, c, ldc, w, s)
                            : zgemm_tn(M, N, K, a, lda, nullptr, b, ldb, c, ldc, false, w, s, 1.0);
+    if (w.ptr) cudaFreeAsync(w.ptr, s);
+    return st;
+}
+
+extern "C" qm_status qm_zgemm_hold(int op, int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C,
+                                   int ldc, size_t scratch, int panel, long long polls, int* panels, void* stream) {
+    clear_error();
+    if (op != 0 && op != 1) return fail(QM_ERR_ARG, "qm_zgemm_hold: op not 0/1");
+    if (panel < -1 || polls < 0 || !panels) return fail(QM_ERR_ARG, "qm_zgemm_hold: bad panel or polls, or NULL panels");
+    qm_status st = check_zgemm(op, M, N, K, A, lda, B, ldb, C, ldc);
+    if (st) return st;
+    *panels = 0;
+    cudaStream_t s = (cudaStream_t)stream;
+    GemmWork w;
+    w.bytes = scratch;
+    w.hold_panel = panel;
+    w.hold_polls = (long)polls;
+    if (scratch && (st = cuda_check(cudaMallocAsync(&w.ptr, scratch, s), "qm_zgemm_hold: workspace"))) return st;
+    if (scratch) *panels = zdigits_panels(op == 0, M, N, K, scratch);
+    st = op == 0 ? zgemm_cn(M, N, K, (const double2*)A, lda, (const double2*)B, ldb, (double2*)C, ldc, w, s)
+                 : zgemm_tn(M, N, K, (const double2*)A, lda, nullptr, (const double2*)B, ldb, (double2*)C, ldc, false, w, s, 1.0);
     if (w.ptr) cudaFreeAsync(w.ptr, s);
     return st;
 }
