@@ -51,7 +51,7 @@ typedef enum {
 } qm_status;
 
 typedef enum {
-    QM_FP64 = 0,   /* everything to FP64 accuracy (large complex products: see qm_zgemm, arith 0) */
+    QM_FP64 = 0,   /* FP64; large complex products to FP64 accuracy by norm (see qm_zgemm, arith 0) */
     QM_MIXED = 1   /* FP32 FFT path and V multiply; nonlocal projection and application as split
                       products of FP16 pairs (row-scaled, 23 bits) on the tensor cores, FP32
                       accumulation; FP32 products on the CUDA cores for small ones */
@@ -386,10 +386,11 @@ typedef struct {
                             of the unconverged bands (GD+k: Stathopoulos & Saad, ETNA 7, 163 (1998)),
                             as many as fit beside the next corrections; 1 = plain restart from the
                             Ritz vectors only */
-    int fp64_exact;      /* 0 or 1; both run the FP64 phase of QM_MIXED on the products of QM_FP64 (FP64
-                            multiply-adds, or exact digit products on the tensor cores where those are
-                            faster, see qm_zgemm), whose error is never above FP64 arithmetic's.  (The
-                            field chose a 47-bit arithmetic before those products existed.) */
+    int fp64_exact;      /* the plane-wave-length products of QM_FP64 and of QM_MIXED's FP64 phase (H_sub
+                            columns, Ritz vectors, orthogonalisation, the nonlocal GEMMs of its H psi):
+                            0 (default) = as qm_zgemm with arith 0 (digit products on the tensor cores
+                            where those are faster: FP64 accuracy by norm); 1 = in FP64 multiply-adds at
+                            every size (arith 3) */
 } qm_davidson_opts;
 
 /* Counters of one qm_davidson call (the paper's "H-psi calls" are band_applies / nb). */
@@ -536,13 +537,20 @@ qm_status qm_eigh_lowest(int m, int nev, const void* A, int lda, double* evals, 
  * own so that their arithmetic can be checked:
  *   op 0 (cn): C[m][n] = sum_k conj(A[m][k]) B[n][k]     A: M x K, B: N x K (k contiguous)
  *   op 1 (tn): C[m][n] = sum_k A[k][m] B[k][n]           A: K x M, B: K x N (m, n contiguous)
- *  arith   0 = FP64: multiply-adds for small products; larger ones as exact sums of 8-bit digit
- *          products on the tensor cores, every operand element rounded at 2^-56 of the largest
- *          component of its row (of A or B along k) and the sum rounded once, which measures
- *          closer to the exact value than FP64 multiply-adds (rows with non-finite values, or with
- *          nothing above 2^-960, run in multiply-adds); 1 = the same (a 47-bit arithmetic before);
+ *  arith   0 = FP64 accuracy by norm: multiply-adds for small products; larger ones as exact sums
+ *          of 8-bit digit products on the tensor cores, every operand element rounded at 2^-55 of
+ *          the largest component of its row (of A or B along k), products kept to 2^-59 of both
+ *          rows' largest, and the sum rounded once (rows with non-finite values, or with nothing
+ *          above 2^-960, run in multiply-adds).  The error of an output is at most about
+ *          2^-55 (max|a| sum|b| + max|b| sum|a|) over its two rows: closer to the exact value than
+ *          multiply-adds where large elements meet large ones, as in the products of a Davidson, but
+ *          elements far below their row's largest keep fewer bits than FP64 gives them, and none
+ *          below 2^-56 of it.  Where such elements decide a sum (rows that fall where the other
+ *          operand's rise), take arith 3.
+ *          1 = the same as 0 (a 47-bit arithmetic before);
  *          2 = 3-term BF16 split products on the tensor cores accumulated in FP32 (the precision
- *          form's FP32 phase; FP32-level accuracy; synchronises the stream).
+ *          form's FP32 phase; FP32-level accuracy; synchronises the stream);
+ *          3 = FP64 multiply-adds at every size.
  *  A, B, C device, complex double, row-major with the leading dimensions given; C is written.
  *  stream  cudaStream_t.  Partial sums, digit planes (at most about 600 MB) and tensor-core
  *          workspaces are allocated with cudaMallocAsync on the stream.

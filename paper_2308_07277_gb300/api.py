@@ -292,7 +292,8 @@ def qm_eigh_lowest(A, nev, stream=None):
 
 def qm_zgemm(op, A, B, arith=0, stream=None):
     """op "cn": C = conj(A) B^T for A (M, K), B (N, K); op "tn": C = A^T B for A (K, M), B (K, N).
-    complex128 CUDA tensors; arith 0 and 1 = FP64 accuracy, 2 = FP32 accuracy.  Returns C (M, N)."""
+    complex128 CUDA tensors; arith 0 and 1 = FP64 accuracy by norm, 2 = FP32 accuracy, 3 = FP64 multiply-adds.
+    Returns C (M, N)."""
     lib = _lib.load()
     if op == "cn":
         (M, K), N = A.shape, int(B.shape[0])

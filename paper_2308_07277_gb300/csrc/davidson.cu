@@ -280,7 +280,8 @@ struct DavidsonRun {
 
     qm_status hpsi(const double2* in, double2* out, int n) {
         applies += n;
-        if (!mixed) return hpsi_run(g, ik, n, in, ld, vloc, nproj, beta, ldb, nullptr, D, out, ld, QM_FP64, s);
+        if (!mixed) return hpsi_run(g, ik, n, in, ld, vloc, nproj, beta, ldb, nullptr, D, out, ld, QM_FP64, s, false,
+                                   w.part.digits);
         applies_mixed += n;
         qm_status st = convert_rows(in, ld, psi32, ld, n, npw, s);
         if (st) return st;
@@ -523,7 +524,8 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
     const size_t sqb = (size_t)nsq * nb * sizeof(double2);
     const size_t oCp = take(thick ? sqb : 0), oCT = take(thick ? sqb : 0), oPT = take(thick ? sqb : 0),
                  oQT = take(thick ? sqb : 0), oY = take(thick ? big * nb : 0), oHY = take(thick ? big * nb : 0);
-    const size_t part_bytes = std::max(gemm_cn_partial_bytes(false), std::max(zgemm_cn_bytes(nvx, nvx, npw), zgemm_tn_bytes(nvx, npw, nvx)));
+    const bool digits = o.fp64_exact == 0;
+    const size_t part_bytes = std::max(gemm_cn_partial_bytes(false), std::max(zgemm_cn_bytes(nvx, nvx, npw, digits), zgemm_tn_bytes(nvx, npw, nvx, digits)));
     const size_t oPart = take(part_bytes);
     const size_t oEval = take(sizeof(double) * nsq), oEps = take(sizeof(double) * (nsq + nb)),
                  oTk = take(sizeof(double) * nsq),
@@ -561,7 +563,7 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
     w.A = (double2*)(base + oA);
     w.Z = (double2*)(base + oZ);
     w.Cs = (double2*)(base + oCs);
-    w.part = GemmWork{base + oPart, part_bytes, (int*)(base + oInfo) + 3};
+    w.part = GemmWork{base + oPart, part_bytes, (int*)(base + oInfo) + 3, digits};
     if (thick) {
         w.Cp = (double2*)(base + oCp);
         w.CT = (double2*)(base + oCT);

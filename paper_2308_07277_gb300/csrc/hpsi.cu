@@ -36,7 +36,7 @@ struct HpsiLayout {
     size_t vt_off, p_off, part_off, part_bytes, t_off, nl_off, err_off, total, t_bytes;
 };
 
-static HpsiLayout hpsi_layout(qm_gspace g, int ik, int nb, int nproj, bool fp32, bool own_beta, bool gamma) {
+static HpsiLayout hpsi_layout(qm_gspace g, int ik, int nb, int nproj, bool fp32, bool own_beta, bool gamma, bool digits) {
     HpsiLayout L{};
     const size_t cs = fp32 ? sizeof(float2) : sizeof(double2);
     const size_t rs = fp32 ? sizeof(float) : sizeof(double);
@@ -51,7 +51,7 @@ static HpsiLayout hpsi_layout(qm_gspace g, int ik, int nb, int nproj, bool fp32,
     L.part_off = off;
     // scratch of the projector products on the caller's stream
     const bool small = fp32 && small_nonlocal(nproj, nb, npw);
-    L.part_bytes = nproj == 0 ? 0 : fp32 ? (small ? csmall_cn_bytes(nproj, nb, npw) : 0) : std::max(zgemm_cn_bytes(nproj, nb, npw), zgemm_tn_bytes(nb, npw, nproj));
+    L.part_bytes = nproj == 0 ? 0 : fp32 ? (small ? csmall_cn_bytes(nproj, nb, npw) : 0) : std::max(zgemm_cn_bytes(nproj, nb, npw, digits), zgemm_tn_bytes(nb, npw, nproj, digits));
     off = align_up(off + L.part_bytes, 256);
     L.t_off = off;
     // the precision form keeps every band's stick buffer (K1 and K2 of all bands overlap the
@@ -81,7 +81,7 @@ extern "C" qm_status qm_hpsi(qm_gspace g, int ik, int nb, const void* psi, int l
 
 qm_status qm::hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi, const double* vloc_r, int nproj,
                        const void* beta, int ld_beta, const void* beta_prepared, const double* D, void* out,
-                       int ld_out, qm_precision prec, cudaStream_t s, bool gamma) {
+                       int ld_out, qm_precision prec, cudaStream_t s, bool gamma, bool digits) {
     if (!g) return fail(QM_ERR_ARG, "qm_hpsi: NULL gspace");
     if (ik < 0 || ik >= g->nk) return fail(QM_ERR_ARG, "qm_hpsi: ik out of range");
     if (nb < 0 || nproj < 0) return fail(QM_ERR_ARG, "qm_hpsi: negative nb or nproj");
@@ -113,12 +113,12 @@ qm_status qm::hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi,
         if (p.dev && p.beta == beta && p.ld == ld_beta && p.nproj == nproj) beta_prepared = p.dev;
     }
 
-    const HpsiLayout L = hpsi_layout(g, ik, nb, nproj, fp32, beta_prepared == nullptr, gamma);
+    const HpsiLayout L = hpsi_layout(g, ik, nb, nproj, fp32, beta_prepared == nullptr, gamma, digits);
     if ((st = ensure_workspace(g, L.total, s))) return st;
     char* ws = (char*)g->ws.ptr;
     void* vt = ws + L.vt_off;
     void* P = ws + L.p_off;
-    const GemmWork gw{ws + L.part_off, L.part_bytes, (int*)(ws + L.err_off)};
+    const GemmWork gw{ws + L.part_off, L.part_bytes, (int*)(ws + L.err_off), digits};
     void* T = ws + L.t_off;
 
     const bool small = fp32 && nproj > 0 && small_nonlocal(nproj, nb, npw);

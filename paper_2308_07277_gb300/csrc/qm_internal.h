@@ -239,8 +239,8 @@ struct GemmFlags {
     const int *em = nullptr, *en = nullptr;
     int flag = 0;
 };
-size_t zgemm_cn_bytes(int M, int N, int K);
-size_t zgemm_tn_bytes(int M, int N, int K);
+size_t zgemm_cn_bytes(int M, int N, int K, bool digits = true);
+size_t zgemm_tn_bytes(int M, int N, int K, bool digits = true);
 // C[m][n] = sum_k conj(A[m][k]) * B[n][k]   (A: M rows, B: N rows, k contiguous);
 // split over K into partial sums reduced in a fixed order (deterministic).
 qm_status zgemm_cn(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb,
@@ -278,9 +278,10 @@ qm_status nonlocal_tc_prepare(int nproj, int nb, int npw, const float2* beta, in
 // qm_hpsi with the precision form's projectors optionally pre-split (beta_prepared, see
 // nonlocal_tc); qm_hpsi itself passes NULL.
 // gamma: the Gamma-point real-wavefunction FFT path (qm_hpsi_gamma; two bands per transform).
+// digits = false: FP64 multiply-adds in the projector products of QM_FP64 at every size.
 qm_status hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi, const double* vloc_r, int nproj,
                    const void* beta, int ld_beta, const void* beta_prepared, const double* D, void* out, int ld_out,
-                   qm_precision prec, cudaStream_t s, bool gamma = false);
+                   qm_precision prec, cudaStream_t s, bool gamma = false, bool digits = true);
 // Subspace products of the Davidson FP32 phase on the tensor cores: FP64 storage rounded to
 // FP32 on load, BF16x3 split products accumulated in FP32 per K split, splits summed in FP64.
 //   cn: C[i][j] = sum_k conj(A[i][k]) B[j][k]                (as zgemm_cn)

@@ -12,12 +12,16 @@
 // which BF16 holds exactly.  A product of two digits is at most 2^14, so a sum of them is an
 // integer FP32 holds exactly below 2^24: the tensor core's FP32 accumulation commits no rounding.
 // Digit products of equal weight i + j = d share one accumulator; the eight accumulators
-// d = 0 ... 7 (34 of the 49 digit products; the dropped ones are below 2^-61 of max|a| max|b| per
-// term) are read from tensor memory every kDgChunk K tiles and added to 64-bit integers,
+// d = 0 ... 7 (34 of the 49 digit products; the dropped ones sum to at most 2^-59.7 of max|a| max|b| per
+// real term) are read from tensor memory every kDgChunk K tiles and added to 64-bit integers,
 // hi = S_0 2^24 + ... + S_3 and lo = S_4 2^24 + ... + S_7, so the sum over K is exact as well and
 // does not depend on how K is split; one rounding makes the FP64 result.
-// The error of a term is that of its operands' rounding, 2^-56 of the row's largest element, where
-// FP64 multiply-adds round every partial sum.  Relative error (2-norm, against 80-bit sums), FP64
+// The error of a term is that of its operands' rounding, at most 2^-55 of the row's largest component,
+// where FP64 multiply-adds round every partial sum: FP64 accuracy by norm.  It is not element by
+// element: what lies below 2^-56 of its row's largest is lost, so a sum that such elements decide (rows
+// that fall where the other operand's rise, |a_k| = e^(-20 k/K), |b_k| = e^(20 k/K - 20): error 8e-11 of
+// sum |a| |b|, FP64 3e-17) needs the FP64 kernels: qm_zgemm's arith 3, qm_davidson_opts.fp64_exact.
+// Relative error (2-norm, against 80-bit sums) of rows that fall together, FP64
 // multiply-adds / digits: 2.7e-15 / 1.3e-16 at 480 x 157 x 18232 (rows falling off 13-fold), 2.4e-15 /
 // 8.9e-17 (200-fold), 3.8e-15 / 9.6e-17 at 640 x 100 x 40000, 8.6e-16 / 8.4e-17 at 512 x 64 x 400;
 // tn 2.3e-16 / 7.2e-17 at 64 x 12000 x 17, 2.7e-15 / 1.2e-16 at 157 x 18232 x 480.

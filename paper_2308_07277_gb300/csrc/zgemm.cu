@@ -487,12 +487,12 @@ int zgemm_cn_splits(int M, int N, int K) {
     return std::max(1, std::min(64, (K + kCnK - 1) / kCnK));
 }
 
-size_t zgemm_cn_bytes(int M, int N, int K) {
+size_t zgemm_cn_bytes(int M, int N, int K, bool digits) {
     if (M <= 0 || N <= 0) return 0;
     const int splits = zcn_splits(M, N, K, 64);
-    return std::max(zdigits_bytes(true, M, N, K), splits > 1 ? (size_t)splits * M * N * sizeof(double2) : 0);
+    return std::max(digits ? zdigits_bytes(true, M, N, K) : 0, splits > 1 ? (size_t)splits * M * N * sizeof(double2) : 0);
 }
-size_t zgemm_tn_bytes(int M, int N, int K) { return M <= 0 || N <= 0 ? 0 : zdigits_bytes(false, M, N, K); }
+size_t zgemm_tn_bytes(int M, int N, int K, bool digits) { return M <= 0 || N <= 0 || !digits ? 0 : zdigits_bytes(false, M, N, K); }
 
 qm_status zgemm_cn(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb, double2* C, int ldc,
                    const GemmWork& w, cudaStream_t s) {
@@ -551,7 +551,7 @@ static qm_status check_zgemm(int op, int M, int N, int K, const void* A, int lda
 extern "C" qm_status qm_zgemm(int op, int arith, int M, int N, int K, const void* A, int lda, const void* B, int ldb,
                               void* C, int ldc, void* stream) {
     clear_error();
-    if ((op != 0 && op != 1) || arith < 0 || arith > 2) return fail(QM_ERR_ARG, "qm_zgemm: op not 0/1 or arith not 0..2");
+    if ((op != 0 && op != 1) || arith < 0 || arith > 3) return fail(QM_ERR_ARG, "qm_zgemm: op not 0/1 or arith not 0..2 or 3");
     if (qm_status st = check_zgemm(op, M, N, K, A, lda, B, ldb, C, ldc)) return st;
     cudaStream_t s = (cudaStream_t)stream;
     const double2* a = (const double2*)A;
@@ -579,8 +579,9 @@ extern "C" qm_status qm_zgemm(int op, int arith, int M, int N, int K, const void
         if (!st && e) st = fail(QM_ERR_TIMEOUT, "qm_zgemm: a bounded tensor-core wait expired");
         return st;
     }
-    const size_t bytes = op == 0 ? zgemm_cn_bytes(M, N, K) : zgemm_tn_bytes(M, N, K);
     GemmWork w;
+    w.digits = arith != 3;
+    const size_t bytes = op == 0 ? zgemm_cn_bytes(M, N, K, w.digits) : zgemm_tn_bytes(M, N, K, w.digits);
     w.bytes = bytes;
     if (bytes && cudaMallocAsync(&w.ptr, bytes, s) != cudaSuccess) {
         cudaGetLastError();
