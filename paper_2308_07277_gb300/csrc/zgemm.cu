@@ -335,8 +335,21 @@ int zcn_splits(int M, int N, int K, long cap, int per_term = 128) {
     return best;
 }
 
+// a launch's row tiles are its y blocks, at most 65535: more rows take several launches
+constexpr int kMaxRowTiles = 65535;
+GemmFlags flags_from(GemmFlags f, int row) {
+    if (f.em) f.em += row;
+    return f;
+}
+
 template <class T>
 qm_status cn_small(int M, int N, int K, const T* A, int lda, const T* B, int ldb, T* C, int ldc, T* partial, size_t partial_bytes, const GemmFlags& f, cudaStream_t s) {
+    constexpr int most = kMaxRowTiles * kCnTile;
+    if (M > most) {
+        qm_status st = cn_small(most, N, K, A, lda, B, ldb, C, ldc, partial, partial_bytes, f, s);
+        return st ? st : cn_small(M - most, N, K, A + (size_t)most * lda, lda, B, ldb, C + (size_t)most * ldc, ldc, partial,
+                                  partial_bytes, flags_from(f, most), s);
+    }
     const long cap = partial ? (long)(partial_bytes / sizeof(T)) / ((long)M * N) : 1;
     int splits = zcn_splits(M, N, K, std::max<long>(1, cap), sizeof(T) == 8 ? 12 : 128);
     int kchunk = std::max(kCnK, ((K + splits - 1) / splits + kCnK - 1) / kCnK * kCnK);
@@ -356,14 +369,20 @@ qm_status cn_small(int M, int N, int K, const T* A, int lda, const T* B, int ldb
 template <class T>
 qm_status tn_small(int M, int N, int K, const T* A, int lda, const double* d, double alpha, const T* B, int ldb, T* C,
                    int ldc, bool accumulate, const GemmFlags& f, cudaStream_t s) {
-    ProfScope pf(PF_GEMM_TN, s);
     // Rows per CTA, 8 or 4, in FP64: a warp's FP64 instruction holds one of the SM's four partitions, so eight
     // rows take twice the time of four and are worth it only where the tiles fill the SMs that often anyway
     // (8 x 1500 outputs, K up to 32: 5.2 us with 4 rows on 94 SMs, 6.9 us with 8 on 47)
     const auto tiles = [&](int rows) { return (long)((N + kTnN - 1) / kTnN) * ((M + rows - 1) / rows); };
     const long sms = device_sms(), load8 = (tiles(8) + sms - 1) / sms * 2, load4 = (tiles(4) + sms - 1) / sms;
     const int rows = sizeof(T) == sizeof(double2) && load4 < load8 ? 4 : 8;
+    if (M > kMaxRowTiles * rows) {
+        const int most = kMaxRowTiles * rows;
+        qm_status st = tn_small(most, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate, f, s);
+        return st ? st : tn_small(M - most, N, K, A + most, lda, d, alpha, B, ldb, C + (size_t)most * ldc, ldc, accumulate,
+                                  flags_from(f, most), s);
+    }
     const dim3 grid((N + kTnN - 1) / kTnN, (M + rows - 1) / rows);
+    ProfScope pf(PF_GEMM_TN, s);
     if (rows == 4) k_tn<T, 4><<<grid, 128, 0, s>>>(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate ? 1 : 0, f);
     else k_tn<T, 8><<<grid, 256, 0, s>>>(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate ? 1 : 0, f);
     return cuda_check(cudaGetLastError(), "gemm_tn launch");
