@@ -424,8 +424,11 @@ typedef struct {
  *  stream         cudaStream_t.  Synchronous with respect to the host: the call returns
  *                 after the last iteration; it reads small results (Ritz values, residual
  *                 norms) back every iteration.
- * Uses a grow-only device workspace owned by the handle (about (2 nvecx + 5 nb) npw
- * complex doubles plus O(nvecx^2)).
+ * Uses a grow-only device workspace owned by the handle: about (2 nvecx + 5 nb) npw complex
+ * doubles (7 nb with thick restarts), O(nvecx^2), and the scratch of its largest digit products
+ * (see qm_zgemm with M, N = nvecx, nvecx; 62 MB when less than that can be allocated; with
+ * fp64_exact = 1 always 62 MB).  The H psi workspace of the handle holds the same for the
+ * projector products of QM_FP64 (M, N = nproj, nb).
  * Errors: QM_ERR_ARG, QM_ERR_OOM, QM_ERR_CUDA; QM_ERR_NUMERIC (non-finite values,
  * rank-deficient start); QM_ERR_NOT_CONVERGED (max_iter reached: outputs hold the last
  * Ritz pairs).
@@ -552,8 +555,12 @@ qm_status qm_eigh_lowest(int m, int nev, const void* A, int lda, double* evals, 
  *          form's FP32 phase; FP32-level accuracy; synchronises the stream);
  *          3 = FP64 multiply-adds at every size.
  *  A, B, C device, complex double, row-major with the leading dimensions given; C is written.
- *  stream  cudaStream_t.  Partial sums, digit planes (at most about 600 MB) and tensor-core
- *          workspaces are allocated with cudaMallocAsync on the stream.
+ *  stream  cudaStream_t.  Workspaces are allocated with cudaMallocAsync on the stream.  Digit
+ *          products take, op 0: the digit planes of a panel of K, at most 512 MB, and 32 bytes per
+ *          output and split of K (M padded to 128, N to 32; at most 160 splits, as many as fill
+ *          the GPU); op 1: 56 bytes per element of A (M padded to 32, K to 8), and at most 512 MB
+ *          for a panel of B's columns.  If that much cannot be allocated, at most 62 MB: smaller
+ *          panels, or FP64 multiply-adds.
  * M, N, K >= 1.  Errors: QM_ERR_ARG, QM_ERR_CUDA, QM_ERR_OOM, QM_ERR_TIMEOUT (arith 2).
  */
 qm_status qm_zgemm(int op, int arith, int M, int N, int K, const void* A, int lda, const void* B, int ldb, void* C,

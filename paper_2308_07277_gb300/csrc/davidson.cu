@@ -525,15 +525,23 @@ extern "C" qm_status qm_davidson(qm_gspace g, int ik, int nb, void* psi_inout, i
     const size_t oCp = take(thick ? sqb : 0), oCT = take(thick ? sqb : 0), oPT = take(thick ? sqb : 0),
                  oQT = take(thick ? sqb : 0), oY = take(thick ? big * nb : 0), oHY = take(thick ? big * nb : 0);
     const bool digits = o.fp64_exact == 0;
-    const size_t part_bytes = std::max(gemm_cn_partial_bytes(false), std::max(zgemm_cn_bytes(nvx, nvx, npw, digits), zgemm_tn_bytes(nvx, npw, nvx, digits)));
-    const size_t oPart = take(part_bytes);
     const size_t oEval = take(sizeof(double) * nsq), oEps = take(sizeof(double) * (nsq + nb)),
                  oTk = take(sizeof(double) * nsq),
                  oSel = take(sizeof(int) * nsq), oRank = take(sizeof(int) * nsq), oInfo = take(sizeof(int) * 4),
                  oHeev = take(heev_work_bytes(nsq, nsq));
     const size_t oHd = take(o.precond == 1 ? sizeof(double) * npw : 0),
                  oVp = take(o.precond == 1 ? sizeof(double) * kVmeanBlocks : 0);
-    if ((st = ensure_dav_workspace(g, off, s))) return st;
+    // scratch of the FP64 products, last: less of it when the whole cannot be allocated
+    size_t part_bytes = std::max(gemm_cn_partial_bytes(false), std::max(zgemm_cn_bytes(nvx, nvx, npw, digits), zgemm_tn_bytes(nvx, npw, nvx, digits)));
+    const size_t lean_bytes = zgemm_lean_bytes(part_bytes);
+    if (g->lean) part_bytes = lean_bytes;
+    const size_t oPart = off;
+    st = ensure_dav_workspace(g, oPart + part_bytes, s);
+    if (st == QM_ERR_OOM && part_bytes > lean_bytes && !(st = ensure_dav_workspace(g, oPart + lean_bytes, s))) {
+        part_bytes = lean_bytes;
+        g->lean = true;
+    }
+    if (st) return st;
     char* base = (char*)g->dws.ptr;
     Ws& w = run.w;
     w.V = (double2*)(base + oV);

@@ -36,7 +36,8 @@ struct HpsiLayout {
     size_t vt_off, p_off, part_off, part_bytes, t_off, nl_off, err_off, total, t_bytes;
 };
 
-static HpsiLayout hpsi_layout(qm_gspace g, int ik, int nb, int nproj, bool fp32, bool own_beta, bool gamma, bool digits) {
+static HpsiLayout hpsi_layout(qm_gspace g, int ik, int nb, int nproj, bool fp32, bool own_beta, bool gamma, bool digits,
+                              bool lean) {
     HpsiLayout L{};
     const size_t cs = fp32 ? sizeof(float2) : sizeof(double2);
     const size_t rs = fp32 ? sizeof(float) : sizeof(double);
@@ -52,6 +53,7 @@ static HpsiLayout hpsi_layout(qm_gspace g, int ik, int nb, int nproj, bool fp32,
     // scratch of the projector products on the caller's stream
     const bool small = fp32 && small_nonlocal(nproj, nb, npw);
     L.part_bytes = nproj == 0 ? 0 : fp32 ? (small ? csmall_cn_bytes(nproj, nb, npw) : 0) : std::max(zgemm_cn_bytes(nproj, nb, npw, digits), zgemm_tn_bytes(nb, npw, nproj, digits));
+    if (!fp32 && lean) L.part_bytes = zgemm_lean_bytes(L.part_bytes);
     off = align_up(off + L.part_bytes, 256);
     L.t_off = off;
     // the precision form keeps every band's stick buffer (K1 and K2 of all bands overlap the
@@ -113,8 +115,14 @@ qm_status qm::hpsi_run(qm_gspace g, int ik, int nb, const void* psi, int ld_psi,
         if (p.dev && p.beta == beta && p.ld == ld_beta && p.nproj == nproj) beta_prepared = p.dev;
     }
 
-    const HpsiLayout L = hpsi_layout(g, ik, nb, nproj, fp32, beta_prepared == nullptr, gamma, digits);
-    if ((st = ensure_workspace(g, L.total, s))) return st;
+    HpsiLayout L = hpsi_layout(g, ik, nb, nproj, fp32, beta_prepared == nullptr, gamma, digits, g->lean);
+    st = ensure_workspace(g, L.total, s);
+    if (st == QM_ERR_OOM && !g->lean) {
+        const size_t full = L.total;
+        L = hpsi_layout(g, ik, nb, nproj, fp32, beta_prepared == nullptr, gamma, digits, true);
+        if (L.total < full && !(st = ensure_workspace(g, L.total, s))) g->lean = true;
+    }
+    if (st) return st;
     char* ws = (char*)g->ws.ptr;
     void* vt = ws + L.vt_off;
     void* P = ws + L.p_off;

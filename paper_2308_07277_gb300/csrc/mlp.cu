@@ -840,9 +840,10 @@ extern "C" qm_status qm_mlp_pairs(qm_gspace g, int ik, int n, const void* psi, i
     GemmWork gw;
     gw.bytes = std::max(zgemm_cn_bytes(nu, n, npw), zgemm_tn_bytes(n, npw, nu));
     DevBuf S(s), part(s), P(s), ok(s);
-    if ((st = S.get(sizeof(double2) * (size_t)nu * n)) || (gw.bytes && (st = part.get(gw.bytes))) ||
-        (st = P.get(sizeof(double2) * (size_t)n * npw)) || (st = ok.get(sizeof(int) * (size_t)n)))
+    if ((st = S.get(sizeof(double2) * (size_t)nu * n)) || (st = P.get(sizeof(double2) * (size_t)n * npw)) || (st = ok.get(sizeof(int) * (size_t)n)))
         return st;
+    if (gw.bytes && (st = part.get(gw.bytes)) == QM_ERR_OOM) st = part.get(gw.bytes = zgemm_lean_bytes(gw.bytes));
+    if (st) return st;
     gw.ptr = part.p;
     if ((st = zgemm_cn(nu, n, npw, (const double2*)U, ld_u, (const double2*)psi, ld_psi, (double2*)S.p, n, gw, s)))
         return st;

@@ -96,6 +96,7 @@ struct qm_gspace_s {
     std::vector<qm::NlPrep> prep;  // per k-point prepared projectors (qm_hpsi_prepare)
     qm::Workspace ws;    // qm_hpsi workspace
     qm::Workspace dws;   // qm_davidson workspace
+    bool lean = false;   // the digit products' full scratch could not be had once: zgemm_lean_bytes of it since
     // second stream of qm_hpsi(QM_MIXED): the tensor-core nonlocal part runs on it while the
     // FFT path runs on the caller's stream (fork / join events); created with the tables
     cudaStream_t aux = nullptr;
@@ -241,6 +242,8 @@ struct GemmFlags {
 };
 size_t zgemm_cn_bytes(int M, int N, int K, bool digits = true);
 size_t zgemm_tn_bytes(int M, int N, int K, bool digits = true);
+// what is asked for instead when that much cannot be allocated: no more than the FP64 kernels' partial sums
+size_t zgemm_lean_bytes(size_t bytes);
 // C[m][n] = sum_k conj(A[m][k]) * B[n][k]   (A: M rows, B: N rows, k contiguous);
 // split over K into partial sums reduced in a fixed order (deterministic).
 qm_status zgemm_cn(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb,

@@ -513,6 +513,8 @@ size_t zgemm_cn_bytes(int M, int N, int K, bool digits) {
 }
 size_t zgemm_tn_bytes(int M, int N, int K, bool digits) { return M <= 0 || N <= 0 || !digits ? 0 : zdigits_bytes(false, M, N, K); }
 
+size_t zgemm_lean_bytes(size_t bytes) { return std::min(bytes, gemm_cn_partial_bytes(false)); }
+
 qm_status zgemm_cn(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb, double2* C, int ldc,
                    const GemmWork& w, cudaStream_t s) {
     if (M <= 0 || N <= 0) return QM_OK;
@@ -600,11 +602,15 @@ extern "C" qm_status qm_zgemm(int op, int arith, int M, int N, int K, const void
     }
     GemmWork w;
     w.digits = arith != 3;
-    const size_t bytes = op == 0 ? zgemm_cn_bytes(M, N, K, w.digits) : zgemm_tn_bytes(M, N, K, w.digits);
-    w.bytes = bytes;
-    if (bytes && cudaMallocAsync(&w.ptr, bytes, s) != cudaSuccess) {
+    w.bytes = op == 0 ? zgemm_cn_bytes(M, N, K, w.digits) : zgemm_tn_bytes(M, N, K, w.digits);
+    if (w.bytes && cudaMallocAsync(&w.ptr, w.bytes, s) != cudaSuccess) {
         cudaGetLastError();
-        return fail(QM_ERR_OOM, "qm_zgemm: workspace");
+        w.ptr = nullptr;
+        w.bytes = zgemm_lean_bytes(w.bytes);
+        if (cudaMallocAsync(&w.ptr, w.bytes, s) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(QM_ERR_OOM, "qm_zgemm: workspace");
+        }
     }
     qm_status st = op == 0 ? zgemm_cn(M, N, K, a, lda, b, ldb, c, ldc, w, s)
                            : zgemm_tn(M, N, K, a, lda, nullptr, b, ldb, c, ldc, false, w, s, 1.0);
