@@ -96,6 +96,9 @@ __device__ __forceinline__ float row_scale(int hmax) {
     return __uint_as_float((uint32_t)(k + 127) << 23);
 }
 __device__ __forceinline__ float inv_scale(float s) { return __uint_as_float((254u << 23) - __float_as_uint(s)); }
+// a product of scaled operands times both inverse scales, the smaller first: large rows against small ones
+// give an ordinary number, but the larger scale alone could take it past FP32's range
+__device__ __forceinline__ float unscale(float a, float s, float t) { return a * fminf(s, t) * fmaxf(s, t); }
 __device__ __forceinline__ int f_abs(float x) { return __float_as_int(x) & 0x7FFFFFFF; }
 // The kernels of one call form a chain whose members are launched while the one before still runs
 // (launch_chained) and wait for its results here.  What the kernel before wrote is read by volatile loads:
@@ -288,7 +291,7 @@ __global__ void __launch_bounds__(256) k_reduce_p(const float* __restrict__ part
     if (w == 0 && e < total) {
 #pragma unroll
         for (int i = 1; i < 8; ++i) a += red[i][threadIdx.x];
-        Pd[e] = a * __ldg(inv_p + p) * ld_dep(inv_b + (c >> 1)) * (float)__ldg(D + p);
+        Pd[e] = unscale(a, __ldg(inv_p + p), ld_dep(inv_b + (c >> 1))) * (float)__ldg(D + p);
     }
 }
 
@@ -330,8 +333,8 @@ __global__ void __launch_bounds__(256) k_expand_e(const float* __restrict__ Pd, 
                 a.y += v.y;
             }
             const float ip = __ldg(inv_p + p), d = (float)__ldg(D + p);
-            a.x = a.x * ip * ib * d;
-            a.y = a.y * ip * ib * d;
+            a.x = unscale(a.x, ip, ib) * d;
+            a.y = unscale(a.y, ip, ib) * d;
         }
         sp[p * 4 + q4] = a;
         h = max(h, max(f_abs(a.x), f_abs(a.y)));
@@ -527,8 +530,8 @@ k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__
                                 const float in = __ldg(inv_n + g);
                                 float2 o = t ? make_float2(y[j], __uint_as_float(v[8 + j]))
                                              : make_float2(__uint_as_float(v[j]), y[j]);
-                                o.x = o.x * im * in;
-                                o.y = o.y * im * in;
+                                o.x = unscale(o.x, im, in);
+                                o.y = unscale(o.y, im, in);
                                 if (accumulate) {
                                     const float2 a = orow[g];
                                     o.x += a.x;
