@@ -356,7 +356,8 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
     // (a non-finite matrix is left as it is; a zero one has nothing to scale)
     int ex = (s_max >> 20) - 1023;  // the largest component is in [2^ex, 2^(ex+1))
     const bool scaled = (ex < -kTriRange || ex > kTriRange) && ex < 1024 && s_max > 0;
-    const double up = scaled ? ldexp(1.0, max(-1000, min(1000, -ex))) : 1.0, back = scaled ? 1.0 / up : 1.0;
+    const int shift = scaled ? max(-1000, min(1000, -ex)) : 0;
+    const double up = __hiloint2double((1023 + shift) << 20, 0), back = __hiloint2double((1023 - shift) << 20, 0);
     if (scaled) {
         for (int i = tid; i < m * m; i += 256) {
             double2& x = a[(i / m) * ld + i % m];
@@ -365,7 +366,9 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
         }
         ex = 0;
     }
-    const double drop = ldexp(1.0, 2 * (ex - kTriDrop));  // on the square of a column's norm
+    // high word of the bound on the square of a column's norm (compared as integers: a comparison of doubles
+    // holds the pipe like any other FP64 instruction)
+    const int drop = max(0, min(2046, 1023 + 2 * (ex - kTriDrop))) << 20;
     // the reflector of column k but for tau (one warp)
     auto reflector = [&](int k) {
         const int n = m - k - 1;
@@ -379,7 +382,7 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
         }
         for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
         const double2 alpha = a[(k + 1) * ld + k];
-        const bool none = part < drop;
+        const bool none = __double2hiint(part) < drop;
         double beta = 0.0;
         if (__any_sync(0xffffffffu, below) && !none) beta = -copysign(sqrt(part), alpha.x);
         for (int i = lane; i < n; i += 32) {
@@ -476,7 +479,10 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
         }
     }
     __syncthreads();
-    if (tid == 0) d[m - 1] = a[(m - 1) * ld + m - 1].x * back;
+    if (tid == 0) {
+        const double x = a[(m - 1) * ld + m - 1].x;
+        d[m - 1] = scaled ? x * back : x;
+    }
 }
 
 // number of eigenvalues of T smaller than x: sign changes of the leading minors' determinants by their
