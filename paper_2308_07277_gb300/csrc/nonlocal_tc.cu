@@ -127,13 +127,12 @@ __device__ __forceinline__ int max_segs(const int* __restrict__ emax, int n, int
     return h;
 }
 
-// largest magnitude (bits) of each row of src over column segment blockIdx.y
-__global__ void __launch_bounds__(256) k_nl_rowmax(const float2* __restrict__ src, int ld, int rows, int cols,
-                                                   int* __restrict__ emax) {
+// largest magnitude (bits) of row r of src over column segment seg (one CTA)
+__device__ __forceinline__ void nl_rowmax(const float2* __restrict__ src, int ld, int rows, int cols, int* __restrict__ emax, int r,
+                                          int seg) {
     __shared__ int red[8];
-    chain_next();
-    const int r = blockIdx.x, per = (cols + kNlSegs - 1) / kNlSegs;
-    const int c0 = blockIdx.y * per, c1 = min(cols, c0 + per);
+    const int per = (cols + kNlSegs - 1) / kNlSegs;
+    const int c0 = seg * per, c1 = min(cols, c0 + per);
     const float2* p = src + (size_t)r * ld;
     int h = 0;
 #pragma unroll 4
@@ -147,44 +146,55 @@ __global__ void __launch_bounds__(256) k_nl_rowmax(const float2* __restrict__ sr
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int w = 1; w < 8; ++w) h = max(h, red[w]);
-        emax[(size_t)blockIdx.y * rows + r] = h;
+        emax[(size_t)seg * rows + r] = h;
     }
 }
-// the same per column of src [K][cols] over K segment blockIdx.y
-__global__ void __launch_bounds__(256) k_nl_colmax(const float2* __restrict__ src, int ld, int K, int cols,
-                                                   int* __restrict__ emax) {
-    const int c = blockIdx.x * 256 + threadIdx.x, per = (K + kNlSegs - 1) / kNlSegs;
+// the same per column of src [K][cols] over K segment seg, columns from 256 cb on
+__device__ __forceinline__ void nl_colmax(const float2* __restrict__ src, int ld, int K, int cols, int* __restrict__ emax, int cb,
+                                          int seg) {
+    const int c = cb * 256 + threadIdx.x, per = (K + kNlSegs - 1) / kNlSegs;
     if (c >= cols) return;
-    const int k0 = blockIdx.y * per, k1 = min(K, k0 + per);
+    const int k0 = seg * per, k1 = min(K, k0 + per);
     int h = 0;
 #pragma unroll 8
     for (int k = k0; k < k1; ++k) {
         const float2 v = __ldg(src + (size_t)k * ld + c);
         h = max(h, max(f_abs(v.x), f_abs(v.y)));
     }
-    emax[(size_t)blockIdx.y * cols + c] = h;
+    emax[(size_t)seg * cols + c] = h;
+}
+__global__ void __launch_bounds__(256) k_nl_rowmax(const float2* __restrict__ src, int ld, int rows, int cols,
+                                                   int* __restrict__ emax) {
+    chain_next();
+    nl_rowmax(src, ld, rows, cols, emax, blockIdx.x, blockIdx.y);
+}
+// both of the projectors: the first `rows` blocks of x the rows, the others the columns
+__global__ void __launch_bounds__(256) k_nl_maxima(const float2* __restrict__ src, int ld, int rows, int cols,
+                                                   int* __restrict__ erow, int* __restrict__ ecol) {
+    chain_next();
+    if ((int)blockIdx.x < rows) nl_rowmax(src, ld, rows, cols, erow, blockIdx.x, blockIdx.y);
+    else nl_colmax(src, ld, rows, cols, ecol, blockIdx.x - rows, blockIdx.y);
 }
 
 // Rows of complex src (K = 2 ncols interleaved reals) -> blocked split operand.  expand = 0:
 // row r is src row r as stored; expand = 1: rows 2b, 2b+1 are src row b as stored and its
 // rotation (im, -re).  Rows >= nsrc (resp. 2 nsrc) and K beyond 2 ncols are written as zeros.
-// CTA: 8 rows (one core-matrix row group, blockIdx.y) x 32 chunks of 8 K values (blockIdx.x);
+// CTA: 8 rows (one core-matrix row group, by) x 32 chunks of 8 K values (bx);
 // the 8 rows of a core matrix on consecutive threads (one 128-byte run per plane), the 2
 // chunks of a K tile on consecutive thread octets.  inv: the source rows' inverse scales.
 constexpr int kSplitChunks = 32;
 constexpr int kFoldReduce = 1024;  // projectors x splits up to which the expansion sums the splits (one CTA per 4 bands)
 constexpr int kSelfScale = 2048;  // plane waves up to which a row's scale is found in its splitting CTA
-__global__ void __launch_bounds__(256) k_split_rows(const float2* __restrict__ src, int ld, int nsrc, int ncols,
-                                                    int expand, int R, int nkt, const int* __restrict__ emax,
-                                                    float* __restrict__ inv, unsigned char* __restrict__ blk) {
-    chain_wait();
-    const int r = blockIdx.y * 8 + (threadIdx.x & 7);
-    int ch = blockIdx.x * kSplitChunks + (threadIdx.x >> 3);
+__device__ __forceinline__ void split_rows(const float2* __restrict__ src, int ld, int nsrc, int ncols, int expand, int R, int nkt,
+                                           const int* __restrict__ emax, float* __restrict__ inv, unsigned char* __restrict__ blk,
+                                           int bx, int by) {
+    const int r = by * 8 + (threadIdx.x & 7);
+    int ch = bx * kSplitChunks + (threadIdx.x >> 3);
     const int b = expand ? (r >> 1) : r;
     float sc = 1.f;
     if (!emax) {  // short rows, one CTA per row group: the rows' largest values are found here
         __shared__ int smax[8];
-        const int nrow = expand ? 4 : 8, l = threadIdx.x & 31, b0 = blockIdx.y * nrow;
+        const int nrow = expand ? 4 : 8, l = threadIdx.x & 31, b0 = by * nrow;
         for (int q = threadIdx.x >> 5; q < nrow; q += 8) {
             int h = 0;
             if (b0 + q < nsrc)
@@ -242,11 +252,11 @@ __global__ void __launch_bounds__(256) k_split_rows(const float2* __restrict__ s
 // CTA tile: 64 rows g x 16 projectors (two K tiles), transposed through shared memory so the
 // global reads run along g.  Rows g >= G (up to rows_pad) and p >= P are zeros.
 constexpr int kTG = 64, kTP = 16;
-__global__ void __launch_bounds__(256) k_split_t(const float2* __restrict__ beta, int ld, int P, int G, int R, int nkt,
-                                                 const int* __restrict__ emax, float* __restrict__ inv,
-                                                 unsigned char* __restrict__ blk) {
+__device__ __forceinline__ void split_t(const float2* __restrict__ beta, int ld, int P, int G, int R, int nkt,
+                                        const int* __restrict__ emax, float* __restrict__ inv, unsigned char* __restrict__ blk,
+                                        int bx, int by) {
     __shared__ float2 t[kTP][kTG + 1];
-    const int g0 = blockIdx.x * kTG, p0 = blockIdx.y * kTP;
+    const int g0 = bx * kTG, p0 = by * kTP;
     for (int i = threadIdx.x; i < kTP * kTG; i += blockDim.x) {
         const int pp = i / kTG, gg = i - pp * kTG;
         const int p = p0 + pp, g = g0 + gg;
@@ -257,8 +267,8 @@ __global__ void __launch_bounds__(256) k_split_t(const float2* __restrict__ beta
     const int rlo = threadIdx.x & 7, ch = (threadIdx.x >> 3) & 3, rg = threadIdx.x >> 5;
     const int gg = rg * 8 + rlo, g = g0 + gg;
     const float sc = g < G ? row_scale(max_segs(emax, G, g)) : 1.f;
-    if (blockIdx.y == 0 && ch == 0 && g < G) inv[g] = inv_scale(sc);
-    if ((int)blockIdx.y * 2 + (ch >> 1) >= nkt) return;
+    if (by == 0 && ch == 0 && g < G) inv[g] = inv_scale(sc);
+    if (by * 2 + (ch >> 1) >= nkt) return;
     float v[8];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -267,6 +277,29 @@ __global__ void __launch_bounds__(256) k_split_t(const float2* __restrict__ beta
         v[2 * j + 1] = x.y;
     }
     put8(blk, R, nkt, g, p0 * 2 + ch * 8, v, sc);
+}
+
+__global__ void __launch_bounds__(256) k_split_rows(const float2* __restrict__ src, int ld, int nsrc, int ncols,
+                                                    int expand, int R, int nkt, const int* __restrict__ emax,
+                                                    float* __restrict__ inv, unsigned char* __restrict__ blk) {
+    chain_wait();
+    split_rows(src, ld, nsrc, ncols, expand, R, nkt, emax, inv, blk, blockIdx.x, blockIdx.y);
+}
+// both layouts of the projectors beta [P][G]: the first nxk * nyk blocks betaK (nxk blocks per row group), the
+// others betaT (nxt blocks of columns)
+__global__ void __launch_bounds__(256) k_split_beta(const float2* __restrict__ beta, int ld, int P, int G, int nxk, int nyk, int nktk,
+                                                    const int* __restrict__ ek, float* __restrict__ invk,
+                                                    unsigned char* __restrict__ blkk, int nxt, int Rt, int nktt,
+                                                    const int* __restrict__ et, float* __restrict__ invt,
+                                                    unsigned char* __restrict__ blkt) {
+    chain_wait();
+    int b = blockIdx.x;
+    if (b < nxk * nyk) {
+        split_rows(beta, ld, P, G, 0, TM, nktk, ek, invk, blkk, b % nxk, b / nxk);
+    } else {
+        b -= nxk * nyk;
+        split_t(beta, ld, P, G, Rt, nktt, et, invt, blkt, b % nxt, b / nxt);
+    }
 }
 
 // sum the split-K partials of the projection C[z][p][c] (FP32, ldc; c = 2b + t) in a fixed order,
@@ -492,6 +525,9 @@ k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__
         if (__all_sync(0xffffffffu, ok && nk > 0 && !*abort) && u < nsub) {
             const int mrow = (mt + u) * TM + q * 32 + lane;  // this thread's accumulator row
             const float im = EPI == 1 && mrow < M ? ld_dep(inv_m + (mrow >> 1)) : 1.f;
+            // (as unscale: the row's scale before the column's if it is below one, else after it)
+            const float im_lo = fminf(im, 1.f), im_hi = fmaxf(im, 1.f);
+            const bool low = __all_sync(0xffffffffu, im <= 1.f);
 #pragma unroll 1
             for (int c0 = 0; c0 < BN; c0 += 16) {
                 uint32_t v[16];
@@ -527,11 +563,15 @@ k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__
                         for (int j = 0; j < 8; ++j) {
                             const int g = g0 + j;
                             if (g < N) {
-                                const float in = __ldg(inv_n + g);
+                                const float in = __ldg(inv_n + g) * im_lo;
                                 float2 o = t ? make_float2(y[j], __uint_as_float(v[8 + j]))
                                              : make_float2(__uint_as_float(v[j]), y[j]);
-                                o.x = unscale(o.x, im, in);
-                                o.y = unscale(o.y, im, in);
+                                o.x *= in;
+                                o.y *= in;
+                                if (!low) {
+                                    o.x *= im_hi;
+                                    o.y *= im_hi;
+                                }
                                 if (accumulate) {
                                     const float2 a = orow[g];
                                     o.x += a.x;
@@ -652,34 +692,6 @@ qm_status check_limits(const NlLayout& L) {
     return QM_OK;
 }
 
-qm_status split_beta(int nproj, int npw, const float2* beta, int ld_beta, const NlLayout& L, unsigned char* base, cudaStream_t s) {
-    float* invk = (float*)(base + L.inv_off);
-    float* invt = invk + nproj;
-    int* ek = (int*)(invt + npw);
-    int* et = ek + (size_t)kNlSegs * nproj;
-    {
-        ProfScope pf(PF_SPLIT, s);
-        k_nl_rowmax<<<dim3((unsigned)nproj, kNlSegs), 256, 0, s>>>(beta, ld_beta, nproj, npw, ek);
-    }
-    {
-        ProfScope pf(PF_SPLIT, s);
-        k_nl_colmax<<<dim3((unsigned)((npw + 255) / 256), kNlSegs), 256, 0, s>>>(beta, ld_beta, nproj, npw, et);
-    }
-    {
-        ProfScope pf(PF_SPLIT, s);
-        const dim3 grid((unsigned)((L.nkt_p * (KT / 8) + kSplitChunks - 1) / kSplitChunks), (unsigned)(L.mtile_p * TM / 8));
-        k_split_rows<<<grid, 256, 0, s>>>(beta, ld_beta, nproj, npw, 0, TM, L.nkt_p, ek, invk, base + L.betaK_off);
-    }
-    qm_status st = cuda_check(cudaGetLastError(), "k_split_rows launch");
-    if (st) return st;
-    {
-        ProfScope pf(PF_SPLIT, s);
-        dim3 grid((unsigned)(L.ntile_a * kAppBN / kTG), (unsigned)((L.nkt_a + 1) / 2));
-        k_split_t<<<grid, 256, 0, s>>>(beta, ld_beta, nproj, npw, kAppBN, L.nkt_a, et, invt, base + L.betaT_off);
-    }
-    return cuda_check(cudaGetLastError(), "k_split_t launch");
-}
-
 // Launch while the kernel before in the stream still runs (programmatic dependent launch): its last CTAs, the
 // launch and the set-up of this one overlap, 1 to 2 us at each link of the chain (64 atoms: 2 bands 73.6 ->
 // 64.6 us, 24 bands 107 -> 98; 128 bands 427 -> 420).  The kernel calls chain_wait before it uses or
@@ -699,6 +711,23 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t 
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+qm_status split_beta(int nproj, int npw, const float2* beta, int ld_beta, const NlLayout& L, unsigned char* base, cudaStream_t s) {
+    float* invk = (float*)(base + L.inv_off);
+    float* invt = invk + nproj;
+    int* ek = (int*)(invt + npw);
+    int* et = ek + (size_t)kNlSegs * nproj;
+    {
+        ProfScope pf(PF_SPLIT, s);
+        k_nl_maxima<<<dim3((unsigned)(nproj + (npw + 255) / 256), kNlSegs), 256, 0, s>>>(beta, ld_beta, nproj, npw, ek, et);
+    }
+    const int nxk = (L.nkt_p * (KT / 8) + kSplitChunks - 1) / kSplitChunks, nyk = L.mtile_p * TM / 8;
+    const int nxt = L.ntile_a * kAppBN / kTG, nyt = (L.nkt_a + 1) / 2;
+    ProfScope pf(PF_SPLIT, s);
+    return cuda_check(launch_chained(k_split_beta, dim3((unsigned)((long)nxk * nyk + (long)nxt * nyt)), 256, 0, s, beta, ld_beta, nproj,
+                                     npw, nxk, nyk, L.nkt_p, ek, invk, base + L.betaK_off, nxt, kAppBN, L.nkt_a, et, invt,
+                                     base + L.betaT_off), "k_split_beta launch");
 }
 
 template <int EPI>
