@@ -25,12 +25,14 @@ constexpr size_t kStickBudget = 48ull << 20;
 constexpr size_t kStickBudgetOverlap = 1ull << 30;
 
 // Whether the precision form's nonlocal part is small enough for FP32 products on the CUDA cores, on the
-// caller's stream: the tensor-core chain is five or six launches (nine where the projectors are split on
+// caller's stream: the tensor-core chain is five or six launches (two more where the projectors are split on
 // the call) behind a fork and before a join.  With the chain's early launches the tensor cores win from about
 // 1.5e6 (nproj nb npw) on: whole call, CUDA cores / tensor cores, us: 1.3e6 41 / about 40, 3.4e6 54 / 48; a
 // propagation step of 16 atoms with 10 bands (3.1e6, four H psi) 269 / 189.  One line for prepared and split
 // projectors, so that preparing them does not change the result.
-static bool small_nonlocal(int nproj, int nb, int npw) { return (double)nproj * nb * npw <= 1.5e6; }
+// Up to 16 projectors (four atoms) always: the split products' 23 bits would show beside the FFT path's error
+// (16 x 128 x 808: 4.95e-8, FP32 4.72e-8); 71 us instead of 61, 141 instead of 130 with 400 bands.
+static bool small_nonlocal(int nproj, int nb, int npw) { return nproj <= 16 || (double)nproj * nb * npw <= 1.5e6; }
 
 struct HpsiLayout {
     size_t vt_off, p_off, part_off, part_bytes, t_off, nl_off, err_off, total, t_bytes;

@@ -11,7 +11,13 @@
 // every sum it adds to an accumulator, 12 sums per 32 terms with six products, 6 with three (and
 // the projection's K is split twice as often).  Measured error of H psi against 64 bits, six BF16
 // products / these: 3.5e-6 / 1.4e-6 (255 atoms), 5.3e-6 / 2.2e-6 (216 atoms), 3.1e-7 / 1.5e-7 (64 atoms),
-// 8.9e-8 / 8.0e-8 (32 atoms), 5.7e-8 / 6.2e-8 (8 atoms, where the FP32 path below hpsi.cu's line has 4.7e-8).
+// 8.9e-8 / 8.0e-8 (32 atoms).  With fewer projectors the six were ahead: 7.4e-8 / 9.1e-8 with 32 of them (1060
+// plane waves, 56 to 90 bands; FP32 arithmetic 4.6e-8).  Up to kFewProj projectors the two small products
+// therefore go to accumulators of their own, so that the large one is truncated once per K tile instead of three
+// times, and both are added in the epilogue: 5.7e-8.  It halves the error of larger ones too, but doubles the tensor
+// memory and the drain (propagation step of 32 atoms 1046 -> 1066 us), and their error is below the six
+// products' as it is.  (x1 y1 as a fourth product on top: 5.6e-8, no difference.)  Up to 16 projectors the 23 bits
+// themselves show beside the FFT path's error (4.95e-8, six products 4.77e-8): hpsi.cu keeps those in FP32.
 //
 // Operands are split ONCE into FP16 planes stored in global memory in a tile-blocked order:
 // block (row tile, K tile) holds, for both planes, the R x 16 tile in the canonical no-swizzle
@@ -412,7 +418,7 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile
 // bsub parts per CTA.  EPI 0: C is FP32 [m][n] (ldc) at
 // C + z*zstride (split-K partials, operands' scales not undone); EPI 1: row m = 2b + t, column g -> complex
 // out[b][g] component t (ldc = complex row stride) times inv_m[b] inv_n[g], accumulate: add to out.
-template <int EPI>
+template <int EPI, bool kDual>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__ B, int nkt, int BN, int bsub, int msub, int M,
           int N, int mtiles, int kt_per_split, float* __restrict__ C, size_t ldc, size_t zstride, int accumulate,
@@ -435,7 +441,7 @@ k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__
     const uint32_t acols = BN <= 32 ? 32 : BN <= 64 ? 64 : BN <= 128 ? 128 : 256;  // columns between the accumulators
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(tc::smem_u32(&tmem_base)),
-                     "r"(msub * acols));
+                     "r"(kDual ? 2 * msub * acols : msub * acols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
     }
     if (tid == 0) {
@@ -498,10 +504,11 @@ k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__
                 for (int q = 0; q < 3; ++q) {
                     const uint64_t da = tc::sdesc(sa + u * a_bytes + pa[q] * (uint32_t)plane_bytes(TM), 128, 256);
                     const uint64_t db = tc::sdesc(sb + pb[q] * (uint32_t)plane_bytes(BN), 128, 256);
-                    const uint32_t acc = (it > 0 || q > 0) ? 1u : 0u;
+                    const uint32_t acc = (it > 0 || q == 1 || (q == 2 && !kDual)) ? 1u : 0u;
+                    const uint32_t td = tmem + (kDual && q < 2 ? u + msub : u) * acols;
                     asm volatile(
                         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + u * acols),
+                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(td),
                         "l"(da), "l"(db), "r"(idesc), "r"(acc));
                 }
             }
@@ -539,7 +546,21 @@ k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__
                       "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
                       "=r"(v[15])
                     : "r"(taddr));
-                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                if (!kDual) {
+                    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                } else {
+                    uint32_t x[16];
+                    asm volatile(
+                        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+                        "%13, %14, %15}, [%16];\n"
+                        : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7]),
+                          "=r"(x[8]), "=r"(x[9]), "=r"(x[10]), "=r"(x[11]), "=r"(x[12]), "=r"(x[13]), "=r"(x[14]),
+                          "=r"(x[15])
+                        : "r"(taddr + msub * acols));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(x[j]));
+                }
                 const int n0 = nt * BN + c0;
                 if (EPI == 0) {
                     if (mrow < M) {
@@ -599,7 +620,7 @@ k_nl_gemm(const unsigned char* __restrict__ A, const unsigned char* __restrict__
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
     __syncthreads();
-    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(msub * acols));
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kDual ? 2 * msub * acols : msub * acols));
 }
 
 inline size_t rup(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -617,9 +638,11 @@ constexpr int kAppBN = 256;
 // operands at 45 bytes per clock, at least the 400 a step takes), plus start, fill and drain.
 struct GemmShape {
     int msub, bsub, splits;
+    bool dual;  // the small terms in accumulators of their own
 };
-GemmShape gemm_shape(int mtiles, int ntiles, int BN, int nkt, int max_bsub, int max_splits) {
-    GemmShape best{std::min(2, mtiles), 1, 1};
+constexpr int kFewProj = 48;  // projectors up to which they are (64: 1.3e-7 with six products, 9.9e-8 in one accumulator)
+GemmShape gemm_shape(int mtiles, int ntiles, int BN, int nkt, int max_bsub, int max_splits, bool few) {
+    GemmShape best{1, 1, 1, few};
     double cost = -1;
     const int sms = device_sms();
     for (int msub = std::min(2, mtiles); msub >= 1; --msub)
@@ -628,15 +651,16 @@ GemmShape gemm_shape(int mtiles, int ntiles, int BN, int nkt, int max_bsub, int 
             const int sp = (int)std::max<long>(1, std::min<long>({(long)max_splits, (long)std::max(1, nkt / 8), sms / tiles}));
             const int per = (nkt + sp - 1) / sp, m = std::min(msub, mtiles), bn = BN / bsub;
             const double tile = std::max(1.5 * m * bn, (m * 8192.0 + bn * 64.0) / 45.0);
+            if (few && 2 * msub * (bn <= 32 ? 32 : bn <= 64 ? 64 : bn <= 128 ? 128 : 256) > 512) continue;  // (bn and msub halve)
             // CTAs an SM holds, by shared memory and tensor memory; more than one share its throughput
-            const int cols = msub * (bn <= 32 ? 32 : bn <= 64 ? 64 : bn <= 128 ? 128 : 256);
+            const int cols = (few ? 2 : 1) * msub * (bn <= 32 ? 32 : bn <= 64 ? 64 : bn <= 128 ? 128 : 256);
             const long occ = std::min<long>((226 << 10) / (long)(kNlStages * (msub * block_bytes(TM) + block_bytes(bn))), 512 / cols);
             const long n = tiles * sp;
             const double load = occ > 1 ? std::max(1.0, (double)n / sms) : (double)((n + sms - 1) / sms);
             const double c = std::max(load * per * tile, (double)((n + sms * occ - 1) / (sms * occ)) * per * std::max(tile, 400.0)) + 6000.0;
             if (cost < 0 || c < cost) {
                 cost = c;
-                best = GemmShape{msub, bsub, (nkt + per - 1) / per};
+                best = GemmShape{msub, bsub, (nkt + per - 1) / per, few};
             }
         }
     return best;
@@ -660,8 +684,9 @@ NlLayout nl_layout(int nproj, int nb, int npw, bool with_beta) {
     L.mtile_a = (2 * nb + TM - 1) / TM;
     L.ntile_a = (npw + kAppBN - 1) / kAppBN;
     L.nkt_a = (int)(rup(2 * (size_t)nproj, KT) / KT);
-    L.sp = gemm_shape(L.mtile_p, L.ntile_p, L.bn_p, L.nkt_p, 1, kMaxUmmaSplits);
-    L.sa = gemm_shape(L.mtile_a, L.ntile_a, kAppBN, L.nkt_a, 4, 1);
+    const bool few = nproj <= kFewProj;
+    L.sp = gemm_shape(L.mtile_p, L.ntile_p, L.bn_p, L.nkt_p, 1, kMaxUmmaSplits, few);
+    L.sa = gemm_shape(L.mtile_a, L.ntile_a, kAppBN, L.nkt_a, 4, 1, few);
     L.splits = L.sp.splits;
     L.zstride = (size_t)L.mtile_p * TM * L.ntile_p * L.bn_p;
     size_t off = 0;
@@ -738,11 +763,12 @@ qm_status gemm_launch(const unsigned char* A, const unsigned char* B, int nkt, i
     const size_t stage = sh.msub * block_bytes(TM) + block_bytes(bn);
     const int mg = (mt + sh.msub - 1) / sh.msub, ng = ntl * sh.bsub;
     const size_t smem = kNlStages * stage;
-    qm_status st = allow_dynamic_smem((const void*)k_nl_gemm<EPI>, smem, "tensor-core nonlocal GEMM shared memory");
+    const auto kern = sh.dual ? k_nl_gemm<EPI, true> : k_nl_gemm<EPI, false>;
+    qm_status st = allow_dynamic_smem((const void*)kern, smem, "tensor-core nonlocal GEMM shared memory");
     if (st) return st;
     ProfScope pf(PF_UMMA, s);
     const dim3 grid = EPI == 0 ? dim3(ng, mg, sh.splits) : dim3(mg, ng, sh.splits);
-    st = cuda_check(launch_chained(k_nl_gemm<EPI>, grid, kGemmThreads, smem, s, A, B, nkt, bn, sh.bsub, sh.msub, M, N, mt, per, C,
+    st = cuda_check(launch_chained(kern, grid, kGemmThreads, smem, s, A, B, nkt, bn, sh.bsub, sh.msub, M, N, mt, per, C,
                                    ldc, zstride, accumulate ? 1 : 0, inv_m, inv_n, err), "k_nl_gemm launch");
     if (st) return st;
     return cuda_check(cudaGetLastError(), "k_nl_gemm launch");

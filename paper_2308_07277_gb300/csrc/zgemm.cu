@@ -220,6 +220,12 @@ k_gemm_tn(int M, int N, int K, const float2* __restrict__ A, int lda, const doub
 // two steps 1249 -> 164 ms, H psi of the two-atom cell (8 x 8 x 411) 518 -> 65 us, and at large
 // sizes 1.22 instead of 1.01 TFLOP/s (480 x 157 x 18232, 10.9 -> 9.0 ms).
 constexpr int kCnTile = 8, kCnK = 32, kCnGroups = 4;
+// hi + lo <- hi + lo + a, hi the rounded sum (the error of the addition by Knuth's two-sum goes to lo)
+__device__ __forceinline__ void add_comp(float& hi, float& lo, float a) {
+    const float s = hi + a, t = s - hi;
+    lo += (hi - (s - t)) + (a - t);
+    hi = s;
+}
 template <class C>
 __global__ void __launch_bounds__(NTH)
 k_cn(int M, int N, int K, const C* __restrict__ A, int lda, const C* __restrict__ B, int ldb, C* __restrict__ out, int ldo, int kchunk, const GemmFlags f) {
@@ -229,7 +235,7 @@ k_cn(int M, int N, int K, const C* __restrict__ A, int lda, const C* __restrict_
     const int m0 = blockIdx.y * kCnTile, n0 = blockIdx.x * kCnTile;
     const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
     const int lrow = tid / kCnK, lk = tid % kCnK;  // this thread's element of a tile (one row per warp)
-    C acc = czero<C>();
+    C acc = czero<C>(), hi = acc, lo = acc;
     const bool va = m0 + lrow < M, vb = n0 + lrow < N;
     const C* pa = A + (size_t)(va ? m0 + lrow : 0) * lda + lk;
     const C* pb = B + (size_t)(vb ? n0 + lrow : 0) * ldb + lk;
@@ -253,7 +259,16 @@ k_cn(int M, int N, int K, const C* __restrict__ A, int lda, const C* __restrict_
             acc.x = fma(a.x, b.x, fma(a.y, b.y, acc.x));
             acc.y = fma(a.x, b.y, fma(-a.y, b.x, acc.y));
         }
+        if constexpr (sizeof(C) == sizeof(float2)) {  // the tiles' sums compensated: K / 32 of them without their rounding
+            add_comp(hi.x, lo.x, acc.x);
+            add_comp(hi.y, lo.y, acc.y);
+            acc = czero<C>();
+        }
         __syncthreads();
+    }
+    if constexpr (sizeof(C) == sizeof(float2)) {
+        acc.x = hi.x + lo.x;
+        acc.y = hi.y + lo.y;
     }
     C* red = &As[0][0];  // 3 x 64 partial sums of the K groups, added in group order
     if (kg) red[(kg - 1) * 64 + ty * 8 + tx] = acc;
@@ -534,8 +549,10 @@ qm_status zgemm_tn(int M, int N, int K, const double2* A, int lda, const double*
     if (st) return st;
     return tn_small(M, N, K, A, lda, d, alpha, B, ldb, C, ldc, accumulate, f, s);
 }
-// FP32 products on the same small tiles (the precision form's nonlocal part of small cells): sums of at
-// most a few tens of terms per thread, then of the groups and splits, in FP32
+// FP32 products on the same small tiles (the precision form's nonlocal part of small cells).  cn: chains of eight
+// multiply-adds per thread, the sums of K / 32 of them compensated, then four groups and at most 64 splits in FP32;
+// without the compensation a split of several hundred terms showed (8 x 200 x 401: 4.86e-8 of H psi, now 4.54e-8).
+// tn: one chain of K multiply-adds
 size_t csmall_cn_bytes(int M, int N, int K) {
     const int splits = zcn_splits(M, N, K, 64, 12);
     return splits > 1 ? (size_t)splits * M * N * sizeof(float2) : 0;
