@@ -348,7 +348,7 @@ struct DavidsonRun {
             qm_status s2;
             int kk = 0;
             if ((s2 = zgemm_cn(n, n, m, src, nsq, src, nsq, w.G, n, w.part, s)) ||
-                (s2 = chol_transform(w.G, n, n, drop, w.sel, w.rank, w.info, w.A, w.Z, 0, s)) ||
+                (s2 = chol_transform(w.G, n, n, drop, w.sel, w.rank, w.info, w.A, w.Z, s)) ||
                 (s2 = cuda_check(cudaMemcpyAsync(&kk, w.info, sizeof(int), cudaMemcpyDeviceToHost, s), "D2H kept")) ||
                 (s2 = cuda_check(cudaStreamSynchronize(s), "stream sync")))
                 return s2;
@@ -388,7 +388,7 @@ struct DavidsonRun {
         qm_status st = exact ? cn64(n_in, n_in, src, src, w.G, n_in) : cn_tc(n_in, n_in, src, src, w.G, n_in);
         if (st) return st;
         int k = 0;
-        if ((st = chol_transform(w.G, n_in, n_in, drop, w.sel, w.rank, w.info, w.A, w.Cs, 0, s)) ||
+        if ((st = chol_transform(w.G, n_in, n_in, drop, w.sel, w.rank, w.info, w.A, w.Cs, s)) ||
             (st = cuda_check(cudaMemcpyAsync(&k, w.info, sizeof(int), cudaMemcpyDeviceToHost, s), "D2H kept")) ||
             (st = cuda_check(cudaStreamSynchronize(s), "stream sync")))
             return st;

@@ -290,8 +290,7 @@ __global__ void k_rank(const int* __restrict__ keep, int nd, int* __restrict__ r
 // S = Y Y^H, given in S (lds), destroyed).  keep/rank: nd ints each; X: nd x nd scratch;
 // kept_dev: 1 int.  Asynchronous; the caller reads kept_dev.
 qm_status chol_transform(double2* S, int lds, int nd, double drop_rel, int* keep, int* rank, int* kept_dev,
-                         double2* X, double2* W, int ldw_max, cudaStream_t s) {
-    (void)ldw_max;
+                         double2* X, double2* W, cudaStream_t s) {
     if (nd <= kFused) {
         ProfScope pf(PF_CHOL, s);
         k_chol_small<<<1, 32 * nd, 0, s>>>(S, lds, nd, drop_rel, keep, rank, kept_dev, W);

@@ -138,7 +138,7 @@ extern "C" qm_status qm_hpsi_noalloc(qm_gspace g, int ik, int nb, const void* ps
     size_t o_part = 0;
     if (nproj > 0 && c.off < (size_t)QM_HPSI_NOALLOC_SCRATCH_BYTES) {
         const size_t left = (size_t)QM_HPSI_NOALLOC_SCRATCH_BYTES - c.off;
-        splits = (int)std::min<size_t>((size_t)zgemm_cn_splits(nproj, nb, npw), left / std::max<size_t>(1, pbytes_split));
+        splits = (int)std::min<size_t>((size_t)zgemm_cn_splits(npw), left / std::max<size_t>(1, pbytes_split));
         splits = std::max(1, splits);
         if (splits > 1) o_part = c.take((size_t)splits * pbytes_split);
     }

@@ -252,7 +252,7 @@ qm_status zgemm_cn(int M, int N, int K, const double2* A, int lda, const double2
 qm_status zgemm_tn(int M, int N, int K, const double2* A, int lda, const double* d,
                    const double2* B, int ldb, double2* C, int ldc, bool accumulate, const GemmWork& w,
                    cudaStream_t s, double alpha = 1.0);
-int zgemm_cn_splits(int M, int N, int K);
+int zgemm_cn_splits(int K);  // splits of K that cn can use at most
 // the same products on the tensor cores by digit splitting (zdigits.cu); *done = false: not served
 // (small, or too little scratch), nothing launched.  *flags: what is left to the FP64 kernels
 qm_status zdigits_cn(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb, double2* C, int ldc,
@@ -322,7 +322,7 @@ size_t heev_work_bytes(int m, int nev);
 // destroyed) and counts the kept vectors into kept_dev; chol_transform_rows then writes the
 // nd x kept transform W for gemm_tn (small blocks: chol_transform writes it, if anything was kept).  keep, rank: nd ints; X: nd x nd scratch.
 qm_status chol_transform(double2* S, int lds, int nd, double drop_rel, int* keep, int* rank, int* kept_dev,
-                         double2* X, double2* W, int ldw_max, cudaStream_t s);
+                         double2* X, double2* W, cudaStream_t s);
 qm_status chol_transform_rows(const double2* L, int lds, int nd, const int* keep, const int* rank, int kept,
                               double2* X, double2* W, cudaStream_t s);
 

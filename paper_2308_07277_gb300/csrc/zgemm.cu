@@ -515,11 +515,7 @@ size_t gemm_cn_partial_bytes(bool fp32) {
     return (size_t)kMaxSlots * 80 * 80 * (fp32 ? sizeof(float2) : sizeof(double2));
 }
 
-int zgemm_cn_splits(int M, int N, int K) {
-    (void)M;
-    (void)N;
-    return std::max(1, std::min(64, (K + kCnK - 1) / kCnK));
-}
+int zgemm_cn_splits(int K) { return std::max(1, std::min(64, (K + kCnK - 1) / kCnK)); }
 
 size_t zgemm_cn_bytes(int M, int N, int K, bool digits) {
     if (M <= 0 || N <= 0) return 0;
