@@ -46,6 +46,9 @@ extern "C" qm_status qm_gw_mel(qm_gspace g, int ik_left, int ik_right, int nl, c
     if ((st = ensure_device(g)) || (st = ensure_device(geps))) return st;
     if (g->device != geps->device) return fail(QM_ERR_ARG, "qm_gw_mel: the handles live on different devices");
     cudaStream_t s = (cudaStream_t)stream;
+    // pairs for any number of states: the left boxes and the products halve in number, which outweighs the few
+    // CTAs.  Single / paired, us, 48^3 points: 1 x 1 states 44 / 38, 3 x 3 45 / 41, 8 x 16 101 / 79; 72^3: 1 x 1
+    // 56 / 55, 3 x 3 59 / 61, 8 x 16 216 / 182; 72 x 72 x 36: 1 x 4 47 / 50, 3 x 3 50 / 54, 4 x 4 57 / 54
     if (prec == QM_MIXED && pair_path(g))
         return gw_mel_pair(g, ik_left, ik_right, nl, psi_l, ld_l, nr, psi_r, ld_r, geps, iq, M, ld_m, s);
     if (prec == QM_MIXED)
