@@ -1032,9 +1032,23 @@ def run_ours(args):
                 "large_cells": large,
                 "davidson_216_atoms_learned": dav_large,
                 "cpu_baseline": oracle_sample("config5", args.cpu_baseline_bands)}
-        print(json.dumps(line))
+        print(json.dumps(line), file=sys.stderr)
+        print(json.dumps(headline(line)))
     if world > 1:
         torch.distributed.destroy_process_group()
+
+
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+            "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline")
+
+
+def headline(line):
+    """The line of the run's main result: what it was, the figure, its end-to-end form and its roofline, short
+    enough to survive a log that keeps the end of the output (the whole of `line` goes to stderr)."""
+    out = {k: line[k] for k in HEADLINE}
+    out["forms"] = {k: v["value"] for k, v in line["forms"].items() if isinstance(v, dict)}
+    out["cpu_baseline"] = {k: line["cpu_baseline"][k] for k in ("value", "unit", "cores", "kind")}
+    return out
 
 
 def run_profile(args):

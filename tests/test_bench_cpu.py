@@ -53,3 +53,24 @@ def test_max_over_ranks_two_gloo_ranks():
     for p in ps:
         p.join(timeout=60)
     assert res[0] == [2.0, 5.0] and res[1] == [2.0, 5.0]
+
+
+def test_headline_is_short_and_whole():
+    """The line on stdout holds the contract's keys in at most 2500 characters, whatever the details' size."""
+    if ROOT not in sys.path:
+        sys.path.insert(0, ROOT)
+    import bench
+    line = {k: 1.5 for k in bench.HEADLINE}
+    line["config"] = {"workload": "w" * 400}
+    line["e2e"] = {"value": 126074.2608941202, "unit": "band-applies/s", "h2d_bytes_per_step": 883676160, "d2h_bytes_per_step": 883676160}
+    line["clocks"] = {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": [], "samples": 6}
+    line["roofline"] = {"bound": "tensor", "note": "r" * 450}
+    line["forms"] = {"fp64": {"value": 1.0, "kernels": ["k"] * 500}, "mixed_over_fp64": 2.0}
+    line["davidson"] = {"rows": ["x" * 100] * 100}
+    line["cpu_baseline"] = {"value": 1.0, "unit": "u", "cores": 16, "kind": "oracle", "sample": "s" * 300}
+    out = json.dumps(bench.headline(line))
+    assert len(out) <= 2500
+    d = json.loads(out)
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+              "dtype", "data", "config", "e2e", "gpu_launches", "clocks"):
+        assert k in d, k
