@@ -340,10 +340,8 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
     double2 *a = smt, *vb = smt + m * ld, *w = vb + 2 * m;  // [m][ld], reflectors of two columns, product
     __shared__ double s_beta[2], s_half;  // beta (0: no reflection), -|tau|^2 / 2
     __shared__ double2 s_t;
-    __shared__ int s_max;
+    __shared__ int s_max[8];
     const int tid = threadIdx.x, lane = tid & 31;
-    if (tid == 0) s_max = 0;
-    __syncthreads();
     int h = 0;  // largest high word of a component, compared as integers
     for (int i = tid; i < m * m; i += 256) {
         const double2 x = A[(size_t)(i / m) * lda + i % m];
@@ -351,14 +349,16 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
         a[(i / m) * ld + i % m] = x;
     }
     h = __reduce_max_sync(0xffffffffu, h);
-    if (lane == 0) atomicMax(&s_max, h);
+    if (lane == 0) s_max[tid >> 5] = h;
     __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) h = max(h, s_max[i]);
     // (a non-finite matrix is left as it is; a zero one has nothing to scale)
-    int ex = (s_max >> 20) - 1023;  // the largest component is in [2^ex, 2^(ex+1))
-    const bool scaled = (ex < -kTriRange || ex > kTriRange) && ex < 1024 && s_max > 0;
+    int ex = (h >> 20) - 1023;  // the largest component is in [2^ex, 2^(ex+1))
+    const bool scaled = (ex < -kTriRange || ex > kTriRange) && ex < 1024 && h > 0;
     const int shift = scaled ? max(-1000, min(1000, -ex)) : 0;
-    const double up = __hiloint2double((1023 + shift) << 20, 0), back = __hiloint2double((1023 - shift) << 20, 0);
     if (scaled) {
+        const double up = __hiloint2double((1023 + shift) << 20, 0);
         for (int i = tid; i < m * m; i += 256) {
             double2& x = a[(i / m) * ld + i % m];
             x.x *= up;
@@ -392,12 +392,11 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
         }
         if (lane == 0) {
             s_beta[k & 1] = beta;
-            const double ek = none ? 0.0 : beta != 0.0 ? beta : alpha.x, dk = a[k * ld + k].x;
-            e[k] = scaled ? ek * back : ek;
-            d[k] = scaled ? dk * back : dk;
+            e[k] = none ? 0.0 : beta != 0.0 ? beta : alpha.x;
+            d[k] = a[k * ld + k].x;
         }
     };
-    __syncthreads();
+    if (scaled) __syncthreads();
     if (tid < 32) reflector(0);
     for (int k = 0; k < m - 1; ++k) {
         __syncthreads();
@@ -479,9 +478,14 @@ k_tridiag_small(const double2* __restrict__ A, int lda, int m, double2* __restri
         }
     }
     __syncthreads();
-    if (tid == 0) {
-        const double x = a[(m - 1) * ld + m - 1].x;
-        d[m - 1] = scaled ? x * back : x;
+    if (tid == 0) d[m - 1] = a[(m - 1) * ld + m - 1].x;
+    if (scaled) {  // (in a loop of its own: beside each column's stores the products would be taken in any case)
+        const double back = __hiloint2double((1023 - shift) << 20, 0);
+        __syncthreads();
+        for (int i = tid; i < m; i += 256) {
+            d[i] *= back;
+            if (i < m - 1) e[i] *= back;
+        }
     }
 }
 
