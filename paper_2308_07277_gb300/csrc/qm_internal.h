@@ -231,7 +231,7 @@ struct GemmWork {
     int* err = nullptr;
     bool digits = true;
     int hold_panel = -1;
-    long hold_polls = 0;
+    int hold_polls = 0;
 };
 // Rows of a product that the digit products leave to the FP64 kernels: *any != 0 if there are some,
 // output (m, n) is one if em[m] or en[n] equals `flag`.  any = NULL: every output.

@@ -73,7 +73,7 @@ constexpr int kDgEpiWarps = 8;
 constexpr int kDgThreads = 32 * (kDgEpiWarps + 2);
 constexpr int kDgFlag = 0x7FF;     // exponent of a row left to the FP64 kernels
 constexpr int kDgSegs = 4;         // partial maxima per row
-constexpr long kDgSpin = 1L << 26;
+constexpr int kDgSpin = 1 << 26;
 
 __host__ __device__ constexpr size_t dg_plane(int R) { return (size_t)R * kDgK * 2; }
 __host__ __device__ constexpr size_t dg_block(int R) { return kDg * dg_plane(R); }
@@ -295,8 +295,8 @@ __device__ __forceinline__ double dg_value(long long hi, long long lo, int ex) {
 // exponent of the integer unit of a product of rows with exponents ea, eb
 __device__ __forceinline__ int dg_unit(int ea, int eb) { return ea + eb - 2 * 1022 - 70; }
 
-__device__ __forceinline__ bool dg_wait(uint32_t bar, uint32_t parity, volatile int* abort, long polls = kDgSpin) {
-    for (long i = 0; i < polls; ++i) {
+__device__ __forceinline__ bool dg_wait(uint32_t bar, uint32_t parity, volatile int* abort, int polls = kDgSpin) {
+    for (int i = 0; i < polls; ++i) {
         uint32_t done;
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
@@ -313,13 +313,14 @@ __device__ __forceinline__ bool dg_wait(uint32_t bar, uint32_t parity, volatile 
 // blockIdx.z.  EPI 0 (cn): the exact sums (hi, lo) of row m, real column n to
 // part[(z * mpad + m) * npad + n] (add: on top of what an earlier panel of K left there).
 // EPI 1 (tn): C[n / 2][plain row] of the complex FP64 output, component n % 2 (accumulate: added),
-// except outputs of flagged rows.
-template <int EPI>
+// except outputs of flagged rows.  kHold: waits give up after `polls` polls (as a run-time number in every
+// launch it cost 5 us of 316 at 480 x 157 x 18232).
+template <int EPI, bool kHold>
 __global__ void __launch_bounds__(kDgThreads, 1)
 k_dg_gemm(const unsigned char* __restrict__ P, const unsigned char* __restrict__ X, int nkt, int kt_per_split,
           longlong2* __restrict__ part, int mpad, int npad, int add, int* __restrict__ ep,
           const int* __restrict__ ex, int* __restrict__ any, int nplain, int nexp, double2* __restrict__ C, int ldc, int accumulate,
-          int* __restrict__ err, long polls) {
+          int* __restrict__ err, int polls) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) uint64_t full[kDgStages], empty[kDgStages], acc_full, acc_empty, done;
     __shared__ uint32_t tmem_base;
@@ -351,6 +352,7 @@ k_dg_gemm(const unsigned char* __restrict__ P, const unsigned char* __restrict__
     asm volatile("tcgen05.fence::after_thread_sync;\n");
     const uint32_t tmem = tmem_base, sbase = tc::smem_u32(smem);
     volatile int* abort = &abort_flag;
+    const int limit = kHold ? polls : kDgSpin;
     if (warp == kDgEpiWarps) {
         if (lane == 0) {
             const unsigned char* a_src = P + ((size_t)blockIdx.y * nkt + kt0) * a_bytes;
@@ -358,7 +360,7 @@ k_dg_gemm(const unsigned char* __restrict__ P, const unsigned char* __restrict__
             int it = 0;
             for (; it < nk; ++it) {
                 const int s = it % kDgStages;
-                if (it >= kDgStages && !dg_wait(tc::smem_u32(&empty[s]), ((it / kDgStages) & 1) ^ 1, abort, polls)) {
+                if (it >= kDgStages && !dg_wait(tc::smem_u32(&empty[s]), ((it / kDgStages) & 1) ^ 1, abort, limit)) {
                     *abort = 1;
                     break;
                 }
@@ -382,11 +384,11 @@ k_dg_gemm(const unsigned char* __restrict__ P, const unsigned char* __restrict__
             for (; it < nk; ++it) {
                 const int s = it % kDgStages, c = it / kDgChunk;
                 // the drains of the previous chunk must have read the accumulators
-                if (it % kDgChunk == 0 && c > 0 && !dg_wait(tc::smem_u32(&acc_empty), (c - 1) & 1, abort, polls)) {
+                if (it % kDgChunk == 0 && c > 0 && !dg_wait(tc::smem_u32(&acc_empty), (c - 1) & 1, abort, limit)) {
                     *abort = 1;
                     break;
                 }
-                if (!dg_wait(tc::smem_u32(&full[s]), (it / kDgStages) & 1, abort, polls)) {
+                if (!dg_wait(tc::smem_u32(&full[s]), (it / kDgStages) & 1, abort, limit)) {
                     *abort = 1;
                     break;
                 }
@@ -428,7 +430,7 @@ k_dg_gemm(const unsigned char* __restrict__ P, const unsigned char* __restrict__
         for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
         bool ok = true;
         for (int c = 0; c < nchunk; ++c) {
-            ok = dg_wait(tc::smem_u32(&acc_full), c & 1, abort, polls);
+            ok = dg_wait(tc::smem_u32(&acc_full), c & 1, abort, limit);
             if (!ok) *abort = 1;
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
@@ -633,12 +635,13 @@ bool dg_serves(bool cn, int M, int N, int K) {
 template <int EPI>
 qm_status dg_gemm(const unsigned char* P, const unsigned char* X, int nkt, int splits, int pt, int xt, longlong2* part, int mpad,
                   int npad, bool add, int* ep, const int* ex, int* any, int nplain, int nexp, double2* C, int ldc, bool accumulate,
-                  int* err, long polls, cudaStream_t s) {
+                  int* err, int polls, cudaStream_t s) {
     const size_t smem = (size_t)kDgStages * (dg_block(kDgM) + dg_block(kDgN));
-    qm_status st = allow_dynamic_smem((const void*)k_dg_gemm<EPI>, smem, "digit products: shared memory");
+    const auto kern = polls < kDgSpin ? k_dg_gemm<EPI, true> : k_dg_gemm<EPI, false>;
+    qm_status st = allow_dynamic_smem((const void*)kern, smem, "digit products: shared memory");
     if (st) return st;
     ProfScope pf(EPI ? PF_GEMM_TN : PF_GEMM_CN, s);
-    k_dg_gemm<EPI><<<dim3(xt, pt, splits), kDgThreads, smem, s>>>(P, X, nkt, cdiv(nkt, splits), part, mpad, npad, add ? 1 : 0, ep, ex,
+    kern<<<dim3(xt, pt, splits), kDgThreads, smem, s>>>(P, X, nkt, cdiv(nkt, splits), part, mpad, npad, add ? 1 : 0, ep, ex,
                                                                 any, nplain, nexp, C, ldc, accumulate ? 1 : 0, err, polls);
     return cuda_check(cudaGetLastError(), "k_dg_gemm launch");
 }

@@ -643,7 +643,7 @@ extern "C" qm_status qm_zgemm_hold(int op, int M, int N, int K, const void* A, i
     GemmWork w;
     w.bytes = scratch;
     w.hold_panel = panel;
-    w.hold_polls = (long)polls;
+    w.hold_polls = (int)std::min<long long>(polls, 1 << 26);
     if (scratch && (st = cuda_check(cudaMallocAsync(&w.ptr, scratch, s), "qm_zgemm_hold: workspace"))) return st;
     if (scratch) *panels = zdigits_panels(op == 0, M, N, K, scratch);
     st = op == 0 ? zgemm_cn(M, N, K, (const double2*)A, lda, (const double2*)B, ldb, (double2*)C, ldc, w, s)
