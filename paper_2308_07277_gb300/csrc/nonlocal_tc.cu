@@ -719,7 +719,7 @@ qm_status check_limits(const NlLayout& L) {
 
 // Launch while the kernel before in the stream still runs (programmatic dependent launch): its last CTAs, the
 // launch and the set-up of this one overlap, 1 to 2 us at each link of the chain (64 atoms: 2 bands 73.6 ->
-// 64.6 us, 24 bands 107 -> 98; 128 bands 427 -> 420).  The kernel calls chain_wait before it uses or
+// 64.6 us, 24 bands 107 -> 98; 160 bands 427 -> 420).  The kernel calls chain_wait before it uses or
 // overwrites anything.  chain_next in the kernel before lets this one's CTAs take their places early; the
 // products and k_split_rows do not call it: projection CTAs that wait beside the split keep FFT CTAs of the
 // other stream off the SMs (propagation of 32 atoms: 1107 us with it, 1044 without).

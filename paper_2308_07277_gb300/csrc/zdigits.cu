@@ -19,8 +19,8 @@
 // The error of a term is that of its operands' rounding, at most 2^-55 of the row's largest component,
 // where FP64 multiply-adds round every partial sum: FP64 accuracy by norm.  It is not element by
 // element: what lies below 2^-56 of its row's largest is lost, so a sum that such elements decide (rows
-// that fall where the other operand's rise, |a_k| = e^(-20 k/K), |b_k| = e^(20 k/K - 20): error 8e-11 of
-// sum |a| |b|, FP64 3e-17) needs the FP64 kernels: qm_zgemm's arith 3, qm_davidson_opts.fp64_exact.
+// that fall where the other operand's rise, |a_k| = e^(-20 k/K), |b_k| = e^(20 k/K - 20): error 7e-11 of
+// sum |a| |b| at 200 x 60 x 4000, FP64 2e-17; e^-3: 8e-18, 2e-17) needs the FP64 kernels: qm_zgemm's arith 3, qm_davidson_opts.fp64_exact.
 // Relative error (2-norm, against 80-bit sums) of rows that fall together, FP64
 // multiply-adds / digits: 2.7e-15 / 1.3e-16 at 480 x 157 x 18232 (rows falling off 13-fold), 2.4e-15 /
 // 8.9e-17 (200-fold), 3.8e-15 / 9.6e-17 at 640 x 100 x 40000, 8.6e-16 / 8.4e-17 at 512 x 64 x 400;

@@ -1,18 +1,19 @@
 // Complex GEMMs of the nonlocal projector step (Sec. 2.3, KB form: P = beta^H psi, then
 // beta D P) and of the Davidson subspace products (<V_i|H V_j>, rotations by the Ritz
-// coefficients, Gram-Schmidt projections).  SIMT kernels with shared-memory tiles: in FP64
-// the GB300's double rate (about 1.2 TFLOP/s), not memory, bounds these contractions, so
-// register tiling with enough CTAs to fill every SM is what matters.
+// coefficients, Gram-Schmidt projections).
 //
 //   cn : C[m][n] = sum_k conj(A[m][k]) B[n][k]                 (k contiguous in A and B)
 //        split over K into partial sums reduced in a fixed order (deterministic)
-//   tn : C[m][n] = alpha sum_k A[k][m] d[k] B[k][n] (+ C[m][n])  (m, n contiguous)
+//   tn : C[m][n] = alpha sum_k A[k][m] d[k] B[k][n]  (+ C[m][n])  (m, n contiguous)
 //
-// 16 x 16 threads per CTA, each owning a TM x TN block of outputs (tile 16TM x 16TN); the
-// per-call tile is chosen so that the M and N edges waste as little as possible (160
-// bands -> TM = 5, 256 projectors -> TM = 4).  With FP32 arithmetic the products of one K tile
-// (16 terms) are summed in FP32 and the tile sums in FP64, so the rounding error does not grow
-// with K (inner products over 10^4 - 10^5 plane waves keep ~1e-7 relative accuracy).
+// FP64: long products as digit products on the tensor cores (zdigits.cu), the others, and the rows those
+// leave, on small tiles with one output per thread (k_cn, k_tn; the FP64 pipe bounds them).  FP32: the same
+// small tiles for the precision form's small projector products (csmall_*), and register tiles for
+// qm_hpsi_noalloc (cgemm_*): 16 x 16 threads per CTA, each owning a TM x TN block of outputs (tile
+// 16TM x 16TN), the tile chosen per call so that the M and N edges waste as little as possible (160
+// bands -> TM = 5, 256 projectors -> TM = 4); the products of one K tile (16 terms) are summed in FP32 and
+// the tile sums in FP64, so the rounding error does not grow with K (inner products over 10^4 - 10^5 plane
+// waves keep ~1e-7 relative accuracy).
 #include <algorithm>
 
 #include "qm_internal.h"
