@@ -54,7 +54,8 @@ typedef enum {
     QM_FP64 = 0,   /* FP64; large complex products to FP64 accuracy by norm (see qm_zgemm, arith 0) */
     QM_MIXED = 1   /* FP32 FFT path and V multiply; nonlocal projection and application as split
                       products of FP16 pairs (row-scaled, 23 bits) on the tensor cores, FP32
-                      accumulation; FP32 products on the CUDA cores for small ones */
+                      accumulation; FP32 products on the CUDA cores for small ones and up
+                      to 16 projectors */
 } qm_precision;
 
 /*
